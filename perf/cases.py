@@ -112,7 +112,8 @@ def draw(rng):
         nx, ny = _side(rng, int(side) // 2 + 2 ** k, int(side) + 2 ** k, k), _side(rng, int(side), int(1.4 * side), k)
     else:
         side = math.exp(rng.uniform(math.log(40), math.log(520)))
-        nx = ny = _side(rng, 40, 520, _levels(side * side))
+        k = _levels(side * side)
+        nx = ny = int(side) // 2 ** k * 2 ** k
     cells = nx * ny
     return {"kind": kind, "problem": problem, "nx": nx, "ny": ny, "precision": prec,
             "steps": 1 if kind == "host_step" or cells > 4 << 20 else (2 if cells > 1 << 19 else 4)}
