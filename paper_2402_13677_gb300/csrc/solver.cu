@@ -50,7 +50,8 @@ constexpr int NRED = 608;        // blocks of grid-stride kernels (4 x 152 SMs)
 constexpr int SMALL_MAX_F = 1024; // default: levels with at most this many cells run inside k_small (FP32)
 constexpr int SMALL_MAX_F_LIMIT = 4096;   // the shared memory of k_small holds at most this level
 constexpr int SMALL_MAX_D = 1024; // (FP64: half the shared memory per value)
-constexpr int SMALL_THREADS = 1024;
+constexpr int SMALL_THREADS = 512;   // of the single-block levels (k_small, and block 0 of a cooperative launch)
+constexpr int SMALL_INV = 32 * 32;   // entries of the coarsest operator's dense inverse, at most
 constexpr int TX = 32, TY = 32;  // tile of the large-level kernels
 constexpr int NU = 2;            // smoothing sweeps (red-black pairs) before and after
 constexpr int NU_SMALL = 2;      // the same on the levels of the single-block kernel
@@ -73,6 +74,7 @@ struct Lev {
     const T* wl;
     const T* wb;
     long long zs;   // byte stride between the instances of a batched launch (0: one instance)
+    const T* id;    // FP64: reciprocal of the full diagonal (k_diag_inverse); null in FP32
 };
 
 // correctly rounded reciprocal (the same value as 1 / v)
@@ -88,7 +90,32 @@ __device__ inline float rcp_diag(float v) {
 }
 __device__ inline double rcp_diag(double v) { return __drcp_rn(v); }
 
-__device__ inline bool skip(const SolveState* s) { return s->done != 0 || s->odone != 0; }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// residual b - A x of one cell in the smoothers, in flux form (row sums stay exactly D in FP32)
+template <typename T>
+__device__ inline T cell_residual(T b, T d, T w0, T w1, T w2, T w3, T x, T xl, T xr, T xd, T xu) {
+    T ax = d * x + w0 * (x - xl) + w1 * (x - xr) + w2 * (x - xd) + w3 * (x - xu);
+    return b - ax;
+}
+
+// a state word read now, not at its first use: the words a kernel needs before its work travel
+// together with the skip flags (one L2 round trip at the head of these short kernels, not three)
+__device__ __forceinline__ int ld_now(const int* p) {
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double ld_now(const double* p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ inline bool skip(const SolveState* s) {
+    const int a = ld_now(&s->done), b = ld_now(&s->odone);
+    return (a | b) != 0;
+}
 
 __device__ inline unsigned long long gtimer() {
     unsigned long long t;
@@ -100,16 +127,18 @@ __device__ inline unsigned long long gtimer() {
 // (and the first block of each instance counts that instance as active), a block of a converged
 // instance only arrives.  The last block to arrive adds the launch's span (first start to last
 // end), its launch and the algorithmic bytes of its active instances, and resets the timer.
-__device__ inline void timer_begin(KTimer* tm) {
-    if (tm && threadIdx.x == 0) {
+// Outside ebit_timing_begin / ebit_timing_end the timer is off (KTimer::on, read once at the start
+// of a launch): no atomics and no fence at the end of every smoother launch.
+__device__ inline bool timer_on(const KTimer* tm) { return tm && threadIdx.x == 0 && ld_now(&tm->on) != 0; }
+__device__ inline void timer_begin(KTimer* tm, bool on) {   // on: timer_on, thread 0
+    if (on) {
         atomicMin(&tm->start, gtimer());
         if (blockIdx.x == 0 && blockIdx.y == 0) atomicAdd(&tm->active, 1u);
     }
 }
-__device__ inline void timer_arrive(KTimer* tm, double bytes_per_instance, bool ran) {
-    if (!tm) return;
+__device__ inline void timer_arrive(KTimer* tm, bool on, double bytes_per_instance, bool ran) {
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (on) {
         if (ran) atomicMax(&tm->end, gtimer());
         __threadfence();
         unsigned int n = gridDim.x * gridDim.y * gridDim.z;
@@ -129,7 +158,6 @@ __device__ inline void timer_arrive(KTimer* tm, double bytes_per_instance, bool 
         }
     }
 }
-__device__ inline void timer_end(KTimer* tm, double bytes_per_instance) { timer_arrive(tm, bytes_per_instance, true); }
 
 // ---- block reductions ---------------------------------------------------------------
 __device__ inline double bsum(double v, double* sh) {
@@ -150,14 +178,34 @@ __device__ inline double bsum(double v, double* sh) {
 // into slot `slot` of partial (partial[k * nslot + slot], thread 0); once every block of the grid
 // has written its slots, last_block_total returns true in thread 0 of the last block to arrive,
 // with the totals over the nslot slots in tot[0..NV).
+// the NV sums share the two block barriers (their shuffle chains overlap)
 template <int NV>
 __device__ inline void block_partial(const double* v, double* partial, int nslot, int slot) {
-    __shared__ double sh[32];
+    __shared__ double sh[NV][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double r[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        double r = bsum(v[k], sh);
-        if (threadIdx.x == 0) partial[k * nslot + slot] = r;
+    for (int k = 0; k < NV; ++k) r[k] = v[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) r[k] += __shfl_down_sync(0xffffffffu, r[k], o);
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) sh[k][w] = r[k];
+    __syncthreads();
+    if (w == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) r[k] = lane < (int)(blockDim.x >> 5) ? sh[k][lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < NV; ++k) r[k] += __shfl_down_sync(0xffffffffu, r[k], o);
+        if (lane == 0)
+#pragma unroll
+            for (int k = 0; k < NV; ++k) partial[k * nslot + slot] = r[k];
     }
+    __syncthreads();
 }
 // the same block sum in the solver precision T, converted once (thread 0): the r.z of a tile's
 // FP32 cells is summed in FP32 (its slot then joins the FP64 total in tile order), so the tile
@@ -187,33 +235,50 @@ __device__ inline void block_partial_t(const T* v, double* partial, int nslot, i
         if (threadIdx.x == 0) partial[k * nslot + slot] = widen(r);
     }
 }
+// Arrival is one atomic add with acquire-release semantics by thread 0, which wrote the block's
+// slots itself: it publishes them, and in the last block it (and, through the block barrier,
+// every thread) sees the other blocks' slots.  Full fences by every thread around a relaxed
+// add cost about a microsecond per launch at the end of these kernels' dependent chain.
+__device__ inline unsigned arrive_acq_rel(unsigned* p) {
+    unsigned v;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 template <int NV>
 __device__ inline bool last_block_total(double* partial, int nslot, unsigned* ticket, double* tot) {
-    __shared__ double sh[32];
+    __shared__ double sh[NV][32];
     __shared__ bool last;
-    __threadfence();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x * gridDim.y - 1;
+    if (threadIdx.x == 0) last = arrive_acq_rel(ticket) == gridDim.x * gridDim.y - 1;
     __syncthreads();
     if (!last) return false;
-    __threadfence();
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        double s = 0.0;
-        for (int b = threadIdx.x; b < nslot; b += blockDim.x) s += ((volatile double*)partial)[k * nslot + b];
-        s = bsum(s, sh);
-        if (threadIdx.x == 0) tot[k] = s;
+    for (int k = 0; k < NV; ++k) s[k] = 0.0;
+    for (int b = threadIdx.x; b < nslot; b += blockDim.x)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) s[k] += __ldcg(partial + k * nslot + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) s[k] += __shfl_down_sync(0xffffffffu, s[k], o);
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) sh[k][w] = s[k];
+    __syncthreads();
+    if (w == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) s[k] = lane < (int)(blockDim.x >> 5) ? sh[k][lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < NV; ++k) s[k] += __shfl_down_sync(0xffffffffu, s[k], o);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) tot[k] = s[k];
     }
     if (threadIdx.x == 0) *ticket = 0u;
     return threadIdx.x == 0;
 }
-// one slot per block; partial has room for NV x (number of blocks) doubles
-template <int NV>
-__device__ inline bool grid_reduce(const double* v, double* partial, unsigned* ticket, double* tot) {
-    int nb = gridDim.x * gridDim.y;
-    block_partial<NV>(v, partial, nb, blockIdx.y * gridDim.x + blockIdx.x);
-    return last_block_total<NV>(partial, nb, ticket, tot);
-}
-
 // use 1: the loop condition is this solve's own (assigned); use 2: a batched launch, where the
 // condition is the OR over the instances (reset to 0 at the top of each loop body by
 // k_cond_reset, raised to 1 by every instance that continues)
@@ -267,14 +332,10 @@ struct Region {
     static constexpr int SX = TX + 2 * H, SY = TY + 2 * H, HX = SX / 2, NC = SY * HX;
     static constexpr int NSEG = SY / 2, THREADS = HX * NSEG;
     static_assert(SX % 2 == 0 && SY % 2 == 0, "region sides must be even");
-    // the FP64 tile kernels restrict through shared memory (their residuals in registers
-    // would spill at the register count their occupancy allows); the FP32 ones in registers
-    static constexpr bool RES_SMEM = sizeof(T) == 8;
-    T* x0;   // x of colour 0 (NR per cell), then colour 1; then the core residuals (FP64 k_pre)
+    T* x0;   // x of colour 0 (NR per cell), then colour 1
     __device__ Region(unsigned char* base) { x0 = (T*)base; }
     __device__ T* x(int c) const { return x0 + c * (NR * NC); }
-    __device__ T* res() const { return x0 + 2 * NR * NC; }
-    static constexpr size_t BYTES = ((size_t)2 * NC + (RES_SMEM ? TX * TY : 0)) * NR * sizeof(T);
+    static constexpr size_t BYTES = (size_t)2 * NC * NR * sizeof(T);
     __host__ __device__ static constexpr size_t bytes() { return BYTES; }
 };
 template <int H>
@@ -347,11 +408,15 @@ struct Stage {
     static constexpr size_t SB = (size_t)BWS * BHS * sizeof(T);
     static constexpr size_t VB = (size_t)BWV * NR * BHV * sizeof(T);
     static constexpr size_t CB = (size_t)BWC * NR * BHC * sizeof(T);
-    static constexpr size_t OFF_D = 0, OFF_WL = align128(SB), OFF_WB = 2 * align128(SB), OFF_B = 3 * align128(SB);
+    // FP64: pre-smoothing also needs the reciprocal diagonal; post-smoothing needs it instead of D
+    static constexpr bool ID_BOX = sizeof(T) == 8 && !POST;
+    static constexpr int NS = ID_BOX ? 4 : 3;
+    static constexpr size_t OFF_D = 0, OFF_WL = align128(SB), OFF_WB = 2 * align128(SB), OFF_ID = 3 * align128(SB);
+    static constexpr size_t OFF_B = NS * align128(SB);
     static constexpr size_t OFF_XIN = OFF_B + align128(VB), OFF_XC = OFF_XIN + (POST ? align128(VB) : 0);
     static constexpr size_t OFF_BAR = OFF_XC + (POST ? align128(CB) : 0);
     static constexpr size_t BYTES = OFF_BAR + 128;
-    static constexpr uint32_t TX_BYTES = (uint32_t)(3 * SB + VB + (POST ? VB + CB : 0));
+    static constexpr uint32_t TX_BYTES = (uint32_t)(NS * SB + VB + (POST ? VB + CB : 0));
     static_assert(BWS <= 256 && BWV * NR <= 256 && BWC * NR <= 256 && BHS <= 256, "TMA box too large");
 };
 
@@ -362,7 +427,8 @@ __device__ inline void stage_issue(unsigned char* sbase, const TileMaps& M, int 
     uint64_t* bar = reinterpret_cast<uint64_t*>(sbase + Sg::OFF_BAR);
     mbar_expect_tx(bar, Sg::TX_BYTES);
     int xs = gx0 - Sg::OXS, xv = (gx0 - Sg::OXV) * NR;
-    tma_load_2d(sbase + Sg::OFF_D, &M.d, xs, gy0, bar);
+    tma_load_2d(sbase + Sg::OFF_D, sizeof(T) == 8 && POST ? &M.id : &M.d, xs, gy0, bar);
+    if constexpr (Sg::ID_BOX) tma_load_2d(sbase + Sg::OFF_ID, &M.id, xs, gy0, bar);
     tma_load_2d(sbase + Sg::OFF_WL, &M.wl, xs, gy0, bar);
     tma_load_2d(sbase + Sg::OFF_WB, &M.wb, xs, gy0, bar);
     tma_load_2d(sbase + Sg::OFF_B, &M.b, xv, gy0, bar);
@@ -372,18 +438,25 @@ __device__ inline void stage_issue(unsigned char* sbase, const TileMaps& M, int 
     }
 }
 
-// barrier set-up (thread 0), visible to the block after the barrier
+// barrier set-up and the copies of the block's first tile (thread 0), at the very start of the
+// kernel so that they overlap the reads of the solve state
 template <typename T, int NR, int H, bool POST>
-__device__ inline void stage_init(unsigned char* sbase) {
-    uint64_t* bar = reinterpret_cast<uint64_t*>(sbase + Stage<T, NR, H, POST>::OFF_BAR);
+__device__ inline void stage_first(unsigned char* sbase, const TileMaps& M, int tx) {
     if (threadIdx.x == 0) {
-        mbar_init(bar, 1);
+        mbar_init(reinterpret_cast<uint64_t*>(sbase + Stage<T, NR, H, POST>::OFF_BAR), 1);
         mbar_fence_init();
+        stage_issue<T, NR, H, POST>(sbase, M, ((int)blockIdx.x % tx) * TX - H, ((int)blockIdx.x / tx) * TY - H);
     }
-    __syncthreads();
 }
 
-// The tiles of a TMA-staged tile kernel, persistent: block b takes tiles b, b + G, ... (G blocks).
+// a block that leaves without work waits (bounded) for the copies it has in flight
+template <typename T, int NR, int H, bool POST>
+__device__ inline void stage_drain(unsigned char* sbase) {
+    if (threadIdx.x == 0) mbar_wait_bounded(reinterpret_cast<uint64_t*>(sbase + Stage<T, NR, H, POST>::OFF_BAR), 0);
+}
+
+// The tiles of a TMA-staged tile kernel, persistent: block b takes tiles b, b + G, ... (G blocks,
+// at most one per tile; stage_first has requested the first one).
 // The next tile's boxes are requested as soon as the current tile has been read out of them
 // (into registers and the region), so the copies overlap the current tile's sweeps.  work(t,
 // after_load) runs tile t and calls after_load() once the boxes have been read and the block has
@@ -395,11 +468,10 @@ __device__ inline void staged_tiles(unsigned char* sbase, const TileMaps& M, int
                                     Work&& work) {
     using Sg = Stage<T, NR, H, POST>;
     uint64_t* bar = reinterpret_cast<uint64_t*>(sbase + Sg::OFF_BAR);
-    stage_init<T, NR, H, POST>(sbase);
+    __syncthreads();   // the barrier's set-up
     // tile t = by tx + bx, advanced by gridDim.x = gq tx + gr without a division per tile
     int t = blockIdx.x, bx = t % tx, by = t / tx;
     const int gq = (int)gridDim.x / tx, gr = (int)gridDim.x % tx;
-    if (threadIdx.x == 0 && t < nt) stage_issue<T, NR, H, POST>(sbase, M, bx * TX - H, by * TY - H);
     for (uint32_t i = 0; t < nt; ++i) {
         bool landed = mbar_wait_bounded(bar, i & 1u);
         if (__syncthreads_or(!landed)) {
@@ -454,7 +526,8 @@ __device__ inline void tile_load_cells(Region<T, NR, H>& R, Cells<T, NR>& C, int
             int gi = gx0 + rx;
             bool in = !CHECK || (gj >= 0 && gj < L.ny && gi >= 0 && gi < L.nx);
             Vec<T, NR> bv, xv;
-            T dv, wlv, wbv, wrv, wtv;
+            T dv, wlv, wbv, wrv, wtv, idv = T(1);   // FP64: idv loaded (and D only where a residual follows)
+            constexpr bool ID = sizeof(T) == 8;
             if (stage) {
                 // from the TMA boxes (zeros outside the grid)
                 const T* sd = reinterpret_cast<const T*>(stage + Sg::OFF_D);
@@ -463,6 +536,7 @@ __device__ inline void tile_load_cells(Region<T, NR, H>& R, Cells<T, NR>& C, int
                 const T* sb = reinterpret_cast<const T*>(stage + Sg::OFF_B);
                 int qs = ry * Sg::BWS + rx + Sg::OXS, qv = (ry * Sg::BWV + rx + Sg::OXV) * NR;
                 dv = sd[qs];
+                if (ID) idv = POST ? dv : reinterpret_cast<const T*>(stage + Sg::OFF_ID)[qs];
                 wlv = swl[qs];
                 wbv = swb[qs];
                 wrv = swl[qs + 1];
@@ -485,7 +559,8 @@ __device__ inline void tile_load_cells(Region<T, NR, H>& R, Cells<T, NR>& C, int
                 int gic = CHECK ? min(max(gi, 0), L.nx - 1) : gi, gjc = CHECK ? min(max(gj, 0), L.ny - 1) : gj;
                 int g = gjc * L.nx + gic;
                 bv = reinterpret_cast<const Vec<T, NR>*>(b)[g];
-                dv = L.diag[g];
+                if (!(ID && POST)) dv = L.diag[g];
+                if (ID) idv = L.id[g];
                 wlv = L.wl[g];
                 wbv = L.wb[g];
                 wrv = L.wl[!CHECK || gic + 1 < L.nx ? g + 1 : g];
@@ -505,12 +580,12 @@ __device__ inline void tile_load_cells(Region<T, NR, H>& R, Cells<T, NR>& C, int
             if (CHECK && !in) {
 #pragma unroll
                 for (int k2 = 0; k2 < NR; ++k2) { bv.v[k2] = T(0); xv.v[k2] = T(0); }
-                dv = T(1);
+                dv = idv = T(1);
                 wlv = wbv = wrv = wtv = T(0);
             }
             // this cell's colour is e ^ r (both known at compile time)
             bool mine0 = (e ^ r) == 0;
-            T idv = rcp_diag(dv + wlv + wrv + wbv + wtv);
+            if (!ID) idv = rcp_diag(dv + wlv + wrv + wbv + wtv);
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 bool m = (c == 0) == mine0;
@@ -522,7 +597,7 @@ __device__ inline void tile_load_cells(Region<T, NR, H>& R, Cells<T, NR>& C, int
                     C.wr[r][c] = wrv;
                     C.wb[r][c] = wbv;
                     C.wt[r][c] = wtv;
-                    C.d[r][c] = dv;
+                    if (!(ID && POST)) C.d[r][c] = dv;
                 }
             }
             int cc = e ^ r;
@@ -681,10 +756,9 @@ __device__ inline void pre_tile(const Lev<T>& L, const T* __restrict__ b, T* __r
     tile_sweep<T, NR, H, 1, 1>(R, C, tt);
     tile_sweep<T, NR, H, 2, 0>(R, C, tt);
     tile_sweep<T, NR, H, 3, 1>(R, C, tt);
-    // x of the core cells to global memory; their residuals stay in registers ([r][e]: row
-    // ry0 + r, column 2k + e), or go to shared memory (FP64)
+    // x of the core cells to global memory, their residuals in registers ([r][e]: row ry0 + r,
+    // column 2k + e)
     T res[2][2][NR];
-    T* sres = R.res();
     if (act)
         tile_core_cells<T, NR, H>(C, tt, gx0, gy0, L, [&](int r, int c, int rx, int ry, int q, int gi, int gj) {
             const T* xo = R.x(1 - c);
@@ -699,35 +773,15 @@ __device__ inline void pre_tile(const Lev<T>& L, const T* __restrict__ b, T* __r
                 T xrt = e == 0 ? own_h : xo[(q + 1) * NR + k2];
                 T xd = r == 1 ? own_v : xo[(q - HX) * NR + k2];
                 T xu = r == 0 ? own_v : xo[(q + HX) * NR + k2];
-                T ax = C.d[r][c] * x0v + C.wl[r][c] * (x0v - xl) + C.wr[r][c] * (x0v - xrt) +
-                       C.wb[r][c] * (x0v - xd) + C.wt[r][c] * (x0v - xu);
-                if constexpr (Rg::RES_SMEM) sres[((ry - H) * TX + (rx - H)) * NR + k2] = C.b[r][c][k2] - ax;
-                else res[r][e][k2] = C.b[r][c][k2] - ax;
+                res[r][e][k2] = cell_residual(C.b[r][c][k2], C.d[r][c], C.wl[r][c], C.wr[r][c], C.wb[r][c],
+                                              C.wt[r][c], x0v, xl, xrt, xd, xu);
             }
             reinterpret_cast<Vec<T, NR>*>(x)[gj * L.nx + gi] = xv;
         });
-    int cnx = L.nx / 2, cny = L.ny / 2;
-    if constexpr (Rg::RES_SMEM) {
-        __syncthreads();
-        // restriction: sum of the four children (the core starts at an even global index, so
-        // children (2ti + a, 2tj + b) are core cells)
-        for (int t = threadIdx.x; t < (TX / 2) * (TY / 2); t += blockDim.x) {
-            int ti = t % (TX / 2), tj = t / (TX / 2);
-            int ci = bx * (TX / 2) + ti, cj = by * (TY / 2) + tj;
-            if (ci >= cnx || cj >= cny) continue;
-            Vec<T, NR> acc;
-#pragma unroll
-            for (int k2 = 0; k2 < NR; ++k2)
-                acc.v[k2] = sres[((2 * tj) * TX + 2 * ti) * NR + k2] + sres[((2 * tj) * TX + 2 * ti + 1) * NR + k2] +
-                            sres[((2 * tj + 1) * TX + 2 * ti) * NR + k2] +
-                            sres[((2 * tj + 1) * TX + 2 * ti + 1) * NR + k2];
-            reinterpret_cast<Vec<T, NR>*>(bc)[cj * cnx + ci] = acc;
-        }
-        return;
-    }
     // restriction: sum of the four children.  The region starts H (even) cells before the tile,
     // so a thread's 2 x 2 block is the four children of coarse cell (k - H/2, ry0/2 - H/2) of the
     // tile; a coarse cell of the grid has all four children inside the grid, hence computed above
+    int cnx = L.nx / 2, cny = L.ny / 2;
     int ti = k - H / 2, tj = ry0 / 2 - H / 2;
     if (act && ti >= 0 && ti < TX / 2 && tj >= 0 && tj < TY / 2) {
         int ci = bx * (TX / 2) + ti, cj = by * (TY / 2) + tj;
@@ -752,24 +806,28 @@ k_pre(Lev<T> L, const T* __restrict__ b, T* __restrict__ x, T* __restrict__ bc, 
     L.diag = zsh(L.diag, zo);
     L.wl = zsh(L.wl, zo);
     L.wb = zsh(L.wb, zo);
+    L.id = zsh(L.id, zo);
     b = zsh(b, zo);
     x = zsh(x, zo);
     bc = zsh(bc, zo);
     st = zsh(st, zo);
     constexpr double bytes_cell = sizeof(T) * (3.0 + NR * 2.25);
-    if (skip(st)) {
-        timer_arrive(tm, 0.0, false);
-        return;
-    }
     constexpr int H = HPRE;
     using Rg = Region<T, NR, H>;
     extern __shared__ __align__(128) unsigned char smem[];
-    timer_begin(tm);
+    // TMA boxes 128-byte aligned after the region (the launch reserves 128 bytes of slack)
+    unsigned char* stage =
+        reinterpret_cast<unsigned char*>(align128(reinterpret_cast<uintptr_t>(smem) + Rg::BYTES));
+    if (use_tma) stage_first<T, NR, H, false>(stage, maps, (L.nx + TX - 1) / TX);
+    const bool ton = timer_on(tm);
+    if (skip(st)) {
+        if (use_tma) stage_drain<T, NR, H, false>(stage);
+        timer_arrive(tm, ton, 0.0, false);
+        return;
+    }
+    timer_begin(tm, ton);
     if (use_tma) {
-        // persistent blocks over the tiles (1-D grid), TMA boxes 128-byte aligned after the
-        // region (the launch reserves 128 bytes of slack)
-        unsigned char* stage =
-            reinterpret_cast<unsigned char*>(align128(reinterpret_cast<uintptr_t>(smem) + Rg::BYTES));
+        // persistent blocks over the tiles (1-D grid)
         int tx = (L.nx + TX - 1) / TX, nt = tx * ((L.ny + TY - 1) / TY);
         const TileThread tt = tile_thread<H>();
         staged_tiles<T, NR, H, false>(stage, maps, tx, nt, st, [&](int, int bx, int by, auto after_load) {
@@ -779,7 +837,7 @@ k_pre(Lev<T> L, const T* __restrict__ b, T* __restrict__ x, T* __restrict__ bc, 
         pre_tile<T, NR>(L, b, x, bc, blockIdx.x, blockIdx.y, smem, nullptr, tile_thread<H>());
     }
     // algorithmic bytes: b, diag, wl, wb read; x and the quarter-size coarse b written
-    timer_end(tm, (double)L.nx * L.ny * bytes_cell);
+    timer_arrive(tm, ton, (double)L.nx * L.ny * bytes_cell, true);
 }
 
 // post-smoothing of tile (bx, by): x = xin + P xc, then black-red sweeps; returns the tile's
@@ -831,6 +889,7 @@ k_post(Lev<T> L, const T* __restrict__ b, const T* __restrict__ xin, T* __restri
     L.diag = zsh(L.diag, zo);
     L.wl = zsh(L.wl, zo);
     L.wb = zsh(L.wb, zo);
+    L.id = zsh(L.id, zo);
     b = zsh(b, zo);
     xin = zsh(xin, zo);
     x = zsh(x, zo);
@@ -839,19 +898,25 @@ k_post(Lev<T> L, const T* __restrict__ b, const T* __restrict__ xin, T* __restri
     partial = zsh(partial, zo);
     ticket = zsh(ticket, zo);
     constexpr double bytes_cell = sizeof(T) * (3.0 + NR * 3.25);
-    if (skip(st)) {
-        timer_arrive(tm, 0.0, false);
-        return;
-    }
     constexpr int H = HPOST;
     using Rg = Region<T, NR, H>;
     extern __shared__ __align__(128) unsigned char smem[];
-    timer_begin(tm);
+    unsigned char* stage =
+        reinterpret_cast<unsigned char*>(align128(reinterpret_cast<uintptr_t>(smem) + Rg::BYTES));
+    if (use_tma) stage_first<T, NR, H, true>(stage, maps, (L.nx + TX - 1) / TX);
+    const bool ton = timer_on(tm);
+    double rz_old[NR];
+#pragma unroll
+    for (int k2 = 0; k2 < NR; ++k2) rz_old[k2] = DOT ? ld_now(&st->rz[k2]) : 0.0;
+    if (skip(st)) {
+        if (use_tma) stage_drain<T, NR, H, true>(stage);
+        timer_arrive(tm, ton, 0.0, false);
+        return;
+    }
+    timer_begin(tm, ton);
     int nslot = gridDim.x * gridDim.y;
     if (use_tma) {
         // persistent blocks over the tiles (1-D grid); r.z summed over the block's tiles
-        unsigned char* stage =
-            reinterpret_cast<unsigned char*>(align128(reinterpret_cast<uintptr_t>(smem) + Rg::BYTES));
         int tx = (L.nx + TX - 1) / TX, nt = tx * ((L.ny + TY - 1) / TY);
         // r.z: one slot per tile, summed in tile order as with one block per tile
         const TileThread tt = tile_thread<H>();
@@ -870,14 +935,13 @@ k_post(Lev<T> L, const T* __restrict__ b, const T* __restrict__ xin, T* __restri
         if (last_block_total<NR>(partial, nslot, ticket, tot)) {
 #pragma unroll
             for (int k2 = 0; k2 < NR; ++k2) {
-                double old = st->rz[k2];
-                st->beta[k2] = old != 0.0 ? tot[k2] / old : 0.0;
+                st->beta[k2] = rz_old[k2] != 0.0 ? tot[k2] / rz_old[k2] : 0.0;
                 st->rz[k2] = tot[k2];
             }
         }
     }
     // algorithmic bytes: b, x, the quarter-size coarse x, diag, wl, wb read; x written
-    timer_end(tm, (double)L.nx * L.ny * bytes_cell);
+    timer_arrive(tm, ton, (double)L.nx * L.ny * bytes_cell, true);
 }
 
 // ---- small levels: the rest of the V-cycle in one block ---------------------------------
@@ -885,210 +949,347 @@ struct SmallPlan {
     int n;             // number of small levels
     int nx[Solver::MAXLEV], ny[Solver::MAXLEV];
     int soff[Solver::MAXLEV];   // cell offset of each small level inside the shared-memory arrays
+    int xoff[Solver::MAXLEV];   // the same inside the colour-split x array
     size_t goff[Solver::MAXLEV]; // cell offset in the packed global level arrays
     int total;         // cells of all small levels
+    int xtotal;        // entries of the colour-split x array (rows of ceil(nx / 2) per colour)
     long long zs;      // byte stride between the instances of a batched launch
 };
 
-// shared-memory layout: x[NR*total], b[NR*total], diag[total], wl[total], wb[total]
+// What bounds this part is a chain of about forty dependent half-sweeps of a few cells per
+// thread: latency of a shared-memory access, five dependent multiply-adds and a barrier, not
+// bandwidth.  Thread t of a level owns the 2 x 2 block of cells (2I + e, 2J + r), the four
+// children of one cell of the next level, for the level's whole down or up leg:
+//   * coefficients, right-hand side and x of its cells stay in registers through a leg; only x
+//     goes through shared memory, split by colour (unit stride), and two of a cell's four
+//     neighbours are the thread's own cells;
+//   * a level's barriers count only the warps that own cells of it (named barrier 1 + level;
+//     a warp barrier below 33 blocks), so the deep levels run on one warp;
+//   * the restriction is the sum of the block's four residuals, all in one thread.
+// Rows of lanes walking a level with every operand read from shared memory took 29 us per FP64
+// cycle of 32^2 cells (one right-hand side, 64^2 grid) and about 9 us in FP32.
+
+// shared-memory layout: x (colour-split) and b, NR per cell, then diag, wl, wb, id per cell and
+// the transposed inverse of the coarsest operator
 template <typename T, int NR>
 struct SmallMem {
-    T *x, *b, *d, *wl, *wb, *id;   // id: reciprocal of the full diagonal D + the four face weights
-    __device__ SmallMem(unsigned char* base, int total) {
-        x = (T*)base;
-        b = x + (size_t)NR * total;
-        d = b + (size_t)NR * total;
-        wl = d + total;
-        wb = wl + total;
-        id = wb + total;
+    Vec<T, NR>*x, *b;
+    T *d, *wl, *wb, *id, *inv;   // id: reciprocal of the full diagonal D + the four face weights
+    __device__ SmallMem(unsigned char* base, const SmallPlan& P) {
+        x = (Vec<T, NR>*)base;
+        b = x + P.xtotal;
+        d = (T*)(b + P.total);
+        wl = d + P.total;
+        wb = wl + P.total;
+        id = wb + P.total;
+        inv = id + P.total;
     }
-    static size_t bytes(int total) { return (size_t)total * (2 * NR + 4) * sizeof(T); }
-};
-
-// The small levels run in one block.  Their half-sweeps are short, so a block-wide barrier
-// between them costs more than the work; the levels with at most SMALL_WARP_CELLS cells (and
-// every level below them) therefore run on warp 0 alone, with warp barriers.  Team<WARP> is
-// the group of threads of one part: the whole block, or warp 0.
-constexpr int SMALL_WARP_CELLS = 64;
-template <bool WARP>
-struct Team {
-    __device__ static int size() { return WARP ? 32 : (int)blockDim.x; }
-    __device__ static void sync() {
-        if (WARP) __syncwarp();
-        else __syncthreads();
+    static size_t bytes(int total, int xtotal) {
+        return ((size_t)total * (NR + 4) + (size_t)xtotal * NR + SMALL_INV) * sizeof(T);
     }
+    static size_t bytes(const SmallPlan& P) { return bytes(P.total, P.xtotal); }
 };
 
-// lane layout of a row sweep over rows of width w: 2^ls lanes (the smallest power of two >= w,
-// at most 32) take a row, so a warp covers 32 >> ls rows at once and no lane idles on the
-// narrow levels; row j0 + m * jstep, column i0 + m * istep
-template <bool WARP>
-struct RowLanes {
-    int jr, ic, jstep, istep;
-    __device__ RowLanes(int w) {
-        int ls = w <= 1 ? 0 : 32 - __clz(w - 1);
-        ls = ls < 5 ? ls : 5;
-        int rpw = 32 >> ls, lane = threadIdx.x & 31;
-        jr = (WARP ? 0 : (int)(threadIdx.x >> 5)) * rpw + (lane >> ls);
-        ic = lane & ((1 << ls) - 1);
-        jstep = (Team<WARP>::size() >> 5) * rpw;
-        istep = 1 << ls;
-    }
-};
-
-// a small level's sizes, offset and half-sweep lane layout, set up once for all its sweeps
-template <bool WARP>
-struct SmallLevel {
-    int nx, ny, o, hx;
-    RowLanes<WARP> G;
-    __device__ SmallLevel(const SmallPlan& P, int l)
-        : nx(P.nx[l]), ny(P.ny[l]), o(P.soff[l]), hx((P.nx[l] + 1) >> 1), G((P.nx[l] + 1) >> 1) {}
-};
-
-// one red-black half-sweep of colour `color` on a level (a row holds ceil(nx / 2) cells of a
-// colour)
-template <typename T, int NR, bool WARP>
-__device__ inline void small_sweep(const SmallLevel<WARP>& V, SmallMem<T, NR>& M, int color) {
-    const int nx = V.nx, ny = V.ny, o = V.o, hx = V.hx;
-    const RowLanes<WARP>& G = V.G;
-    for (int j = G.jr; j < ny; j += G.jstep)
-        for (int i2 = G.ic; i2 < hx; i2 += G.istep) {
-            int i = 2 * i2 + ((color + j) & 1);
-            if (i >= nx) continue;
-            int q = o + j * nx + i;
-            T w0 = M.wl[q], w1 = i < nx - 1 ? M.wl[q + 1] : T(0), w2 = M.wb[q], w3 = j < ny - 1 ? M.wb[q + nx] : T(0);
-            T id = M.id[q];
-#pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                T a = M.b[q * NR + k];
-                if (i > 0) a += w0 * M.x[(q - 1) * NR + k];
-                if (i < nx - 1) a += w1 * M.x[(q + 1) * NR + k];
-                if (j > 0) a += w2 * M.x[(q - nx) * NR + k];
-                if (j < ny - 1) a += w3 * M.x[(q + nx) * NR + k];
-                M.x[q * NR + k] = a * id;
-            }
-        }
-    Team<WARP>::sync();
+// the team of a level: the first `threads` threads of the block (a multiple of 32)
+__device__ inline int small_team(int nx, int ny) {
+    int n = ((nx + 1) >> 1) * ((ny + 1) >> 1);
+    return n >= SMALL_THREADS ? SMALL_THREADS : (n + 31) & ~31;
+}
+__device__ inline void team_sync(int l, int threads) {
+    if (threads <= 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(l + 1), "r"(threads) : "memory");
 }
 
-// down-leg smoothing of level l from x = 0 (its first colour-0 half-sweep reads only zeros and
-// reduces to x = b / (full diagonal), written together with zeros on colour 1), then the
-// residual restricted to level l + 1
-template <typename T, int NR, bool WARP>
-__device__ inline void small_down(const SmallPlan& P, int l, SmallMem<T, NR>& M) {
-    SmallLevel<WARP> V(P, l);
-    const int nx = V.nx, ny = V.ny, o = V.o;
-    {
-        RowLanes<WARP> G(nx);
-        for (int j = G.jr; j < ny; j += G.jstep)
-            for (int i = G.ic; i < nx; i += G.istep) {
-                int q = o + j * nx + i;
-                bool c0 = ((i + j) & 1) == 0;
-                T id = M.id[q];
+// a thread's 2 x 2 block: [r][e] = row 2J + r, column 2I + e (colour e ^ r); wl[r][0..2] the
+// weights of the row's three vertical faces, wb[0..2][e] of the column's three horizontal ones.
+// Cells beyond an odd side (coarsest level only) have b = x = 0 and zero weights.
+template <typename T, int NR>
+struct SmallBlk {
+    Vec<T, NR> b[2][2], x[2][2];
+    T id[2][2], wl[2][3], wb[3][2];
+    int q;        // x index of the block's first row: row r of either colour at q + r hx
+    unsigned m;   // bit 0 owns a block; 1..4 has left, right, lower, upper neighbours; 5 + 2r + e cell in the grid
+    __device__ bool own() const { return m & 1u; }
+    __device__ bool has(int side) const { return (m >> (1 + side)) & 1u; }
+    __device__ bool cell(int r, int e) const { return (m >> (5 + 2 * r + e)) & 1u; }
+};
+
+template <typename T, int NR>
+__device__ inline void small_place(SmallBlk<T, NR>& B, int nx, int ny, int t) {
+    const int hx = (nx + 1) >> 1, hy = (ny + 1) >> 1, I = t % hx, J = t / hx;
+    unsigned m = 0;
+    if (J < hy) {
+        m = 1u;
+        if (I > 0) m |= 2u;
+        if (2 * I + 2 < nx) m |= 4u;
+        if (J > 0) m |= 8u;
+        if (2 * J + 2 < ny) m |= 16u;
 #pragma unroll
-                for (int k = 0; k < NR; ++k) M.x[q * NR + k] = c0 ? M.b[q * NR + k] * id : T(0);
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                if (2 * I + e < nx && 2 * J + r < ny) m |= 32u << (2 * r + e);
+    }
+    B.m = m;
+    B.q = 2 * J * hx + I;
+}
+
+// the block's weights, reciprocal diagonals and right-hand side from shared memory; DOWN: also D,
+// and in FP32 the reciprocal diagonals are computed here and kept in shared memory for the up leg
+// (read back by the same thread)
+template <typename T, int NR, bool DOWN>
+__device__ inline void small_load(SmallBlk<T, NR>& B, T (&d)[2][2], const SmallPlan& P, int l, SmallMem<T, NR>& M,
+                                  int t) {
+    const int nx = P.nx[l], hx = (nx + 1) >> 1, I = t % hx, J = t / hx;
+    const int c0 = P.soff[l] + 2 * J * nx + 2 * I;   // cell (0, 0) of the block
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const bool in = B.cell(r, e);
+            const int c = in ? c0 + r * nx + e : P.soff[l];
+            B.wl[r][e] = in ? M.wl[c] : T(0);
+            B.wb[r][e] = in ? M.wb[c] : T(0);
+            if (DOWN) d[r][e] = in ? M.d[c] : T(1);
+            if (!DOWN || sizeof(T) == 8) B.id[r][e] = in ? M.id[c] : T(1);
+            Vec<T, NR> bv = M.b[c];
+#pragma unroll
+            for (int k = 0; k < NR; ++k) B.b[r][e].v[k] = in ? bv.v[k] : T(0);
+        }
+        const bool right = B.has(1) && B.cell(r, 1);
+        B.wl[r][2] = right ? M.wl[c0 + r * nx + 2] : T(0);
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const bool up = B.has(3) && B.cell(1, e);
+        B.wb[2][e] = up ? M.wb[c0 + 2 * nx + e] : T(0);
+    }
+    if (DOWN && sizeof(T) == 4) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                B.id[r][e] = rcp_diag(d[r][e] + B.wl[r][e] + B.wl[r][e + 1] + B.wb[r][e] + B.wb[r + 1][e]);
+                if (B.cell(r, e)) M.id[c0 + r * nx + e] = B.id[r][e];
             }
-        Team<WARP>::sync();
     }
-    small_sweep<T, NR, WARP>(V, M, 1);
-    for (int k = 1; k < NU_SMALL; ++k) {
-        small_sweep<T, NR, WARP>(V, M, 0);
-        small_sweep<T, NR, WARP>(V, M, 1);
-    }
-    int cnx = P.nx[l + 1], cny = P.ny[l + 1], co = P.soff[l + 1];
-    RowLanes<WARP> G(cnx);
-    for (int J = G.jr; J < cny; J += G.jstep)
-        for (int I = G.ic; I < cnx; I += G.istep) {
-            T acc[NR];
+}
+
+// neighbour values of cell (r, e): own cells from registers, the others from the x array of
+// the other colour
+template <typename T, int NR>
+__device__ inline void small_nb(const SmallBlk<T, NR>& B, const Vec<T, NR>* xo, int hx, int r, int e, Vec<T, NR>& xl,
+                                Vec<T, NR>& xr, Vec<T, NR>& xd, Vec<T, NR>& xu) {
+    Vec<T, NR> z;
 #pragma unroll
-            for (int k = 0; k < NR; ++k) acc[k] = T(0);
-            for (int d2 = 0; d2 < 4; ++d2) {
-                int i = 2 * I + (d2 & 1), j = 2 * J + (d2 >> 1);
-                int q = o + j * nx + i;
-                T w0 = M.wl[q], w1 = i < nx - 1 ? M.wl[q + 1] : T(0), w2 = M.wb[q],
-                  w3 = j < ny - 1 ? M.wb[q + nx] : T(0);
+    for (int k = 0; k < NR; ++k) z.v[k] = T(0);
+    const int q = B.q + r * hx;
+    xl = e == 1 ? B.x[r][0] : (B.has(0) ? xo[q - 1] : z);
+    xr = e == 0 ? B.x[r][1] : (B.has(1) ? xo[q + 1] : z);
+    xd = r == 1 ? B.x[0][e] : (B.has(2) ? xo[q - hx] : z);
+    xu = r == 0 ? B.x[1][e] : (B.has(3) ? xo[q + hx] : z);
+}
+
+// one red-black half-sweep of colour COLOR over the K blocks of a thread
+template <typename T, int NR, int K, int COLOR>
+__device__ inline void small_sweep(SmallBlk<T, NR> (&B)[K], Vec<T, NR>* x, int nxc, int hx, int l, int team) {
+    const Vec<T, NR>* xo = x + (1 - COLOR) * nxc;
+    Vec<T, NR>* xs = x + COLOR * nxc;
+#pragma unroll
+    for (int u = 0; u < K; ++u)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int e = COLOR ^ r;
+            if (B[u].cell(r, e)) {
+                Vec<T, NR> xl, xr, xd, xu, a;
+                small_nb(B[u], xo, hx, r, e, xl, xr, xd, xu);
+#pragma unroll
+                for (int k = 0; k < NR; ++k)
+                    a.v[k] = (B[u].b[r][e].v[k] + B[u].wl[r][e] * xl.v[k] + B[u].wl[r][e + 1] * xr.v[k] +
+                              B[u].wb[r][e] * xd.v[k] + B[u].wb[r + 1][e] * xu.v[k]) *
+                             B[u].id[r][e];
+                B[u].x[r][e] = a;
+                xs[B[u].q + r * hx] = a;
+            }
+        }
+    team_sync(l, team);
+}
+
+// down leg of level l from x = 0 (its first colour-0 half-sweep reads only zeros and reduces to
+// x = b / (full diagonal)), then the residual restricted to level l + 1
+template <typename T, int NR, int K>
+__device__ inline void small_down(const SmallPlan& P, int l, SmallMem<T, NR>& M, int team) {
+    static_assert(NU_SMALL == 2, "the sweep sequences below are written out for two pairs");
+    const int nx = P.nx[l], ny = P.ny[l], hx = (nx + 1) >> 1, nxc = hx * ny;
+    Vec<T, NR>* x = M.x + P.xoff[l];
+    SmallBlk<T, NR> B[K];
+    T d[K][2][2];
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        const int t = threadIdx.x + u * team;
+        small_place(B[u], nx, ny, t);
+        if (!B[u].own()) continue;
+        small_load<T, NR, true>(B[u], d[u], P, l, M, t);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int k = 0; k < NR; ++k) {
+                B[u].x[r][r].v[k] = B[u].b[r][r].v[k] * B[u].id[r][r];
+                B[u].x[r][1 - r].v[k] = T(0);
+            }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) x[B[u].q + r * hx] = B[u].x[r][r];
+    }
+    team_sync(l, team);
+    small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
+    small_sweep<T, NR, K, 0>(B, x, nxc, hx, l, team);
+    small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
+    Vec<T, NR>* bc = M.b + P.soff[l + 1];
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        if (!B[u].own()) continue;
+        Vec<T, NR> acc;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) acc.v[k] = T(0);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                Vec<T, NR> xl, xr, xd, xu;
+                const Vec<T, NR> xv = B[u].x[r][e];
+                small_nb(B[u], x + (1 - (r ^ e)) * nxc, hx, r, e, xl, xr, xd, xu);
+                // a face without a neighbour has no flux: its term is w (x - x)
+                if (e == 0 && !B[u].has(0)) xl = xv;
+                if (e == 1 && !B[u].has(1)) xr = xv;
+                if (r == 0 && !B[u].has(2)) xd = xv;
+                if (r == 1 && !B[u].has(3)) xu = xv;
 #pragma unroll
                 for (int k = 0; k < NR; ++k) {
-                    T xq = M.x[q * NR + k];
-                    T ax = M.d[q] * xq;
-                    if (i > 0) ax += w0 * (xq - M.x[(q - 1) * NR + k]);
-                    if (i < nx - 1) ax += w1 * (xq - M.x[(q + 1) * NR + k]);
-                    if (j > 0) ax += w2 * (xq - M.x[(q - nx) * NR + k]);
-                    if (j < ny - 1) ax += w3 * (xq - M.x[(q + nx) * NR + k]);
-                    acc[k] += M.b[q * NR + k] - ax;
+                    // (the rounding of the first sum: one right-hand side fuses D x of the
+                    // cells with a left neighbour in the block, two fuse the flux)
+                    T ax;
+                    if (NR == 1 && e == 1) {
+                        ax = fma_rn(d[u][r][e], xv.v[k], B[u].wl[r][e] * (xv.v[k] - xl.v[k]));
+                    } else {
+                        ax = d[u][r][e] * xv.v[k];
+                        ax = fma_rn(B[u].wl[r][e], xv.v[k] - xl.v[k], ax);
+                    }
+                    ax = fma_rn(B[u].wl[r][e + 1], xv.v[k] - xr.v[k], ax);
+                    ax = fma_rn(B[u].wb[r][e], xv.v[k] - xd.v[k], ax);
+                    ax = fma_rn(B[u].wb[r + 1][e], xv.v[k] - xu.v[k], ax);
+                    acc.v[k] += B[u].b[r][e].v[k] - ax;
                 }
             }
-#pragma unroll
-            for (int k = 0; k < NR; ++k) M.b[(co + J * cnx + I) * NR + k] = acc[k];
-        }
-    Team<WARP>::sync();
+        bc[threadIdx.x + u * team] = acc;
+    }
+    team_sync(l, team);
 }
 
 // coarsest level: exact solve with the precomputed inverse (up to 32 cells), else a symmetric
 // red-black sweep sequence from zero
-template <typename T, int NR, bool WARP>
-__device__ inline void small_coarsest(const SmallPlan& P, SmallMem<T, NR>& M, const T* __restrict__ inv) {
-    int l = P.n - 1, o = P.soff[l], n = P.nx[l] * P.ny[l];
-    if (n <= 32 && inv[n * n] == T(1)) {
-        if (threadIdx.x < 32) {
-            int r = threadIdx.x;
-            T acc[NR];
+template <typename T, int NR>
+__device__ inline void small_coarsest(const SmallPlan& P, SmallMem<T, NR>& M, bool exact) {
+    const int l = P.n - 1, o = P.soff[l], nx = P.nx[l], ny = P.ny[l], n = nx * ny;
+    const int hx = (nx + 1) >> 1, nxc = hx * ny;
+    Vec<T, NR>* x = M.x + P.xoff[l];
+    const int team = exact ? 32 : small_team(nx, ny);
+    if (threadIdx.x >= team) return;
+    if (exact) {
+        const int r = threadIdx.x;
+        if (r < n) {
+            Vec<T, NR> acc;
 #pragma unroll
-            for (int k = 0; k < NR; ++k) acc[k] = T(0);
-            if (r < n)
-                for (int c = 0; c < n; ++c) {
-                    T a = inv[r * n + c];
+            for (int k = 0; k < NR; ++k) acc.v[k] = T(0);
+#pragma unroll 8
+            for (int c = 0; c < n; ++c) {
+                const T a = M.inv[c * n + r];
+                const Vec<T, NR> bv = M.b[o + c];
 #pragma unroll
-                    for (int k = 0; k < NR; ++k) acc[k] += a * M.b[(o + c) * NR + k];
-                }
-            __syncwarp();
-            if (r < n)
+                for (int k = 0; k < NR; ++k) acc.v[k] += a * bv.v[k];
+            }
+            const int i = r % nx, j = r / nx;
+            x[((i + j) & 1) * nxc + j * hx + (i >> 1)] = acc;
+        }
+        return;
+    }
+    SmallBlk<T, NR> B[1];
+    T d[2][2];
+    small_place(B[0], nx, ny, threadIdx.x);
+    if (B[0].own()) {
+        small_load<T, NR, true>(B[0], d, P, l, M, threadIdx.x);
 #pragma unroll
-                for (int k = 0; k < NR; ++k) M.x[(o + r) * NR + k] = acc[k];
-        }
-        Team<WARP>::sync();
-    } else {
-        int t = WARP ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
-        for (int c = t; c < n * NR; c += Team<WARP>::size()) M.x[o * NR + c] = T(0);
-        Team<WARP>::sync();
-        SmallLevel<WARP> V(P, l);
-        for (int k = 0; k < COARSE_PAIRS; ++k) {
-            small_sweep<T, NR, WARP>(V, M, 0);
-            small_sweep<T, NR, WARP>(V, M, 1);
-        }
-        for (int k = 0; k < COARSE_PAIRS; ++k) {
-            small_sweep<T, NR, WARP>(V, M, 1);
-            small_sweep<T, NR, WARP>(V, M, 0);
-        }
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                for (int k = 0; k < NR; ++k) B[0].x[r][e].v[k] = T(0);
+                if (2 * (B[0].q / (2 * hx)) + r < ny) x[(e ^ r) * nxc + B[0].q + r * hx] = B[0].x[r][e];
+            }
+    }
+    team_sync(l, team);
+    for (int k = 0; k < COARSE_PAIRS; ++k) {
+        small_sweep<T, NR, 1, 0>(B, x, nxc, hx, l, team);
+        small_sweep<T, NR, 1, 1>(B, x, nxc, hx, l, team);
+    }
+    for (int k = 0; k < COARSE_PAIRS; ++k) {
+        small_sweep<T, NR, 1, 1>(B, x, nxc, hx, l, team);
+        small_sweep<T, NR, 1, 0>(B, x, nxc, hx, l, team);
     }
 }
 
-// up-leg of level l: x += P x_{l+1}, then the post-smoothing half-sweeps
-template <typename T, int NR, bool WARP>
-__device__ inline void small_up(const SmallPlan& P, int l, SmallMem<T, NR>& M) {
-    SmallLevel<WARP> V(P, l);
-    const int nx = V.nx, ny = V.ny, o = V.o, cnx = P.nx[l + 1], co = P.soff[l + 1];
-    RowLanes<WARP> G(nx);
-    for (int j = G.jr; j < ny; j += G.jstep)
-        for (int i = G.ic; i < nx; i += G.istep) {
+// up leg of level l: x += P x_{l+1}, then the post-smoothing half-sweeps.  The opening barrier
+// joins the level's team with the warps that worked on the coarser levels.
+template <typename T, int NR, int K>
+__device__ inline void small_up(const SmallPlan& P, int l, SmallMem<T, NR>& M, int team) {
+    const int nx = P.nx[l], ny = P.ny[l], hx = (nx + 1) >> 1, nxc = hx * ny;
+    const int cnx = P.nx[l + 1], chx = (cnx + 1) >> 1, cnxc = chx * P.ny[l + 1];
+    Vec<T, NR>* x = M.x + P.xoff[l];
+    const Vec<T, NR>* xc = M.x + P.xoff[l + 1];
+    SmallBlk<T, NR> B[K];
 #pragma unroll
-            for (int k = 0; k < NR; ++k)
-                M.x[(o + j * nx + i) * NR + k] += M.x[(co + (j >> 1) * cnx + (i >> 1)) * NR + k];
+    for (int u = 0; u < K; ++u) {
+        const int t = threadIdx.x + u * team;
+        small_place(B[u], nx, ny, t);
+        T d[2][2];
+        if (B[u].own()) {
+            small_load<T, NR, false>(B[u], d, P, l, M, t);
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) B[u].x[r][e] = x[(e ^ r) * nxc + B[u].q + r * hx];
         }
-    Team<WARP>::sync();
-    for (int k = 0; k < NU_SMALL; ++k) {
-        small_sweep<T, NR, WARP>(V, M, 1);
-        small_sweep<T, NR, WARP>(V, M, 0);
     }
+    team_sync(l, team);
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        if (!B[u].own()) continue;
+        const int t = threadIdx.x + u * team, I = t % hx, J = t / hx;
+        const Vec<T, NR> cv = xc[((I + J) & 1) * cnxc + J * chx + (I >> 1)];
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                for (int k = 0; k < NR; ++k) B[u].x[r][e].v[k] += cv.v[k];
+                x[(e ^ r) * nxc + B[u].q + r * hx] = B[u].x[r][e];
+            }
+    }
+    team_sync(l, team);
+    small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
+    small_sweep<T, NR, K, 0>(B, x, nxc, hx, l, team);
+    small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
+    small_sweep<T, NR, K, 0>(B, x, nxc, hx, l, team);
 }
 
-// the V-cycle on the small levels in one block, from the level-(first small) rhs b_in to its
-// correction x_out; with DOT (the cycle starts at the finest level) also r.z -> beta
+// the V-cycle on the small levels in one block of SMALL_THREADS threads, from the level-(first
+// small) rhs b_in to its correction x_out; with DOT (the cycle starts at the finest level) also
+// r.z -> beta
 template <typename T, int NR, bool DOT>
-__device__ void small_cycle(const SmallPlan& P, const T* __restrict__ diag, const T* __restrict__ wl,
-                            const T* __restrict__ wb, const T* __restrict__ inv, const T* __restrict__ b_in,
+__device__ void small_cycle(const SmallPlan& P, const T* __restrict__ diag, const T* __restrict__ id,
+                            const T* __restrict__ wl, const T* __restrict__ wb, const T* __restrict__ inv, const T* __restrict__ b_in,
                             T* __restrict__ x_out, SolveState* st, unsigned char* smem) {
-    SmallMem<T, NR> M(smem, P.total);
+    SmallMem<T, NR> M(smem, P);
+    const int nlast = P.nx[P.n - 1] * P.ny[P.n - 1];
     // the small levels are contiguous in the packed level arrays and in shared memory: one flat
     // copy per array, four independent loads in flight per thread and array
     {
@@ -1102,70 +1303,93 @@ __device__ void small_cycle(const SmallPlan& P, const T* __restrict__ diag, cons
             M.d[c] = a;
             M.wl[c] = b2;
             M.wb[c] = c2;
+            if (sizeof(T) == 8) M.id[c] = id[P.goff[0] + c];
         }
     }
-    int n0 = P.nx[0] * P.ny[0];
+    const int n0 = P.nx[0] * P.ny[0];
+    const Vec<T, NR>* bv = reinterpret_cast<const Vec<T, NR>*>(b_in);
 #pragma unroll 4
-    for (int c = threadIdx.x; c < n0 * NR; c += blockDim.x) M.b[c] = b_in[c];
+    for (int c = threadIdx.x; c < n0; c += blockDim.x) M.b[c] = bv[c];
+    const bool exact = nlast <= 32 && inv[nlast * nlast] == T(1);
+    if (exact)
+        for (int c = threadIdx.x; c < nlast * nlast; c += blockDim.x) M.inv[(c % nlast) * nlast + c / nlast] = inv[c];
     __syncthreads();
-    for (int l = 0; l < P.n; ++l) {
-        int nx = P.nx[l], ny = P.ny[l], o = P.soff[l];
-        RowLanes<false> G(nx);
-        for (int j = G.jr; j < ny; j += G.jstep)
-            for (int i = G.ic; i < nx; i += G.istep) {
-                int q = o + j * nx + i;
-                T dg = M.d[q] + M.wl[q] + (i < nx - 1 ? M.wl[q + 1] : T(0)) + M.wb[q] +
-                       (j < ny - 1 ? M.wb[q + nx] : T(0));
-                M.id[q] = rcp_diag(dg);
+    // every level's down leg on its team, the coarsest solve, the up legs: a warp leaves at the first
+    // level it owns no cells of and waits for the others at that level's (the previous team's)
+    // up leg
+    const int tid = threadIdx.x;
+    int lmax = 0;   // levels [0, lmax) with this thread in the team
+    while (lmax < P.n - 1 && tid < small_team(P.nx[lmax], P.ny[lmax])) ++lmax;
+    const bool two = ((P.nx[0] + 1) >> 1) * ((P.ny[0] + 1) >> 1) > SMALL_THREADS;   // level 0: two blocks per thread
+    for (int l = 0; l < lmax; ++l) {
+        const int team = small_team(P.nx[l], P.ny[l]);
+        bool done = false;
+        if constexpr (sizeof(T) == 4)
+            if (l == 0 && two) {
+                small_down<T, NR, 2>(P, l, M, team);
+                done = true;
             }
+        if (!done) small_down<T, NR, 1>(P, l, M, team);
+    }
+    if (lmax == P.n - 1) {
+        small_coarsest<T, NR>(P, M, exact);
+        if (tid < 32) __syncwarp();
+    }
+    for (int l = lmax - 1; l >= 0; --l) {
+        const int team = small_team(P.nx[l], P.ny[l]);
+        bool done = false;
+        if constexpr (sizeof(T) == 4)
+            if (l == 0 && two) {
+                small_up<T, NR, 2>(P, l, M, team);
+                done = true;
+            }
+        if (!done) small_up<T, NR, 1>(P, l, M, team);
     }
     __syncthreads();
-    // down to the first level of at most SMALL_WARP_CELLS cells (lw) on the whole block, the
-    // levels from lw on (coarsest included) on warp 0, then up on the whole block
-    int lw = P.n;
-    for (int l = 0; l < P.n; ++l)
-        if (P.nx[l] * P.ny[l] <= SMALL_WARP_CELLS) {
-            lw = l;
-            break;
-        }
-    int lb = lw < P.n - 1 ? lw : P.n - 1;   // levels [0, lb) have block-wide down and up legs
-    for (int l = 0; l < lb; ++l) small_down<T, NR, false>(P, l, M);
-    if (lw < P.n) {
-        if (threadIdx.x < 32) {
-            for (int l = lw; l < P.n - 1; ++l) small_down<T, NR, true>(P, l, M);
-            small_coarsest<T, NR, true>(P, M, inv);
-            for (int l = P.n - 2; l >= lw; --l) small_up<T, NR, true>(P, l, M);
-        }
-        __syncthreads();
-    } else {
-        small_coarsest<T, NR, false>(P, M, inv);
-    }
-    for (int l = lb - 1; l >= 0; --l) small_up<T, NR, false>(P, l, M);
-    for (int c = threadIdx.x; c < n0 * NR; c += blockDim.x) x_out[c] = M.x[c];
+    const int nx0 = P.nx[0], hx0 = (nx0 + 1) >> 1, nxc0 = hx0 * P.ny[0];
+    const Vec<T, NR>* x0 = M.x + P.xoff[0];
+    auto xat = [&](int c) {
+        const int i = c % nx0, j = c / nx0;
+        return x0[((i + j) & 1) * nxc0 + j * hx0 + (i >> 1)];
+    };
+    for (int c = threadIdx.x; c < n0; c += blockDim.x) reinterpret_cast<Vec<T, NR>*>(x_out)[c] = xat(c);
     if (DOT) {
-        // the cycle started at the finest level: r.z -> beta (one block, fixed order)
+        // the cycle started at the finest level: r.z -> beta, summed as by 1024 threads (virtual
+        // thread t takes the cells t, t + 1024, ...; 32 warp sums, then their sum)
         __shared__ double sh[32];
 #pragma unroll
         for (int k = 0; k < NR; ++k) {
-            double a = 0.0;
-            for (int c = threadIdx.x; c < n0; c += blockDim.x) a += (double)M.x[c * NR + k] * (double)M.b[c * NR + k];
-            a = bsum(a, sh);
-            if (threadIdx.x == 0) {
-                double old = st->rz[k];
-                st->beta[k] = old != 0.0 ? a / old : 0.0;
-                st->rz[k] = a;
+#pragma unroll
+            for (int h = 0; h < 1024 / SMALL_THREADS; ++h) {
+                double a = 0.0;
+                for (int c = h * SMALL_THREADS + threadIdx.x; c < n0; c += 1024)
+                    a += (double)xat(c).v[k] * (double)M.b[c].v[k];
+                for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+                if ((threadIdx.x & 31) == 0) sh[(h * SMALL_THREADS + threadIdx.x) >> 5] = a;
             }
+            __syncthreads();
+            if (threadIdx.x < 32) {
+                double a = sh[threadIdx.x];
+                for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+                if (threadIdx.x == 0) {
+                    double old = st->rz[k];
+                    st->beta[k] = old != 0.0 ? a / old : 0.0;
+                    st->rz[k] = a;
+                }
+            }
+            __syncthreads();
         }
     }
 }
 
 template <typename T, int NR, bool DOT>
 __global__ void __launch_bounds__(SMALL_THREADS) k_small(SmallPlan P, const T* __restrict__ diag,
-                                                         const T* __restrict__ wl, const T* __restrict__ wb,
+                                                         const T* __restrict__ id, const T* __restrict__ wl, const T* __restrict__ wb,
                                                          const T* __restrict__ inv, const T* __restrict__ b_in,
                                                          T* __restrict__ x_out, SolveState* st) {
     const long long zo = zoff(P.zs);
     diag = zsh(diag, zo);
+    id = zsh(id, zo);
     wl = zsh(wl, zo);
     wb = zsh(wb, zo);
     inv = zsh(inv, zo);
@@ -1174,7 +1398,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_small(SmallPlan P, const T* _
     st = zsh(st, zo);
     if (skip(st)) return;
     extern __shared__ __align__(128) unsigned char smem[];
-    small_cycle<T, NR, DOT>(P, diag, wl, wb, inv, b_in, x_out, st, smem);
+    small_cycle<T, NR, DOT>(P, diag, id, wl, wb, inv, b_in, x_out, st, smem);
 }
 
 
@@ -1194,7 +1418,7 @@ struct CoarsePlan {
     T* xo[Solver::MAXLEV];           // final x of level l
     const T* xc[Solver::MAXLEV];     // x of level l + 1 (read by the post phase of level l)
 };
-constexpr int CC_THREADS = 512;
+constexpr int CC_THREADS = SMALL_THREADS;
 
 // grid-wide barrier of a cooperative launch (all blocks resident).  bar[0] counts arrivals and
 // only grows during a launch (the level-0 pre-smoothing kernel, which precedes every launch,
@@ -1227,7 +1451,7 @@ __device__ inline void grid_sync(unsigned* bar, unsigned& target, SolveState* st
 
 template <typename T, int NR>
 __global__ void __launch_bounds__(CC_THREADS) k_coarse_cycle(CoarsePlan<T> C, SmallPlan P, const T* __restrict__ diag,
-                                                             const T* __restrict__ wl, const T* __restrict__ wb,
+                                                             const T* __restrict__ id, const T* __restrict__ wl, const T* __restrict__ wb,
                                                              const T* __restrict__ inv, SolveState* st,
                                                              unsigned* bar) {
     if (skip(st)) return;   // written by an earlier launch: the same for every block
@@ -1243,7 +1467,7 @@ __global__ void __launch_bounds__(CC_THREADS) k_coarse_cycle(CoarsePlan<T> C, Sm
         }
         grid_sync(bar, gen, st, C.spin);
     }
-    if (blockIdx.x == 0) small_cycle<T, NR, false>(P, diag, wl, wb, inv, C.bc[C.nb - 1], C.xo[C.nb], st, smem);
+    if (blockIdx.x == 0) small_cycle<T, NR, false>(P, diag, id, wl, wb, inv, C.bc[C.nb - 1], C.xo[C.nb], st, smem);
     grid_sync(bar, gen, st, C.spin);
     for (int l = C.nb - 1; l >= C.l0; --l) {
         const Lev<T>& L = C.L[l];
@@ -1399,6 +1623,29 @@ __global__ void __launch_bounds__(256) k_setup_tree(SetupPlan P, const double* _
 }
 
 
+// FP64 levels: the reciprocal of every cell's full diagonal D + its four face weights, correctly
+// rounded, once per solve.  The FP64 pipe (one warp instruction per 19 cycles and SM) bounds the
+// FP64 smoothers, and the four sums and the reciprocal were 14 of the 24 to 28 FP64 instructions
+// that a region cell cost in every smoother launch (the reciprocal stored is the same value).
+__global__ void __launch_bounds__(256) k_diag_inverse(SetupPlan P, const double* __restrict__ diag,
+                                                      const double* __restrict__ wl, const double* __restrict__ wb,
+                                                      double* __restrict__ id) {
+    const long long zo = zoff(P.zs);
+    diag = zsh(diag, zo);
+    wl = zsh(wl, zo);
+    wb = zsh(wb, zo);
+    id = zsh(id, zo);
+    for (int l = 0; l < P.nlev; ++l) {
+        const int nx = P.nx[l], ny = P.ny[l];
+        const size_t o = P.off[l];
+        for (CellWalk cw(nx); cw.c < nx * ny; cw.next()) {
+            const size_t c = o + cw.c;
+            id[c] = rcp_diag(diag[c] + wl[c] + (cw.i + 1 < nx ? wl[c + 1] : 0.0) + wb[c] +
+                             (cw.j + 1 < ny ? wb[c + nx] : 0.0));
+        }
+    }
+}
+
 // ---- CG kernels ---------------------------------------------------------------------------
 // p_new = z + beta p_old; q = A p_new; p.q -> alpha = r.z / p.q
 // Dot-product accumulation of a thread: FP64 for FP64 data; for FP32 data an FP32-pair running
@@ -1456,14 +1703,19 @@ __global__ void __launch_bounds__(256) k_apply(Lev<T> L, const T* __restrict__ z
     st = zsh(st, zo);
     partial = zsh(partial, zo);
     ticket = zsh(ticket, zo);
+    const int it = ld_now(&st->iters);
+    T beta[NR];
+    double rz[NR];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+        beta[k] = (T)ld_now(&st->beta[k]);
+        rz[k] = ld_now(&st->rz[k]);
+    }
     if (skip(st)) return;
     const Vec<T, NR>* __restrict__ Z = reinterpret_cast<const Vec<T, NR>*>(z);
-    const Vec<T, NR>* __restrict__ Po = reinterpret_cast<const Vec<T, NR>*>((st->iters & 1) ? p1 : p0);
-    Vec<T, NR>* __restrict__ Pn = reinterpret_cast<Vec<T, NR>*>((st->iters & 1) ? p0 : p1);
+    const Vec<T, NR>* __restrict__ Po = reinterpret_cast<const Vec<T, NR>*>((it & 1) ? p1 : p0);
+    Vec<T, NR>* __restrict__ Pn = reinterpret_cast<Vec<T, NR>*>((it & 1) ? p0 : p1);
     Vec<T, NR>* __restrict__ Q = reinterpret_cast<Vec<T, NR>*>(q);
-    T beta[NR];
-#pragma unroll
-    for (int k = 0; k < NR; ++k) beta[k] = (T)st->beta[k];
     int N = L.nx * L.ny;
     for (int v = blockIdx.x; v < vb; v += gridDim.x) {
         DotAcc<T, NR> acc;
@@ -1518,7 +1770,7 @@ __global__ void __launch_bounds__(256) k_apply(Lev<T> L, const T* __restrict__ z
 #pragma unroll
         for (int k = 0; k < NR; ++k) {
             st->pq[k] = tot[k];
-            st->alpha[k] = tot[k] != 0.0 ? st->rz[k] / tot[k] : 0.0;
+            st->alpha[k] = tot[k] != 0.0 ? rz[k] / tot[k] : 0.0;
         }
     }
 }
@@ -1539,14 +1791,15 @@ __global__ void __launch_bounds__(256) k_update(int N, long long zs, T* __restri
     st = zsh(st, zo);
     partial = zsh(partial, zo);
     ticket = zsh(ticket, zo);
+    const int it = ld_now(&st->iters);
+    T alpha[NR];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) alpha[k] = (T)ld_now(&st->alpha[k]);
     if (skip(st)) return;
-    const Vec<T, NR>* __restrict__ Pn = reinterpret_cast<const Vec<T, NR>*>((st->iters & 1) ? p0 : p1);
+    const Vec<T, NR>* __restrict__ Pn = reinterpret_cast<const Vec<T, NR>*>((it & 1) ? p0 : p1);
     const Vec<T, NR>* __restrict__ Q = reinterpret_cast<const Vec<T, NR>*>(q);
     Vec<T, NR>* __restrict__ X = reinterpret_cast<Vec<T, NR>*>(x);
     Vec<T, NR>* __restrict__ Rr = reinterpret_cast<Vec<T, NR>*>(r);
-    T alpha[NR];
-#pragma unroll
-    for (int k = 0; k < NR; ++k) alpha[k] = (T)st->alpha[k];
     for (int v = blockIdx.x; v < vb; v += gridDim.x) {
         DotAcc<T, NR> acc;
         const int stride = vb * blockDim.x;
@@ -1633,10 +1886,12 @@ __global__ void __launch_bounds__(256) k_apply4(Lev<float> L, const float* __res
     st = zsh(st, zo);
     partial = zsh(partial, zo);
     ticket = zsh(ticket, zo);
+    const int it = ld_now(&st->iters);
+    const float beta = (float)ld_now(&st->beta[0]);
+    const double rz = ld_now(&st->rz[0]);
     if (skip(st)) return;
-    const float* __restrict__ Po = (st->iters & 1) ? p1 : p0;
-    float* __restrict__ Pn = (st->iters & 1) ? p0 : p1;
-    const float beta = (float)st->beta[0];
+    const float* __restrict__ Po = (it & 1) ? p1 : p0;
+    float* __restrict__ Pn = (it & 1) ? p0 : p1;
     const int nx = L.nx, ny = L.ny, nq = nx / 4, NQ = nq * ny;
     // p = z + beta p_old of one cell / of four (beta = 0: p = z, the old p unused)
     auto pn1 = [&](int cc) { return beta != 0.0f ? z[cc] + beta * Po[cc] : z[cc]; };
@@ -1688,7 +1943,7 @@ __global__ void __launch_bounds__(256) k_apply4(Lev<float> L, const float* __res
     double tot[1];
     if (last_block_total<1>(partial, vb, ticket, tot)) {
         st->pq[0] = tot[0];
-        st->alpha[0] = tot[0] != 0.0 ? st->rz[0] / tot[0] : 0.0;
+        st->alpha[0] = tot[0] != 0.0 ? rz / tot[0] : 0.0;
     }
 }
 
@@ -1708,10 +1963,12 @@ __global__ void __launch_bounds__(256) k_apply2(Lev<float> L, const float* __res
     st = zsh(st, zo);
     partial = zsh(partial, zo);
     ticket = zsh(ticket, zo);
+    const int it = ld_now(&st->iters);
+    const float b0 = (float)ld_now(&st->beta[0]), b1 = (float)ld_now(&st->beta[1]);
+    const double rz[2] = {ld_now(&st->rz[0]), ld_now(&st->rz[1])};
     if (skip(st)) return;
-    const float* __restrict__ Po = (st->iters & 1) ? p1 : p0;
-    float* __restrict__ Pn = (st->iters & 1) ? p0 : p1;
-    const float b0 = (float)st->beta[0], b1 = (float)st->beta[1];
+    const float* __restrict__ Po = (it & 1) ? p1 : p0;
+    float* __restrict__ Pn = (it & 1) ? p0 : p1;
     const int nx = L.nx, ny = L.ny, np = nx / 2, NP = np * ny;
     // p = z + beta p_old of one cell (float2) / of two (float4), per right-hand side
     auto pn2 = [&](int cc) {
@@ -1774,7 +2031,7 @@ __global__ void __launch_bounds__(256) k_apply2(Lev<float> L, const float* __res
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             st->pq[k] = tot[k];
-            st->alpha[k] = tot[k] != 0.0 ? st->rz[k] / tot[k] : 0.0;
+            st->alpha[k] = tot[k] != 0.0 ? rz[k] / tot[k] : 0.0;
         }
     }
 }
@@ -1793,13 +2050,14 @@ __global__ void __launch_bounds__(256) k_update4(int N, long long zs, float* __r
     st = zsh(st, zo);
     partial = zsh(partial, zo);
     ticket = zsh(ticket, zo);
+    const int it = ld_now(&st->iters);
+    // element e of a float4 belongs to right-hand side e % NR (NR = 2: liquid, vapour interleaved)
+    const float a0 = (float)ld_now(&st->alpha[0]), a1 = NR > 1 ? (float)ld_now(&st->alpha[1]) : a0;
     if (skip(st)) return;
-    const float4* __restrict__ Pn = reinterpret_cast<const float4*>((st->iters & 1) ? p0 : p1);
+    const float4* __restrict__ Pn = reinterpret_cast<const float4*>((it & 1) ? p0 : p1);
     const float4* __restrict__ Q = reinterpret_cast<const float4*>(q);
     float4* __restrict__ X = reinterpret_cast<float4*>(x);
     float4* __restrict__ R = reinterpret_cast<float4*>(r);
-    // element e of a float4 belongs to right-hand side e % NR (NR = 2: liquid, vapour interleaved)
-    const float a0 = (float)st->alpha[0], a1 = NR > 1 ? (float)st->alpha[1] : a0;
     const int NQ = N * NR / 4;
     for (int v = blockIdx.x; v < vb; v += gridDim.x) {
         DotAcc<float, NR> acc;
@@ -1855,6 +2113,14 @@ __global__ void __launch_bounds__(256) k_update4(int N, long long zs, float* __r
 // arithmetic of each cell is that of the separate kernels; only the grouping of the dot
 // products differs (per block instead of per launch block).
 
+// the single-block levels as a call: inlined into the whole-solve kernel they add to its spills
+template <typename T, int NR>
+__device__ __noinline__ void small_cycle_call(const SmallPlan& P, const T* diag, const T* wl, const T* wb,
+                                              const T* inv, const T* b_in, T* x_out, SolveState* st,
+                                              unsigned char* smem) {
+    small_cycle<T, NR, false>(P, diag, nullptr, wl, wb, inv, b_in, x_out, st, smem);
+}
+
 // grid barrier that gives up: false if this block's wait ran out or a fault is already recorded
 // (every block then leaves at its next barrier, so a fault ends the launch after a bounded time)
 __device__ inline bool grid_sync_ok(unsigned* bar, unsigned& target, SolveState* st, int spin) {
@@ -1898,7 +2164,7 @@ __device__ inline void sum_slots(const double* partial, int nslot, double* tot) 
 }
 
 template <typename T, int NR>
-__global__ void __launch_bounds__(CC_THREADS)
+__global__ void __launch_bounds__(CC_THREADS, 1)
 k_cg_persist(CoarsePlan<T> C, SmallPlan P, const T* __restrict__ diag, const T* __restrict__ wl,
              const T* __restrict__ wb, const T* __restrict__ inv, T* __restrict__ x, T* __restrict__ r,
              T* __restrict__ p0, T* __restrict__ p1, T* __restrict__ q, SolveState* st, double* partial,
@@ -1935,7 +2201,7 @@ k_cg_persist(CoarsePlan<T> C, SmallPlan P, const T* __restrict__ diag, const T* 
             ok = grid_sync_ok(bar, gen, st, C.spin);
         }
         if (!ok) break;
-        if (blockIdx.x == 0) small_cycle<T, NR, false>(P, diag, wl, wb, inv, C.bc[C.nb - 1], C.xo[C.nb], st, smem);
+        if (blockIdx.x == 0) small_cycle_call<T, NR>(P, diag, wl, wb, inv, C.bc[C.nb - 1], C.xo[C.nb], st, smem);
         if (!grid_sync_ok(bar, gen, st, C.spin)) break;
         for (int l = C.nb - 1; l >= 1 && ok; --l) {
             const Lev<T>& L = C.L[l];
@@ -2222,7 +2488,10 @@ __global__ void __launch_bounds__(256) k_ir_residual(Lev<double> L, const double
     st = zsh(st, zo);
     partial = zsh(partial, zo);
     ticket = zsh(ticket, zo);
-    if (st->odone) return;
+    double sc[NR];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) sc[k] = ld_now(&st->scale_next[k]);
+    if (ld_now(&st->odone)) return;
     int N = L.nx * L.ny;
     // the inner FP32 system is solved for s r, s = 2^k a power of two that brings the residual's
     // cell values to order one, set from the previous residual norm (of b on the first pass) by
@@ -2230,11 +2499,9 @@ __global__ void __launch_bounds__(256) k_ir_residual(Lev<double> L, const double
     // r 2^k on the integer pipes and the norm is summed from that copy (FP32 chunks added in
     // FP64; relative accuracy about 1e-7, ample for the convergence test), so the FP64 pipe
     // carries the residual alone.
-    double sc[NR];
     int ksc[NR];
 #pragma unroll
     for (int k = 0; k < NR; ++k) {
-        sc[k] = st->scale_next[k];
         ksc[k] = (int)((__double_as_longlong(sc[k]) >> 52) & 0x7ff) - 1023;
     }
     const Vec<double, NR>* X = reinterpret_cast<const Vec<double, NR>*>(x);
@@ -2311,9 +2578,10 @@ __global__ void k_ir_update(int N, long long zs, double* __restrict__ x, const f
     x = zsh(x, zo);
     e = zsh(e, zo);
     st = zsh(st, zo);
-    if (st->odone) return;
+    const double s0 = ld_now(&st->scale[0]), s1 = NR > 1 ? ld_now(&st->scale[1]) : s0;
+    if (ld_now(&st->odone)) return;
     // powers of two: exact; an even element belongs to the first right-hand side
-    const double inv0 = 1.0 / st->scale[0], inv1 = NR > 1 ? 1.0 / st->scale[1] : inv0;
+    const double inv0 = 1.0 / s0, inv1 = NR > 1 ? 1.0 / s1 : inv0;
     const long long n = (long long)N * NR;
     const int t = blockIdx.x * blockDim.x + threadIdx.x, T = gridDim.x * blockDim.x;
     // four elements per step (one 16-byte load of e, two of x) where both arrays allow it
@@ -2507,6 +2775,12 @@ template <> struct PT<double> {
     static constexpr int prec = 0;
 };
 
+// the FP64 levels' reciprocal diagonals, in the storage of the levels' Dirichlet terms (read by the
+// set-up alone)
+template <typename T> static T* id_of(Solver& s);
+template <> float* id_of<float>(Solver&) { return nullptr; }
+template <> double* id_of<double>(Solver& s) { return s.d_dd; }
+
 // ---- TMA descriptors (host) ----------------------------------------------------------------
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -2557,6 +2831,7 @@ static bool encode_tile_maps(Solver& s, int l, TileMaps& M) {
     size_t o = s.loff[l];
     const T* b = l == 0 ? PT<T>::r(s) : PT<T>::b(s) + 2 * o;
     bool ok = encode_2d<T>(&M.d, PT<T>::diag(s) + o, nx, ny, Sg::BWS, Sg::BHS) &&
+              (sizeof(T) == 4 || encode_2d<T>(&M.id, id_of<T>(s) + o, nx, ny, Sg::BWS, Sg::BHS)) &&
               encode_2d<T>(&M.wl, PT<T>::wl(s) + o, nx, ny, Sg::BWS, Sg::BHS) &&
               encode_2d<T>(&M.wb, PT<T>::wb(s) + o, nx, ny, Sg::BWS, Sg::BHS) &&
               encode_2d<T>(&M.b, b, nx * NR, ny, Sg::BWV * NR, Sg::BHV);
@@ -2592,7 +2867,8 @@ static void ensure_tile_maps(Solver& s) {
 template <typename T>
 static Lev<T> lev(Solver& s, int l) {
     size_t o = s.loff[l];
-    return {s.lnx[l], s.lny[l], PT<T>::diag(s) + o, PT<T>::wl(s) + o, PT<T>::wb(s) + o, s.zs};
+    const T* id = id_of<T>(s);
+    return {s.lnx[l], s.lny[l], PT<T>::diag(s) + o, PT<T>::wl(s) + o, PT<T>::wb(s) + o, s.zs, id ? id + o : nullptr};
 }
 
 template <typename T>
@@ -2614,6 +2890,11 @@ static void setup_levels(Solver& s, const double* cd, const double* dd, const do
                                                    PT<T>::cd(s), PT<T>::dd(s), d64, PT<T>::inv(s), s.tickets + 6);
     }
     ++s.launches;
+    if constexpr (sizeof(T) == 8) {
+        k_diag_inverse<<<dim3(lblocks(s.nx * (long long)s.ny, s.nz), 1, s.nz), RB, 0, stm>>>(
+            P, PT<T>::diag(s), PT<T>::wl(s), PT<T>::wb(s), id_of<T>(s));
+        ++s.launches;
+    }
 }
 
 // z = M r: r is the level-0 rhs, z the level-0 output (both NR-interleaved)
@@ -2627,16 +2908,19 @@ static SmallPlan small_plan(const Solver& s) {
     P.zs = s.zs;
     int nb = nbig_of<T>(s);
     P.n = s.nlev - nb;
-    int so = 0;
+    int so = 0, xo = 0;
     for (int k = 0; k < P.n; ++k) {
         int l = nb + k;
         P.nx[k] = s.lnx[l];
         P.ny[k] = s.lny[l];
         P.soff[k] = so;
+        P.xoff[k] = xo;
         P.goff[k] = s.loff[l];
         so += s.lnx[l] * s.lny[l];
+        xo += 2 * ((s.lnx[l] + 1) / 2) * s.lny[l];
     }
     P.total = so;
+    P.xtotal = xo;
     return P;
 }
 
@@ -2645,7 +2929,7 @@ static SmallPlan small_plan(const Solver& s) {
 template <typename T, int NR>
 static size_t coarse_smem(const SmallPlan& P) {
     size_t a = Region<T, NR, HPRE>::bytes(), b = Region<T, NR, HPOST>::bytes();
-    size_t c = SmallMem<T, NR>::bytes(P.total);
+    size_t c = SmallMem<T, NR>::bytes(P);
     size_t m = a > b ? a : b;
     return m > c ? m : c;
 }
@@ -2666,7 +2950,7 @@ static int coarse_start(Solver& s) {
         size_t smem = Region<T, NR, HPRE>::bytes() > Region<T, NR, HPOST>::bytes()
                           ? Region<T, NR, HPRE>::bytes()
                           : Region<T, NR, HPOST>::bytes();
-        smem = smem > SmallMem<T, NR>::bytes(5461) ? smem : SmallMem<T, NR>::bytes(5461);
+        smem = smem > SmallMem<T, NR>::bytes(5461, 5461) ? smem : SmallMem<T, NR>::bytes(5461, 5461);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_coarse_cycle<T, NR>, CC_THREADS, smem);
         res = per * sms;
         cudaGetLastError();
@@ -2759,19 +3043,21 @@ static void vcycle(Solver& s, const T* r, T* z, SolveState* st, cudaStream_t stm
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaLaunchKernelEx(&cfg, k_coarse_cycle<T, NR>, C, P, (const T*)PT<T>::diag(s), (const T*)PT<T>::wl(s),
+        cudaLaunchKernelEx(&cfg, k_coarse_cycle<T, NR>, C, P, (const T*)PT<T>::diag(s), (const T*)id_of<T>(s), (const T*)PT<T>::wl(s),
                            (const T*)PT<T>::wb(s), (const T*)PT<T>::inv(s), st, s.tickets + 8);
         if (!s.use_graph) ++s.launches;
     } else {
-        size_t smem = SmallMem<T, NR>::bytes(P.total);
+        size_t smem = SmallMem<T, NR>::bytes(P);
         T* x = nb == 0 ? z : X + 2 * s.loff[nb];
         const T* inv = PT<T>::inv(s);
         if (nb == 0)
-            k_small<T, NR, true><<<dim3(1, 1, s.nz), SMALL_THREADS, smem, stm>>>(P, PT<T>::diag(s), PT<T>::wl(s),
-                                                                               PT<T>::wb(s), inv, b, x, st);
+            k_small<T, NR, true><<<dim3(1, 1, s.nz), SMALL_THREADS, smem, stm>>>(P, PT<T>::diag(s), id_of<T>(s),
+                                                                               PT<T>::wl(s), PT<T>::wb(s), inv, b, x,
+                                                                               st);
         else
-            k_small<T, NR, false><<<dim3(1, 1, s.nz), SMALL_THREADS, smem, stm>>>(P, PT<T>::diag(s), PT<T>::wl(s),
-                                                                                PT<T>::wb(s), inv, b, x, st);
+            k_small<T, NR, false><<<dim3(1, 1, s.nz), SMALL_THREADS, smem, stm>>>(P, PT<T>::diag(s), id_of<T>(s),
+                                                                                PT<T>::wl(s), PT<T>::wb(s), inv, b, x,
+                                                                                st);
         if (!s.use_graph) ++s.launches;
     }
     for (int l = l0 - 1; l >= 0; --l) {
@@ -3053,7 +3339,7 @@ void Solver::solve(const double* cd, const double* dd, const double* wl, const d
         // the FP32 hierarchy, plus D in FP64 for the refinement residual (whose face weights are
         // the caller's FP64 arrays)
         setup_levels<float>(*this, cd, dd, wl, wb, d_diag, stm);
-        Lev<double> L64{nx, ny, d_diag, wl, wb, zs};
+        Lev<double> L64{nx, ny, d_diag, wl, wb, zs, nullptr};
         if (nr == 1) solve_mixed<1>(*this, L64, b, x, rtol, max_iter, stm);
         else solve_mixed<2>(*this, L64, b, x, rtol, max_iter, stm);
     }

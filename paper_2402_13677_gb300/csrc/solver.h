@@ -28,6 +28,8 @@ struct KTimer {
     unsigned long long total_ns;
     unsigned long long launches;
     double bytes;      // algorithmic bytes of the timed launches (each launch adds its own)
+    int on;            // nonzero between ebit_timing_begin and ebit_timing_end
+    int pad;
 };
 
 // device-side scalars of one solve; per right-hand side k < 2
@@ -43,9 +45,10 @@ struct SolveState {
 };
 
 // TMA descriptors of one tiled level (precision and right-hand-side count fixed): the level's
-// right-hand side b, the pre-smoothed x (k_post), the next level's x (k_post), and D, wl, wb
+// right-hand side b, the pre-smoothed x (k_post), the next level's x (k_post), D, wl, wb and, in
+// FP64, the reciprocal diagonal
 struct TileMaps {
-    CUtensorMap b, xin, xc, d, wl, wb;
+    CUtensorMap b, xin, xc, d, wl, wb, id;
 };
 
 struct Solver {
@@ -57,7 +60,8 @@ struct Solver {
     int lnx[MAXLEV], lny[MAXLEV];
     size_t loff[MAXLEV];   // cell offset of level l in the packed per-level arrays
     size_t ncells_all = 0;
-    // per-level operators, packed over levels (float and double copies): diag, wl, wb, cd, dd
+    // per-level operators, packed over levels (float and double copies): diag, wl, wb, cd, dd (FP64:
+    // once the hierarchy is built, d_dd holds the levels' reciprocal diagonals)
     float *f_diag, *f_wl, *f_wb, *f_cd, *f_dd;
     double *d_diag, *d_wl, *d_wb, *d_cd, *d_dd;
     // per-level vectors (2 right-hand sides interleaved), packed: x (correction) and b (rhs)
