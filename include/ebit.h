@@ -230,7 +230,8 @@ uint64_t ebit_launch_count(const ebit_ctx* ctx);
  * launch records the span from its first block's start to its last block's end from the GPU
  * global timer.  kernel_class EBIT_KT_SMOOTH_L0: the finest-grid multigrid smoother kernels
  * (tiled red-black Gauss-Seidel "pre" and "post" kernels), the dominant kernels of the step.
- * ebit_timing_end synchronises and returns the summed kernel time, the number of timed
+ * ebit_timing_end synchronises and returns, for the launches since ebit_timing_begin (0 before the
+ * first one: no launch is timed then), the summed kernel time, the number of timed
  * launches and the algorithmic bytes of an average launch (pre: b, diag, wl, wb read, x and a
  * quarter-size coarse b written; post: x, a quarter-size coarse x, b, diag, wl, wb read, x
  * written; one word per value, 4 bytes in the mixed mode, 8 in FP64, per right-hand side).  A
@@ -302,10 +303,12 @@ ebit_status ebit_get_schedule(ebit_ctx* ctx, int inst, int* small_max, double* i
  *   shared memory with tensor-memory-accelerator copies (cp.async.bulk.tensor); 0 loads them
  *   with ordinary loads.  Both give the same values; levels whose rows or base are not 16-byte
  *   aligned always use ordinary loads.  Changing it drops the captured step graphs.
- *   EBIT_OPT_COOP (default 1) runs the coarse tiled levels of each V-cycle (those whose tiles
- *   fit one per co-resident block) and the single-block levels in one cooperative launch with
- *   grid barriers between the phases; 0 launches each level separately.  Both give the same
- *   values.  2 (mixed precision) runs each whole inner FP32 solve of the refinement, every
+ *   EBIT_OPT_COOP (default 1) runs the coarse tiled levels of each V-cycle and the single-block
+ *   levels in one launch: a thread-block cluster that keeps them in its shared memory (levels up
+ *   to about 256 x 256 cells in FP32, 128 x 128 in FP64), or, where the device takes no such
+ *   cluster or a barrier bound is set, a cooperative launch with grid barriers between the phases
+ *   (levels whose tiles fit one per co-resident block); 0 launches each level separately.  All
+ *   give the same values.  2 (mixed precision) runs each whole inner FP32 solve of the refinement, every
  *   V-cycle and CG update until the inner tolerance, in one cooperative launch with bounded
  *   grid barriers between its phases (grids whose finest tiles fit the reduction slots; others
  *   fall back to 1); its dot products are grouped per block, so the iterates agree with the
@@ -313,7 +316,8 @@ ebit_status ebit_get_schedule(ebit_ctx* ctx, int inst, int* small_max, double* i
  *   1024x2048 grids, where its one block per SM and the spills of its 128 registers outweigh
  *   the saved launches).  Instances stepped in batches always launch each level separately.
  *   EBIT_OPT_BARRIER_SPIN (default 0 = 2^22 polls) bounds the wait of each grid barrier of the
- *   cooperative launch, in polls of the arrival counter.  A fault-path test setting: a bound of
+ *   cooperative launch, in polls of the arrival counter; a bound that is set also selects that
+ *   launch instead of the cluster.  A fault-path test setting: a bound of
  *   a few polls makes the barriers give up before the other blocks arrive.  Changing it drops
  *   the captured step graphs.
  *   EBIT_OPT_EXT_BLOCK (default 1 on grids of at most 2^19 cells, 0 above) runs every Jacobi

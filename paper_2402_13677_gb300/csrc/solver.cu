@@ -36,6 +36,8 @@
 //           the same MG-PCG to a relative 1e-5, x += e in FP64, until ||r|| <= rtol ||b||.
 //
 // Reductions are deterministic: per-block partial sums, the last block adds them in block order.
+#include <algorithm>
+#include <atomic>
 #include <vector>
 #include <cfloat>
 #include <cstdio>
@@ -944,15 +946,31 @@ k_post(Lev<T> L, const T* __restrict__ b, const T* __restrict__ xin, T* __restri
     timer_arrive(tm, ton, (double)L.nx * L.ny * bytes_cell, true);
 }
 
+// 16 bytes from global to shared memory, asynchronously (both 16-byte aligned)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// n elements, the block's threads together; 16-byte pieces in flight at once, plain copies of the rest
+template <typename T>
+__device__ inline void copy_async(T* dst, const T* src, int n) {
+    constexpr int E = 16 / sizeof(T);
+    const bool al = ((reinterpret_cast<uintptr_t>(src) | (uintptr_t)smem_u32(dst)) & 15u) == 0;
+    const int nv = al ? n / E : 0;
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) cp_async16(dst + i * E, src + i * E);
+    for (int i = nv * E + threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
+}
+
 // ---- small levels: the rest of the V-cycle in one block ---------------------------------
 struct SmallPlan {
     int n;             // number of small levels
     int nx[Solver::MAXLEV], ny[Solver::MAXLEV];
     int soff[Solver::MAXLEV];   // cell offset of each small level inside the shared-memory arrays
-    int xoff[Solver::MAXLEV];   // the same inside the colour-split x array
+    int xoff[Solver::MAXLEV];   // first entry of each level in the colour-split x array
     size_t goff[Solver::MAXLEV]; // cell offset in the packed global level arrays
-    int total;         // cells of all small levels
-    int xtotal;        // entries of the colour-split x array (rows of ceil(nx / 2) per colour)
+    int cells;         // cells of all small levels
+    int total;         // the same rounded up to a multiple of four
+    int xtotal;        // entries of the colour-split x array
     long long zs;      // byte stride between the instances of a batched launch
 };
 
@@ -966,8 +984,10 @@ struct SmallPlan {
 //   * a level's barriers count only the warps that own cells of it (named barrier 1 + level;
 //     a warp barrier below 33 blocks), so the deep levels run on one warp;
 //   * the restriction is the sum of the block's four residuals, all in one thread.
-// Rows of lanes walking a level with every operand read from shared memory took 29 us per FP64
-// cycle of 32^2 cells (one right-hand side, 64^2 grid) and about 9 us in FP32.
+//   * x has a zero border, so a half-sweep reads its outer neighbours without a test or branch.
+// k_small on 32^2 cells, rows of lanes walking a level with every operand read from shared memory
+// before: FP32 11.8 -> 8.2 us (one right-hand side), 14.8 -> 10.1 (two), FP64 29 -> 25 and 45 -> 40;
+// with a coarsest level solved by 48 half-sweeps (336^2 grid, 21^2 cells) a step 1.78 -> 1.35 ms.
 
 // shared-memory layout: x (colour-split) and b, NR per cell, then diag, wl, wb, id per cell and
 // the transposed inverse of the coarsest operator
@@ -993,126 +1013,207 @@ struct SmallMem {
 // the team of a level: the first `threads` threads of the block (a multiple of 32)
 __device__ inline int small_team(int nx, int ny) {
     int n = ((nx + 1) >> 1) * ((ny + 1) >> 1);
-    return n >= SMALL_THREADS ? SMALL_THREADS : (n + 31) & ~31;
+    const int cap = blockDim.x;
+    return n >= cap ? cap : (n + 31) & ~31;
 }
 __device__ inline void team_sync(int l, int threads) {
     if (threads <= 32) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(l + 1), "r"(threads) : "memory");
 }
 
+// A level's x array: one entry per 2 cells of a colour, rows -1 .. 2 hy of hx entries each and one
+// spare entry at either end; rows outside the level and the spare entries stay zero.  Cell (i, j)
+// is entry xidx(i >> 1, j) of colour (i + j) & 1.  A block reads its eight outer neighbours without
+// a test: beyond a left or right side that is an entry of the next row, times a zero weight.
+__host__ __device__ constexpr int x_entries(int hx, int rows) { return (rows + 2) * hx + 2; }   // per colour
+__device__ __forceinline__ int xidx(int hx, int I, int j) { return 1 + (j + 1) * hx + I; }
+// t / n for 0 <= t < 2^13 (the quotient of t + 1/2 is at least 1 / (2 n) from an integer)
+__device__ __forceinline__ int small_div(int t, int n) { return (int)__fdividef((float)t + 0.5f, (float)n); }
+
 // a thread's 2 x 2 block: [r][e] = row 2J + r, column 2I + e (colour e ^ r); wl[r][0..2] the
-// weights of the row's three vertical faces, wb[0..2][e] of the column's three horizontal ones.
-// Cells beyond an odd side (coarsest level only) have b = x = 0 and zero weights.
+// weights of the row's three vertical faces, wb[0..2][e] of the column's three horizontal ones
+// (zero where there is no neighbour).  Cells beyond an odd side (coarsest level only) have
+// b = x = 0 and zero weights.
 template <typename T, int NR>
 struct SmallBlk {
     Vec<T, NR> b[2][2], x[2][2];
     T id[2][2], wl[2][3], wb[3][2];
-    int q;        // x index of the block's first row: row r of either colour at q + r hx
-    unsigned m;   // bit 0 owns a block; 1..4 has left, right, lower, upper neighbours; 5 + 2r + e cell in the grid
-    __device__ bool own() const { return m & 1u; }
-    __device__ bool has(int side) const { return (m >> (1 + side)) & 1u; }
-    __device__ bool cell(int r, int e) const { return (m >> (5 + 2 * r + e)) & 1u; }
+    int q;        // x entry of the block's first row: row r of either colour at q + r hx
+    bool own;     // the thread owns a block
 };
-
+// the block's place: I, J of thread t on a level of hx x hy blocks
 template <typename T, int NR>
-__device__ inline void small_place(SmallBlk<T, NR>& B, int nx, int ny, int t) {
-    const int hx = (nx + 1) >> 1, hy = (ny + 1) >> 1, I = t % hx, J = t / hx;
-    unsigned m = 0;
-    if (J < hy) {
-        m = 1u;
-        if (I > 0) m |= 2u;
-        if (2 * I + 2 < nx) m |= 4u;
-        if (J > 0) m |= 8u;
-        if (2 * J + 2 < ny) m |= 16u;
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-                if (2 * I + e < nx && 2 * J + r < ny) m |= 32u << (2 * r + e);
-    }
-    B.m = m;
-    B.q = 2 * J * hx + I;
+__device__ __forceinline__ void small_place(SmallBlk<T, NR>& B, int hx, int hy, int t, int& I, int& J) {
+    J = small_div(t, hx);
+    I = t - J * hx;
+    B.own = J < hy;
+    B.q = xidx(hx, I, 2 * J);
 }
 
 // the block's weights, reciprocal diagonals and right-hand side from shared memory; DOWN: also D,
 // and in FP32 the reciprocal diagonals are computed here and kept in shared memory for the up leg
-// (read back by the same thread)
-template <typename T, int NR, bool DOWN>
+// (read back by the same thread).  ODD: the level may have odd sides.
+template <typename T, int NR, bool DOWN, bool ODD>
 __device__ inline void small_load(SmallBlk<T, NR>& B, T (&d)[2][2], const SmallPlan& P, int l, SmallMem<T, NR>& M,
-                                  int t) {
-    const int nx = P.nx[l], hx = (nx + 1) >> 1, I = t % hx, J = t / hx;
-    const int c0 = P.soff[l] + 2 * J * nx + 2 * I;   // cell (0, 0) of the block
+                                  int I, int J) {
+    const int nx = P.nx[l], ny = P.ny[l], c0 = P.soff[l] + 2 * J * nx + 2 * I;   // cell (0, 0) of the block
+    const bool right = 2 * I + 2 < nx, up = 2 * J + 2 < ny;
+    using P2 = Vec<T, 2>;
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
+        const int c = c0 + r * nx;
+        if constexpr (ODD) {
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const bool in = B.cell(r, e);
-            const int c = in ? c0 + r * nx + e : P.soff[l];
-            B.wl[r][e] = in ? M.wl[c] : T(0);
-            B.wb[r][e] = in ? M.wb[c] : T(0);
-            if (DOWN) d[r][e] = in ? M.d[c] : T(1);
-            if (!DOWN || sizeof(T) == 8) B.id[r][e] = in ? M.id[c] : T(1);
-            Vec<T, NR> bv = M.b[c];
+            for (int e = 0; e < 2; ++e) {
+                const bool in = 2 * I + e < nx && 2 * J + r < ny;
+                const int ce = in ? c + e : P.soff[l];
+                B.wl[r][e] = in ? M.wl[ce] : T(0);
+                B.wb[r][e] = in ? M.wb[ce] : T(0);
+                if (DOWN) d[r][e] = in ? M.d[ce] : T(1);
+                if (!DOWN || sizeof(T) == 8) B.id[r][e] = in ? M.id[ce] : T(1);
+                const Vec<T, NR> bv = M.b[ce];
 #pragma unroll
-            for (int k = 0; k < NR; ++k) B.b[r][e].v[k] = in ? bv.v[k] : T(0);
+                for (int k = 0; k < NR; ++k) B.b[r][e].v[k] = in ? bv.v[k] : T(0);
+            }
+            B.wl[r][2] = right && 2 * J + r < ny ? M.wl[c + 2] : T(0);
+        } else {
+            const P2 w = *reinterpret_cast<const P2*>(M.wl + c), v = *reinterpret_cast<const P2*>(M.wb + c);
+            const Vec<T, 2 * NR> bv = *reinterpret_cast<const Vec<T, 2 * NR>*>(M.b + c);
+            const T wr = M.wl[c + 2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                B.wl[r][e] = w.v[e];
+                B.wb[r][e] = v.v[e];
+#pragma unroll
+                for (int k = 0; k < NR; ++k) B.b[r][e].v[k] = bv.v[e * NR + k];
+            }
+            B.wl[r][2] = right ? wr : T(0);
+            if (DOWN) {
+                const P2 dv = *reinterpret_cast<const P2*>(M.d + c);
+                d[r][0] = dv.v[0];
+                d[r][1] = dv.v[1];
+            }
+            if (!DOWN || sizeof(T) == 8) {
+                const P2 iv = *reinterpret_cast<const P2*>(M.id + c);
+                B.id[r][0] = iv.v[0];
+                B.id[r][1] = iv.v[1];
+            }
         }
-        const bool right = B.has(1) && B.cell(r, 1);
-        B.wl[r][2] = right ? M.wl[c0 + r * nx + 2] : T(0);
     }
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-        const bool up = B.has(3) && B.cell(1, e);
-        B.wb[2][e] = up ? M.wb[c0 + 2 * nx + e] : T(0);
+        if constexpr (ODD) {
+            B.wb[2][e] = up && 2 * I + e < nx ? M.wb[c0 + 2 * nx + e] : T(0);
+        } else {
+            const T wt = M.wb[c0 + 2 * nx + e];
+            B.wb[2][e] = up ? wt : T(0);
+        }
     }
     if (DOWN && sizeof(T) == 4) {
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
+        for (int r = 0; r < 2; ++r) {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 B.id[r][e] = rcp_diag(d[r][e] + B.wl[r][e] + B.wl[r][e + 1] + B.wb[r][e] + B.wb[r + 1][e]);
-                if (B.cell(r, e)) M.id[c0 + r * nx + e] = B.id[r][e];
+                if (ODD && 2 * I + e < nx && 2 * J + r < ny) M.id[c0 + r * nx + e] = B.id[r][e];
             }
+            if constexpr (!ODD) {
+                P2 iv;
+                iv.v[0] = B.id[r][0];
+                iv.v[1] = B.id[r][1];
+                *reinterpret_cast<P2*>(M.id + c0 + r * nx) = iv;
+            }
+        }
     }
-}
-
-// neighbour values of cell (r, e): own cells from registers, the others from the x array of
-// the other colour
-template <typename T, int NR>
-__device__ inline void small_nb(const SmallBlk<T, NR>& B, const Vec<T, NR>* xo, int hx, int r, int e, Vec<T, NR>& xl,
-                                Vec<T, NR>& xr, Vec<T, NR>& xd, Vec<T, NR>& xu) {
-    Vec<T, NR> z;
 #pragma unroll
-    for (int k = 0; k < NR; ++k) z.v[k] = T(0);
-    const int q = B.q + r * hx;
-    xl = e == 1 ? B.x[r][0] : (B.has(0) ? xo[q - 1] : z);
-    xr = e == 0 ? B.x[r][1] : (B.has(1) ? xo[q + 1] : z);
-    xd = r == 1 ? B.x[0][e] : (B.has(2) ? xo[q - hx] : z);
-    xu = r == 0 ? B.x[1][e] : (B.has(3) ? xo[q + hx] : z);
+    for (int r = 0; r < 2; ++r) B.wl[r][0] = I > 0 ? B.wl[r][0] : T(0);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) B.wb[0][e] = J > 0 ? B.wb[0][e] : T(0);
 }
 
-// one red-black half-sweep of colour COLOR over the K blocks of a thread
+// (b + sum of w x_n) / diagonal of cell (r, e), its outer neighbours' values h (horizontal) and v
+// (vertical) given, the other two the thread's own cells
+template <typename T, int NR>
+__device__ __forceinline__ Vec<T, NR> small_update(const SmallBlk<T, NR>& B, int r, int e, const Vec<T, NR>& h,
+                                                   const Vec<T, NR>& v) {
+    Vec<T, NR> a;
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+        const T xl = e == 1 ? B.x[r][0].v[k] : h.v[k], xr = e == 0 ? B.x[r][1].v[k] : h.v[k];
+        const T xd = r == 1 ? B.x[0][e].v[k] : v.v[k], xu = r == 0 ? B.x[1][e].v[k] : v.v[k];
+        a.v[k] = (B.b[r][e].v[k] + B.wl[r][e] * xl + B.wl[r][e + 1] * xr + B.wb[r][e] * xd + B.wb[r + 1][e] * xu) *
+                 B.id[r][e];
+    }
+    return a;
+}
+// the outer neighbours of the block's two cells of colour COLOR, (0, COLOR) and (1, 1 - COLOR)
+template <typename T, int NR, int COLOR>
+__device__ __forceinline__ void small_outer(const SmallBlk<T, NR>& B, const Vec<T, NR>* xo, int hx, Vec<T, NR>& h0,
+                                            Vec<T, NR>& v0, Vec<T, NR>& h1, Vec<T, NR>& v1) {
+    h0 = xo[B.q + (COLOR ? 1 : -1)];
+    v0 = xo[B.q - hx];
+    h1 = xo[B.q + hx + (COLOR ? -1 : 1)];
+    v1 = xo[B.q + 2 * hx];
+}
+
+// one red-black half-sweep of colour COLOR over the K blocks of a thread (x: nxc entries per colour)
 template <typename T, int NR, int K, int COLOR>
 __device__ inline void small_sweep(SmallBlk<T, NR> (&B)[K], Vec<T, NR>* x, int nxc, int hx, int l, int team) {
     const Vec<T, NR>* xo = x + (1 - COLOR) * nxc;
     Vec<T, NR>* xs = x + COLOR * nxc;
 #pragma unroll
     for (int u = 0; u < K; ++u)
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int e = COLOR ^ r;
-            if (B[u].cell(r, e)) {
-                Vec<T, NR> xl, xr, xd, xu, a;
-                small_nb(B[u], xo, hx, r, e, xl, xr, xd, xu);
-#pragma unroll
-                for (int k = 0; k < NR; ++k)
-                    a.v[k] = (B[u].b[r][e].v[k] + B[u].wl[r][e] * xl.v[k] + B[u].wl[r][e + 1] * xr.v[k] +
-                              B[u].wb[r][e] * xd.v[k] + B[u].wb[r + 1][e] * xu.v[k]) *
-                             B[u].id[r][e];
-                B[u].x[r][e] = a;
-                xs[B[u].q + r * hx] = a;
-            }
+        if (B[u].own) {
+            Vec<T, NR> h0, v0, h1, v1;
+            small_outer<T, NR, COLOR>(B[u], xo, hx, h0, v0, h1, v1);
+            const Vec<T, NR> a0 = small_update(B[u], 0, COLOR, h0, v0), a1 = small_update(B[u], 1, 1 - COLOR, h1, v1);
+            B[u].x[0][COLOR] = a0;
+            B[u].x[1][1 - COLOR] = a1;
+            xs[B[u].q] = a0;
+            xs[B[u].q + hx] = a1;
         }
     team_sync(l, team);
+}
+
+// residual of a cell of column parity e on the single-block levels: the flux form with the
+// rounding of its first sum fixed (one right-hand side fuses D x in the cells whose left
+// neighbour is in their block, two fuse the first flux)
+template <typename T, int NR>
+__device__ __forceinline__ T small_residual(int e, T b, T d, T w0, T w1, T w2, T w3, T x, T xl, T xr, T xd, T xu) {
+    T ax;
+    if (NR == 1 && e == 1) ax = fma_rn(d, x, w0 * (x - xl));
+    else ax = fma_rn(w0, x - xl, d * x);
+    ax = fma_rn(w1, x - xr, ax);
+    ax = fma_rn(w2, x - xd, ax);
+    ax = fma_rn(w3, x - xu, ax);
+    return b - ax;
+}
+// sum of the residuals of the block's four cells; TILE: in the form of the tile kernels
+template <typename T, int NR, bool TILE>
+__device__ __forceinline__ Vec<T, NR> small_restrict(const SmallBlk<T, NR>& B, const T (&d)[2][2], const Vec<T, NR>* x,
+                                                     int nxc, int hx) {
+    Vec<T, NR> h[2][2], v[2][2], acc;   // outer neighbours of cell (r, e)
+    small_outer<T, NR, 0>(B, x + nxc, hx, h[0][0], v[0][0], h[1][1], v[1][1]);
+    small_outer<T, NR, 1>(B, x, hx, h[0][1], v[0][1], h[1][0], v[1][0]);
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+        T res[2][2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const T xl = e == 1 ? B.x[r][0].v[k] : h[r][e].v[k], xr = e == 0 ? B.x[r][1].v[k] : h[r][e].v[k];
+                const T xd = r == 1 ? B.x[0][e].v[k] : v[r][e].v[k], xu = r == 0 ? B.x[1][e].v[k] : v[r][e].v[k];
+                if constexpr (TILE)
+                    res[r][e] = cell_residual(B.b[r][e].v[k], d[r][e], B.wl[r][e], B.wl[r][e + 1], B.wb[r][e],
+                                              B.wb[r + 1][e], B.x[r][e].v[k], xl, xr, xd, xu);
+                else
+                    res[r][e] = small_residual<T, NR>(e, B.b[r][e].v[k], d[r][e], B.wl[r][e], B.wl[r][e + 1],
+                                                      B.wb[r][e], B.wb[r + 1][e], B.x[r][e].v[k], xl, xr, xd, xu);
+            }
+        acc.v[k] = res[0][0] + res[0][1] + res[1][0] + res[1][1];
+    }
+    return acc;
 }
 
 // down leg of level l from x = 0 (its first colour-0 half-sweep reads only zeros and reduces to
@@ -1120,68 +1221,34 @@ __device__ inline void small_sweep(SmallBlk<T, NR> (&B)[K], Vec<T, NR>* x, int n
 template <typename T, int NR, int K>
 __device__ inline void small_down(const SmallPlan& P, int l, SmallMem<T, NR>& M, int team) {
     static_assert(NU_SMALL == 2, "the sweep sequences below are written out for two pairs");
-    const int nx = P.nx[l], ny = P.ny[l], hx = (nx + 1) >> 1, nxc = hx * ny;
+    const int hx = P.nx[l] >> 1, hy = P.ny[l] >> 1, nxc = x_entries(hx, 2 * hy);
     Vec<T, NR>* x = M.x + P.xoff[l];
     SmallBlk<T, NR> B[K];
     T d[K][2][2];
 #pragma unroll
     for (int u = 0; u < K; ++u) {
-        const int t = threadIdx.x + u * team;
-        small_place(B[u], nx, ny, t);
-        if (!B[u].own()) continue;
-        small_load<T, NR, true>(B[u], d[u], P, l, M, t);
+        int I, J;
+        small_place(B[u], hx, hy, threadIdx.x + u * team, I, J);
+        if (!B[u].own) continue;
+        small_load<T, NR, true, false>(B[u], d[u], P, l, M, I, J);
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
+        for (int r = 0; r < 2; ++r) {
 #pragma unroll
             for (int k = 0; k < NR; ++k) {
                 B[u].x[r][r].v[k] = B[u].b[r][r].v[k] * B[u].id[r][r];
                 B[u].x[r][1 - r].v[k] = T(0);
             }
-#pragma unroll
-        for (int r = 0; r < 2; ++r) x[B[u].q + r * hx] = B[u].x[r][r];
+            x[B[u].q + r * hx] = B[u].x[r][r];
+        }
     }
     team_sync(l, team);
     small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
     small_sweep<T, NR, K, 0>(B, x, nxc, hx, l, team);
     small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
-    Vec<T, NR>* bc = M.b + P.soff[l + 1];
 #pragma unroll
-    for (int u = 0; u < K; ++u) {
-        if (!B[u].own()) continue;
-        Vec<T, NR> acc;
-#pragma unroll
-        for (int k = 0; k < NR; ++k) acc.v[k] = T(0);
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                Vec<T, NR> xl, xr, xd, xu;
-                const Vec<T, NR> xv = B[u].x[r][e];
-                small_nb(B[u], x + (1 - (r ^ e)) * nxc, hx, r, e, xl, xr, xd, xu);
-                // a face without a neighbour has no flux: its term is w (x - x)
-                if (e == 0 && !B[u].has(0)) xl = xv;
-                if (e == 1 && !B[u].has(1)) xr = xv;
-                if (r == 0 && !B[u].has(2)) xd = xv;
-                if (r == 1 && !B[u].has(3)) xu = xv;
-#pragma unroll
-                for (int k = 0; k < NR; ++k) {
-                    // (the rounding of the first sum: one right-hand side fuses D x of the
-                    // cells with a left neighbour in the block, two fuse the flux)
-                    T ax;
-                    if (NR == 1 && e == 1) {
-                        ax = fma_rn(d[u][r][e], xv.v[k], B[u].wl[r][e] * (xv.v[k] - xl.v[k]));
-                    } else {
-                        ax = d[u][r][e] * xv.v[k];
-                        ax = fma_rn(B[u].wl[r][e], xv.v[k] - xl.v[k], ax);
-                    }
-                    ax = fma_rn(B[u].wl[r][e + 1], xv.v[k] - xr.v[k], ax);
-                    ax = fma_rn(B[u].wb[r][e], xv.v[k] - xd.v[k], ax);
-                    ax = fma_rn(B[u].wb[r + 1][e], xv.v[k] - xu.v[k], ax);
-                    acc.v[k] += B[u].b[r][e].v[k] - ax;
-                }
-            }
-        bc[threadIdx.x + u * team] = acc;
-    }
+    for (int u = 0; u < K; ++u)   // block t is the four children of cell t of level l + 1
+        if (B[u].own)
+            M.b[P.soff[l + 1] + threadIdx.x + u * team] = small_restrict<T, NR, false>(B[u], d[u], x, nxc, hx);
     team_sync(l, team);
 }
 
@@ -1190,7 +1257,7 @@ __device__ inline void small_down(const SmallPlan& P, int l, SmallMem<T, NR>& M,
 template <typename T, int NR>
 __device__ inline void small_coarsest(const SmallPlan& P, SmallMem<T, NR>& M, bool exact) {
     const int l = P.n - 1, o = P.soff[l], nx = P.nx[l], ny = P.ny[l], n = nx * ny;
-    const int hx = (nx + 1) >> 1, nxc = hx * ny;
+    const int hx = (nx + 1) >> 1, hy = (ny + 1) >> 1, nxc = x_entries(hx, 2 * hy);
     Vec<T, NR>* x = M.x + P.xoff[l];
     const int team = exact ? 32 : small_team(nx, ny);
     if (threadIdx.x >= team) return;
@@ -1207,23 +1274,24 @@ __device__ inline void small_coarsest(const SmallPlan& P, SmallMem<T, NR>& M, bo
 #pragma unroll
                 for (int k = 0; k < NR; ++k) acc.v[k] += a * bv.v[k];
             }
-            const int i = r % nx, j = r / nx;
-            x[((i + j) & 1) * nxc + j * hx + (i >> 1)] = acc;
+            const int j = small_div(r, nx), i = r - j * nx;
+            x[((i + j) & 1) * nxc + xidx(hx, i >> 1, j)] = acc;
         }
         return;
     }
     SmallBlk<T, NR> B[1];
     T d[2][2];
-    small_place(B[0], nx, ny, threadIdx.x);
-    if (B[0].own()) {
-        small_load<T, NR, true>(B[0], d, P, l, M, threadIdx.x);
+    int I, J;
+    small_place(B[0], hx, hy, threadIdx.x, I, J);
+    if (B[0].own) {
+        small_load<T, NR, true, true>(B[0], d, P, l, M, I, J);
 #pragma unroll
         for (int r = 0; r < 2; ++r)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
 #pragma unroll
                 for (int k = 0; k < NR; ++k) B[0].x[r][e].v[k] = T(0);
-                if (2 * (B[0].q / (2 * hx)) + r < ny) x[(e ^ r) * nxc + B[0].q + r * hx] = B[0].x[r][e];
+                x[(e ^ r) * nxc + B[0].q + r * hx] = B[0].x[r][e];
             }
     }
     team_sync(l, team);
@@ -1241,18 +1309,20 @@ __device__ inline void small_coarsest(const SmallPlan& P, SmallMem<T, NR>& M, bo
 // joins the level's team with the warps that worked on the coarser levels.
 template <typename T, int NR, int K>
 __device__ inline void small_up(const SmallPlan& P, int l, SmallMem<T, NR>& M, int team) {
-    const int nx = P.nx[l], ny = P.ny[l], hx = (nx + 1) >> 1, nxc = hx * ny;
-    const int cnx = P.nx[l + 1], chx = (cnx + 1) >> 1, cnxc = chx * P.ny[l + 1];
+    const int hx = P.nx[l] >> 1, hy = P.ny[l] >> 1, nxc = x_entries(hx, 2 * hy);
+    const int chx = (P.nx[l + 1] + 1) >> 1, cnxc = x_entries(chx, (P.ny[l + 1] + 1) & ~1);
     Vec<T, NR>* x = M.x + P.xoff[l];
     const Vec<T, NR>* xc = M.x + P.xoff[l + 1];
     SmallBlk<T, NR> B[K];
+    int qc[K];
 #pragma unroll
     for (int u = 0; u < K; ++u) {
-        const int t = threadIdx.x + u * team;
-        small_place(B[u], nx, ny, t);
+        int I, J;
+        small_place(B[u], hx, hy, threadIdx.x + u * team, I, J);
+        qc[u] = ((I + J) & 1) * cnxc + xidx(chx, I >> 1, J);
         T d[2][2];
-        if (B[u].own()) {
-            small_load<T, NR, false>(B[u], d, P, l, M, t);
+        if (B[u].own) {
+            small_load<T, NR, false, false>(B[u], d, P, l, M, I, J);
 #pragma unroll
             for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -1262,9 +1332,8 @@ __device__ inline void small_up(const SmallPlan& P, int l, SmallMem<T, NR>& M, i
     team_sync(l, team);
 #pragma unroll
     for (int u = 0; u < K; ++u) {
-        if (!B[u].own()) continue;
-        const int t = threadIdx.x + u * team, I = t % hx, J = t / hx;
-        const Vec<T, NR> cv = xc[((I + J) & 1) * cnxc + J * chx + (I >> 1)];
+        if (!B[u].own) continue;
+        const Vec<T, NR> cv = xc[qc[u]];
 #pragma unroll
         for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -1281,50 +1350,20 @@ __device__ inline void small_up(const SmallPlan& P, int l, SmallMem<T, NR>& M, i
     small_sweep<T, NR, K, 0>(B, x, nxc, hx, l, team);
 }
 
-// the V-cycle on the small levels in one block of SMALL_THREADS threads, from the level-(first
-// small) rhs b_in to its correction x_out; with DOT (the cycle starts at the finest level) also
-// r.z -> beta
-template <typename T, int NR, bool DOT>
-__device__ void small_cycle(const SmallPlan& P, const T* __restrict__ diag, const T* __restrict__ id,
-                            const T* __restrict__ wl, const T* __restrict__ wb, const T* __restrict__ inv, const T* __restrict__ b_in,
-                            T* __restrict__ x_out, SolveState* st, unsigned char* smem) {
-    SmallMem<T, NR> M(smem, P);
-    const int nlast = P.nx[P.n - 1] * P.ny[P.n - 1];
-    // the small levels are contiguous in the packed level arrays and in shared memory: one flat
-    // copy per array, four independent loads in flight per thread and array
-    {
-        const T* gd = diag + P.goff[0];
-        const T* gl = wl + P.goff[0];
-        const T* gb = wb + P.goff[0];
-        int tot = P.total;
-#pragma unroll 4
-        for (int c = threadIdx.x; c < tot; c += blockDim.x) {
-            T a = gd[c], b2 = gl[c], c2 = gb[c];
-            M.d[c] = a;
-            M.wl[c] = b2;
-            M.wb[c] = c2;
-            if (sizeof(T) == 8) M.id[c] = id[P.goff[0] + c];
-        }
-    }
-    const int n0 = P.nx[0] * P.ny[0];
-    const Vec<T, NR>* bv = reinterpret_cast<const Vec<T, NR>*>(b_in);
-#pragma unroll 4
-    for (int c = threadIdx.x; c < n0; c += blockDim.x) M.b[c] = bv[c];
-    const bool exact = nlast <= 32 && inv[nlast * nlast] == T(1);
-    if (exact)
-        for (int c = threadIdx.x; c < nlast * nlast; c += blockDim.x) M.inv[(c % nlast) * nlast + c / nlast] = inv[c];
-    __syncthreads();
-    // every level's down leg on its team, the coarsest solve, the up legs: a warp leaves at the first
-    // level it owns no cells of and waits for the others at that level's (the previous team's)
-    // up leg
+// the cycle on levels whose operators and level-0 right-hand side are in shared memory: every
+// level's down leg on its team, the coarsest solve, the up legs.  A warp leaves at the first level
+// it owns no cells of and waits for the others at the up leg of the level before.  BIG: the first
+// level may have more blocks than the team has threads (two per thread).
+template <typename T, int NR, bool BIG>
+__device__ inline void small_core(const SmallPlan& P, SmallMem<T, NR>& M, bool exact) {
     const int tid = threadIdx.x;
     int lmax = 0;   // levels [0, lmax) with this thread in the team
     while (lmax < P.n - 1 && tid < small_team(P.nx[lmax], P.ny[lmax])) ++lmax;
-    const bool two = ((P.nx[0] + 1) >> 1) * ((P.ny[0] + 1) >> 1) > SMALL_THREADS;   // level 0: two blocks per thread
+    const bool two = BIG && ((P.nx[0] + 1) >> 1) * ((P.ny[0] + 1) >> 1) > (int)blockDim.x;   // level 0: two blocks per thread
     for (int l = 0; l < lmax; ++l) {
         const int team = small_team(P.nx[l], P.ny[l]);
         bool done = false;
-        if constexpr (sizeof(T) == 4)
+        if constexpr (BIG)
             if (l == 0 && two) {
                 small_down<T, NR, 2>(P, l, M, team);
                 done = true;
@@ -1338,7 +1377,7 @@ __device__ void small_cycle(const SmallPlan& P, const T* __restrict__ diag, cons
     for (int l = lmax - 1; l >= 0; --l) {
         const int team = small_team(P.nx[l], P.ny[l]);
         bool done = false;
-        if constexpr (sizeof(T) == 4)
+        if constexpr (BIG)
             if (l == 0 && two) {
                 small_up<T, NR, 2>(P, l, M, team);
                 done = true;
@@ -1346,11 +1385,71 @@ __device__ void small_cycle(const SmallPlan& P, const T* __restrict__ diag, cons
         if (!done) small_up<T, NR, 1>(P, l, M, team);
     }
     __syncthreads();
-    const int nx0 = P.nx[0], hx0 = (nx0 + 1) >> 1, nxc0 = hx0 * P.ny[0];
+}
+
+// the small levels' operators into shared memory (asynchronous copies: the caller waits and meets
+// at a block barrier), x zeroed; true if the coarsest level has its inverse
+template <typename T, int NR>
+__device__ inline bool small_operators(const SmallPlan& P, SmallMem<T, NR>& M, const T* diag, const T* id, const T* wl,
+                                       const T* wb, const T* inv) {
+    const size_t g = P.goff[0];
+    const int n = P.nx[P.n - 1] * P.ny[P.n - 1];
+    const bool try_inv = n <= 32;
+    copy_async(M.d, diag + g, P.cells);
+    copy_async(M.wl, wl + g, P.cells);
+    copy_async(M.wb, wb + g, P.cells);
+    if (sizeof(T) == 8) copy_async(M.id, id + g, P.cells);
+    // the inverse is copied whether usable or not, beside the word that says so
+    T usable = T(0), v[2] = {T(0), T(0)};
+    if (try_inv) {
+        usable = inv[n * n];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int c = threadIdx.x + u * blockDim.x;
+            if (c < n * n) v[u] = inv[c];
+        }
+    }
+    for (int c = threadIdx.x; c < P.xtotal; c += blockDim.x) {
+        Vec<T, NR> z;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) z.v[k] = T(0);
+        M.x[c] = z;
+    }
+    if (try_inv)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int c = threadIdx.x + u * blockDim.x;
+            if (c < n * n) {
+                const int r = small_div(c, n);
+                M.inv[(c - r * n) * n + r] = v[u];
+            }
+        }
+    if (try_inv)
+        for (int c = threadIdx.x + 2 * blockDim.x; c < n * n; c += blockDim.x) M.inv[(c % n) * n + c / n] = inv[c];
+    return try_inv && usable == T(1);
+}
+
+// the V-cycle on the small levels in one block of SMALL_THREADS threads, from the level-(first
+// small) rhs b_in to its correction x_out; with DOT (the cycle starts at the finest level) also
+// r.z -> beta
+template <typename T, int NR, bool DOT>
+__device__ void small_cycle(const SmallPlan& P, const T* __restrict__ diag, const T* __restrict__ id,
+                            const T* __restrict__ wl, const T* __restrict__ wb, const T* __restrict__ inv, const T* __restrict__ b_in,
+                            T* __restrict__ x_out, SolveState* st, unsigned char* smem) {
+    SmallMem<T, NR> M(smem, P);
+    const int n0 = P.nx[0] * P.ny[0];
+    // the small levels are contiguous in the packed level arrays and in shared memory: one flat
+    // asynchronous copy per array, all in flight together
+    copy_async((T*)M.b, b_in, n0 * NR);
+    const bool exact = small_operators<T, NR>(P, M, diag, id, wl, wb, inv);
+    cp_async_wait_all();
+    __syncthreads();
+    small_core<T, NR, sizeof(T) == 4>(P, M, exact);
+    const int nx0 = P.nx[0], hx0 = (nx0 + 1) >> 1, nxc0 = x_entries(hx0, (P.ny[0] + 1) & ~1);
     const Vec<T, NR>* x0 = M.x + P.xoff[0];
     auto xat = [&](int c) {
-        const int i = c % nx0, j = c / nx0;
-        return x0[((i + j) & 1) * nxc0 + j * hx0 + (i >> 1)];
+        const int j = small_div(c, nx0), i = c - j * nx0;
+        return x0[((i + j) & 1) * nxc0 + xidx(hx0, i >> 1, j)];
     };
     for (int c = threadIdx.x; c < n0; c += blockDim.x) reinterpret_cast<Vec<T, NR>*>(x_out)[c] = xat(c);
     if (DOT) {
@@ -1477,6 +1576,335 @@ __global__ void __launch_bounds__(CC_THREADS) k_coarse_cycle(CoarsePlan<T> C, Sm
             __syncthreads();
         }
         if (l > C.l0) grid_sync(bar, gen, st, C.spin);
+    }
+}
+
+// ---- the coarse part of the V-cycle in one thread-block cluster ----------------------------
+// The coarse levels of a single instance are latency-bound: in the grid-barrier launch above a
+// phase costs 2 to 3 us (load a tile from L2, sweep, store) and a barrier 0.9 to 1.4 us.  Here one
+// cluster of up to 16 blocks (16 SMs) keeps the levels [l0, nb) in its shared memory: block k of
+// the cluster owns rows [k rp, (k + 1) rp) of a level (rp even), thread t of it 2 x 2 blocks of
+// cells as in the single-block levels.  After a half-sweep of one colour the edge rows' new
+// values are stored into the neighbour blocks' halo rows through distributed shared memory, and
+// a cluster barrier (0.2 us; store, barrier and read of a pushed value 0.3 to 0.4 us) ends the
+// phase.  Operators are copied from global memory once per launch, the levels exchange their
+// right-hand sides and corrections through distributed shared memory, and block 0 runs the
+// single-block levels.  The arithmetic of every cell is that of the tile kernels.
+// Measured per launch against the grid-barrier launch or the separate ones (one right-hand side):
+// FP32 on a 128^2 grid 17.6 -> 12.8 us, on 512^2 31.2 -> 29 (its 256^2 level costs what two separate
+// launches do); FP64 from the 128^2 level down 80 -> 47 us.  A 64^2 level of four rows per block
+// spends about 1000 cycles a phase, 750 of them push and barrier.
+constexpr int CL_MAX = 6;            // levels kept by the cluster, at most
+constexpr int CL_BLOCKS = 16;        // blocks of the cluster (16 needs the non-portable attribute)
+constexpr int CL_THREADS = 512;      // threads per block, at most (the registers are budgeted for it)
+struct ClPlan {
+    int nl;                          // levels kept by the cluster
+    int nt;                          // of these, the first nt are tiled levels of the separate launches
+    int nx[CL_MAX], ny[CL_MAX], rp[CL_MAX];
+    int off[CL_MAX];                 // byte offset of the level's arrays in every block's shared memory
+    size_t goff[CL_MAX];             // cell offset in the packed level arrays
+    SmallPlan S;                     // the single-block levels, at byte offset soff of block 0
+    int soff;
+};
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// the same shared-memory object in block `rank` of the cluster (a generic address)
+template <class P>
+__device__ __forceinline__ P* cluster_map(P* p, unsigned rank) {
+    unsigned long long r;
+    asm("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"((unsigned long long)(uintptr_t)p), "r"(rank));
+    return reinterpret_cast<P*>((uintptr_t)r);
+}
+// a level's arrays in a block's shared memory: x (rows -1 .. rp, as on the single-block levels),
+// b, then D, wl, wb (one row more) and, in FP64, the reciprocal diagonals
+template <typename T, int NR>
+struct ClMem {
+    Vec<T, NR>*x, *b;
+    T *d, *wl, *wb, *id;
+    __host__ __device__ static int xn(int nx, int rp) { return (2 * x_entries(nx >> 1, rp) + 3) & ~3; }
+    __device__ ClMem(unsigned char* base, int nx, int rp) {
+        x = (Vec<T, NR>*)base;
+        b = x + xn(nx, rp);
+        d = (T*)(b + rp * nx);
+        wl = d + rp * nx;
+        id = wl + rp * nx;
+        wb = id + (sizeof(T) == 8 ? rp * nx : 0);
+    }
+    static int bytes(int nx, int rp) {
+        size_t v = (size_t)(xn(nx, rp) + rp * nx) * NR, c = (size_t)(3 * rp + 1) * nx + (sizeof(T) == 8 ? rp * nx : 0);
+        return (int)(((v + c + 2) * sizeof(T) + 127) & ~size_t(127));
+    }
+};
+// a block's slab of a level
+struct ClSlab {
+    int nx, hx, rp, j0, j1, nxc;     // rows [j0, j1); nxc entries per colour of x
+    __device__ ClSlab(const ClPlan& P, int l, int rank) {
+        nx = P.nx[l];
+        hx = nx >> 1;
+        rp = P.rp[l];
+        j0 = min(rank * rp, P.ny[l]);
+        j1 = min(j0 + rp, P.ny[l]);
+        nxc = x_entries(hx, rp);
+    }
+};
+// edge of a slab that a block of cells lies on (its new values are pushed there)
+constexpr unsigned CL_DOWN = 1, CL_UP = 2;
+
+// the block's place, weights, reciprocal diagonals, D and right-hand side
+template <typename T, int NR>
+__device__ inline unsigned cl_load(SmallBlk<T, NR>& B, T (&d)[2][2], const ClSlab& S, int ny, const ClMem<T, NR>& M,
+                                   int t, int& I, int& J) {
+    small_place(B, S.hx, (S.j1 - S.j0) >> 1, t, I, J);
+    if (!B.own) return 0;
+    const int c0 = 2 * J * S.nx + 2 * I;
+    using P2 = Vec<T, 2>;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int c = c0 + r * S.nx;
+        const P2 w = *reinterpret_cast<const P2*>(M.wl + c), v = *reinterpret_cast<const P2*>(M.wb + c);
+        const P2 dv = *reinterpret_cast<const P2*>(M.d + c);
+        const Vec<T, 2 * NR> bv = *reinterpret_cast<const Vec<T, 2 * NR>*>(M.b + c);
+        const T wr = M.wl[c + 2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            B.wl[r][e] = w.v[e];
+            B.wb[r][e] = v.v[e];
+            d[r][e] = dv.v[e];
+#pragma unroll
+            for (int k = 0; k < NR; ++k) B.b[r][e].v[k] = bv.v[e * NR + k];
+        }
+        B.wl[r][2] = I + 1 < S.hx ? wr : T(0);
+        if (sizeof(T) == 8) {
+            const P2 iv = *reinterpret_cast<const P2*>(M.id + c);
+            B.id[r][0] = iv.v[0];
+            B.id[r][1] = iv.v[1];
+        }
+    }
+    const P2 wt = *reinterpret_cast<const P2*>(M.wb + c0 + 2 * S.nx);
+    B.wb[2][0] = wt.v[0];
+    B.wb[2][1] = wt.v[1];
+    if (sizeof(T) == 4) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                B.id[r][e] = rcp_diag(d[r][e] + B.wl[r][e] + B.wl[r][e + 1] + B.wb[r][e] + B.wb[r + 1][e]);
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) B.wl[r][0] = I > 0 ? B.wl[r][0] : T(0);
+    return (J == 0 && S.j0 > 0 ? CL_DOWN : 0u) | (S.j0 + 2 * J + 2 == S.j1 && S.j1 < ny ? CL_UP : 0u);
+}
+// the new values of colour COLOR in the block's edge rows, into the neighbour slabs' halo rows
+template <typename T, int NR>
+__device__ __forceinline__ void cl_push(const SmallBlk<T, NR>& B, unsigned edge, const ClSlab& S, Vec<T, NR>* xdn,
+                                        Vec<T, NR>* xup, int color) {
+    // entries of the block's column in row rp of the slab below and in row -1 of the slab above
+    if (edge & CL_DOWN) xdn[color * S.nxc + B.q + S.rp * S.hx] = color ? B.x[0][1] : B.x[0][0];
+    if (edge & CL_UP) xup[color * S.nxc + B.q - (S.j1 - S.j0 - 1) * S.hx] = color ? B.x[1][0] : B.x[1][1];
+}
+template <typename T, int NR, int K, int COLOR, bool LAST = false>
+__device__ inline void cl_sweep(SmallBlk<T, NR> (&B)[K], const unsigned (&edge)[K], const ClSlab& S, Vec<T, NR>* x,
+                                Vec<T, NR>* xdn, Vec<T, NR>* xup) {
+    const Vec<T, NR>* xo = x + (1 - COLOR) * S.nxc;
+    Vec<T, NR>* xs = x + COLOR * S.nxc;
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        if (!B[u].own) continue;
+        Vec<T, NR> h0, v0, h1, v1;
+        small_outer<T, NR, COLOR>(B[u], xo, S.hx, h0, v0, h1, v1);
+        const Vec<T, NR> a0 = small_update(B[u], 0, COLOR, h0, v0), a1 = small_update(B[u], 1, 1 - COLOR, h1, v1);
+        B[u].x[0][COLOR] = a0;
+        B[u].x[1][1 - COLOR] = a1;
+        if (!LAST) {
+            xs[B[u].q] = a0;
+            xs[B[u].q + S.hx] = a1;
+            if (edge[u]) cl_push(B[u], edge[u], S, xdn, xup, COLOR);
+        }
+    }
+    if (!LAST) cluster_barrier();
+}
+
+// down leg; TILE: the residual as in the tile kernels, else as on the single-block levels
+template <typename T, int NR, int K, bool TILE>
+__device__ inline void cl_down(const ClPlan& P, int l, int rank, unsigned char* smem) {
+    const ClSlab S(P, l, rank);
+    const ClMem<T, NR> M(smem + P.off[l], S.nx, S.rp);
+    Vec<T, NR>* xdn = cluster_map(M.x, rank > 0 ? rank - 1 : 0);
+    Vec<T, NR>* xup = cluster_map(M.x, rank + 1 < CL_BLOCKS ? rank + 1 : rank);
+    SmallBlk<T, NR> B[K];
+    T d[K][2][2];
+    unsigned edge[K];
+    int I[K], J[K];
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        edge[u] = cl_load(B[u], d[u], S, P.ny[l], M, threadIdx.x + u * blockDim.x, I[u], J[u]);
+        if (!B[u].own) continue;
+        // the first colour-0 half-sweep from x = 0 reduces to x = b / (full diagonal)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+#pragma unroll
+            for (int k = 0; k < NR; ++k) {
+                B[u].x[r][r].v[k] = B[u].b[r][r].v[k] * B[u].id[r][r];
+                B[u].x[r][1 - r].v[k] = T(0);
+            }
+            M.x[B[u].q + r * S.hx] = B[u].x[r][r];
+        }
+        if (edge[u]) cl_push(B[u], edge[u], S, xdn, xup, 0);
+    }
+    cluster_barrier();
+    cl_sweep<T, NR, K, 1>(B, edge, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 0>(B, edge, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 1>(B, edge, S, M.x, xdn, xup);
+    // the block's residual summed into the right-hand side of the next level, in the shared memory
+    // of the block that owns that cell
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        if (!B[u].own) continue;
+        const Vec<T, NR> acc = small_restrict<T, NR, TILE>(B[u], d[u], M.x, S.nxc, S.hx);
+        const int Jg = (S.j0 >> 1) + J[u];
+        if (l + 1 < P.nl) {
+            const int own = small_div(Jg, P.rp[l + 1]);
+            const ClMem<T, NR> N(smem + P.off[l + 1], P.nx[l + 1], P.rp[l + 1]);
+            cluster_map(N.b, own)[(Jg - own * P.rp[l + 1]) * P.nx[l + 1] + I[u]] = acc;
+        } else {
+            const SmallMem<T, NR> N(smem + P.soff, P.S);
+            cluster_map(N.b, 0)[Jg * P.S.nx[0] + I[u]] = acc;
+        }
+    }
+    cluster_barrier();
+}
+
+// up leg; the result of the first kept level (TOP) goes to x_out, the others' stay in shared memory
+template <typename T, int NR, int K, bool TOP>
+__device__ inline void cl_up(const ClPlan& P, int l, int rank, unsigned char* smem, T* __restrict__ x_out) {
+    const ClSlab S(P, l, rank);
+    const ClMem<T, NR> M(smem + P.off[l], S.nx, S.rp);
+    Vec<T, NR>* xdn = cluster_map(M.x, rank > 0 ? rank - 1 : 0);
+    Vec<T, NR>* xup = cluster_map(M.x, rank + 1 < CL_BLOCKS ? rank + 1 : rank);
+    SmallBlk<T, NR> B[K];
+    unsigned edge[K];
+    int I[K], J[K];
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        T d[2][2];
+        edge[u] = cl_load(B[u], d, S, P.ny[l], M, threadIdx.x + u * blockDim.x, I[u], J[u]);
+        if (!B[u].own) continue;
+        const int Jg = (S.j0 >> 1) + J[u];
+        Vec<T, NR> cv;
+        if (l + 1 < P.nl) {
+            const int own = small_div(Jg, P.rp[l + 1]), chx = P.nx[l + 1] >> 1, cnxc = x_entries(chx, P.rp[l + 1]);
+            const ClMem<T, NR> N(smem + P.off[l + 1], P.nx[l + 1], P.rp[l + 1]);
+            cv = cluster_map(N.x, own)[((I[u] + Jg) & 1) * cnxc + xidx(chx, I[u] >> 1, Jg - own * P.rp[l + 1])];
+        } else {
+            const int chx = (P.S.nx[0] + 1) >> 1, cnxc = x_entries(chx, (P.S.ny[0] + 1) & ~1);
+            const SmallMem<T, NR> N(smem + P.soff, P.S);
+            cv = cluster_map(N.x, 0)[P.S.xoff[0] + ((I[u] + Jg) & 1) * cnxc + xidx(chx, I[u] >> 1, Jg)];
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                Vec<T, NR>* p = M.x + (e ^ r) * S.nxc + B[u].q + r * S.hx;
+                B[u].x[r][e] = *p;
+#pragma unroll
+                for (int k = 0; k < NR; ++k) B[u].x[r][e].v[k] += cv.v[k];
+                *p = B[u].x[r][e];
+            }
+        if (edge[u]) cl_push(B[u], edge[u], S, xdn, xup, 0);
+    }
+    cluster_barrier();
+    cl_sweep<T, NR, K, 1>(B, edge, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 0>(B, edge, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 1>(B, edge, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 0, TOP>(B, edge, S, M.x, xdn, xup);
+    if (TOP) {
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            if (!B[u].own) continue;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                Vec<T, 2 * NR> o;
+#pragma unroll
+                for (int k = 0; k < NR; ++k) {
+                    o.v[k] = B[u].x[r][0].v[k];
+                    o.v[NR + k] = B[u].x[r][1].v[k];
+                }
+                reinterpret_cast<Vec<T, 2 * NR>*>(x_out)[(size_t)(S.j0 + 2 * J[u] + r) * S.hx + I[u]] = o;
+            }
+        }
+    }
+}
+
+template <typename T, int NR>
+__global__ void __launch_bounds__(CL_THREADS, 1)
+k_coarse_cluster(const __grid_constant__ ClPlan P, const T* __restrict__ diag, const T* __restrict__ id,
+                 const T* __restrict__ wl, const T* __restrict__ wb, const T* __restrict__ inv,
+                 const T* __restrict__ b_in, T* __restrict__ x_out, const SolveState* st) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int rank = cluster_rank();
+    // operators and the first level's right-hand side, all copies in flight at once; x zeroed
+    for (int l = 0; l < P.nl; ++l) {
+        const ClSlab S(P, l, rank);
+        const ClMem<T, NR> M(smem + P.off[l], S.nx, S.rp);
+        const int nr = S.j1 - S.j0, n = nr * S.nx;
+        const size_t g = P.goff[l] + (size_t)S.j0 * S.nx;
+        const int nwb = nr > 0 && S.j1 < P.ny[l] ? n + S.nx : n;
+        copy_async(M.d, diag + g, n);
+        copy_async(M.wl, wl + g, n);
+        copy_async(M.wb, wb + g, nwb);
+        if (sizeof(T) == 8) copy_async(M.id, id + g, n);
+        if (l == 0) copy_async((T*)M.b, b_in + (size_t)S.j0 * S.nx * NR, n * NR);
+        if (nwb == n)
+            for (int i = threadIdx.x; i < S.nx; i += blockDim.x) M.wb[n + i] = T(0);   // the grid's upper side
+        for (int i = threadIdx.x; i < 2 * S.nxc; i += blockDim.x) {
+            Vec<T, NR> z;
+#pragma unroll
+            for (int k = 0; k < NR; ++k) z.v[k] = T(0);
+            M.x[i] = z;
+        }
+    }
+    bool exact = false;
+    if (rank == 0) {
+        SmallMem<T, NR> M(smem + P.soff, P.S);
+        exact = small_operators<T, NR>(P.S, M, diag, id, wl, wb, inv);
+    }
+    const bool off = skip(st);   // written by an earlier launch: the same for every block
+    cp_async_wait_all();
+    if (off) return;
+    cluster_barrier();
+    for (int l = 0; l < P.nl; ++l) {
+        if (P.rp[l] * (P.nx[l] >> 1) > 2 * (int)blockDim.x) {
+            if constexpr (sizeof(T) == 4) cl_down<T, NR, 2, true>(P, l, rank, smem);
+        } else if (sizeof(T) == 4 || l < P.nt) {
+            cl_down<T, NR, 1, true>(P, l, rank, smem);
+        } else {
+            if constexpr (sizeof(T) == 8) cl_down<T, NR, 1, false>(P, l, rank, smem);
+        }
+    }
+    if (rank == 0) {
+        SmallMem<T, NR> M(smem + P.soff, P.S);
+        small_core<T, NR, false>(P.S, M, exact);
+    }
+    cluster_barrier();
+    for (int l = P.nl - 1; l >= 0; --l) {
+        const bool two = P.rp[l] * (P.nx[l] >> 1) > 2 * (int)blockDim.x;
+        if (two) {
+            if constexpr (sizeof(T) == 4) {
+                if (l == 0) cl_up<T, NR, 2, true>(P, l, rank, smem, x_out);
+                else cl_up<T, NR, 2, false>(P, l, rank, smem, nullptr);
+            }
+        } else if (l == 0) {
+            cl_up<T, NR, 1, true>(P, l, rank, smem, x_out);
+        } else {
+            cl_up<T, NR, 1, false>(P, l, rank, smem, nullptr);
+        }
     }
 }
 
@@ -2903,10 +3331,10 @@ template <> int nbig_of<float>(const Solver& s) { return s.nbig_f; }
 template <> int nbig_of<double>(const Solver& s) { return s.nbig_d; }
 
 template <typename T>
-static SmallPlan small_plan(const Solver& s) {
+static SmallPlan small_plan(const Solver& s, int first = -1) {
     SmallPlan P;
     P.zs = s.zs;
-    int nb = nbig_of<T>(s);
+    int nb = first >= 0 ? first : nbig_of<T>(s);
     P.n = s.nlev - nb;
     int so = 0, xo = 0;
     for (int k = 0; k < P.n; ++k) {
@@ -2917,9 +3345,10 @@ static SmallPlan small_plan(const Solver& s) {
         P.xoff[k] = xo;
         P.goff[k] = s.loff[l];
         so += s.lnx[l] * s.lny[l];
-        xo += 2 * ((s.lnx[l] + 1) / 2) * s.lny[l];
+        xo += (2 * x_entries((s.lnx[l] + 1) / 2, (s.lny[l] + 1) & ~1) + 3) & ~3;
     }
-    P.total = so;
+    P.cells = so;
+    P.total = (so + 3) & ~3;   // (a multiple of 16 bytes in every array)
     P.xtotal = xo;
     return P;
 }
@@ -2950,13 +3379,86 @@ static int coarse_start(Solver& s) {
         size_t smem = Region<T, NR, HPRE>::bytes() > Region<T, NR, HPOST>::bytes()
                           ? Region<T, NR, HPRE>::bytes()
                           : Region<T, NR, HPOST>::bytes();
-        smem = smem > SmallMem<T, NR>::bytes(5461, 5461) ? smem : SmallMem<T, NR>::bytes(5461, 5461);
+        smem = smem > SmallMem<T, NR>::bytes(5464, 2 * 3072) ? smem : SmallMem<T, NR>::bytes(5464, 2 * 3072);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_coarse_cycle<T, NR>, CC_THREADS, smem);
         res = per * sms;
         cudaGetLastError();
     }
     for (int l = 1; l < nb; ++l)
         if ((long long)((s.lnx[l] + TX - 1) / TX) * ((s.lny[l] + TY - 1) / TY) <= res) return l;
+    return nb;
+}
+
+// Plan of the cluster launch: the first tiled level l0 >= 1 from which every level fits the
+// cluster's shared memory and threads (l0 = nb: none; the finest level stays separate, its
+// post-smoothing carries the r.z of CG).  In FP64, where a half-sweep of 32 x 32 cells takes one
+// SM 0.8 us of FP64 issue against 0.45 us over the cluster, the levels above 256 cells stay in the
+// cluster; in FP32 those above the single-block size.  Single instances; a bound set for the grid
+// barriers (EBIT_OPT_BARRIER_SPIN) asks for the grid-barrier launch.
+template <typename T, int NR>
+static int cluster_plan(Solver& s, ClPlan& P, int& threads, size_t& smem) {
+    const int nb = nbig_of<T>(s);
+    if (s.use_coop != 1 || s.barrier_spin > 0 || s.nz != 1 || nb < 2) return nb;
+    static std::atomic<int> usable[64][2][2];   // per device, precision, NR: 0 not asked, 1 yes, 2 no
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return nb;
+    constexpr size_t SMEM_MAX = 216 * 1024;
+    std::atomic<int>& u = usable[dev][PT<T>::prec][NR - 1];
+    if (u.load() == 0) {
+        cudaError_t first = cudaSuccess;
+        allow_smem(k_coarse_cluster<T, NR>, (int)SMEM_MAX, &first);
+        cudaError_t e = cudaFuncSetAttribute(k_coarse_cluster<T, NR>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(CL_BLOCKS);
+        cfg.blockDim = dim3(CL_THREADS);
+        cfg.dynamicSmemBytes = SMEM_MAX;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = CL_BLOCKS;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (first == cudaSuccess && e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_coarse_cluster<T, NR>, &cfg);
+        u.store(first == cudaSuccess && e == cudaSuccess && n > 0 ? 1 : 2);
+        cudaGetLastError();
+    }
+    if (u.load() != 1) return nb;
+    int ls = nb;   // first single-block level
+    if (sizeof(T) == 8)
+        while (ls < s.nlev - 1 && s.lnx[ls] * s.lny[ls] > 256) ++ls;
+    P.S = small_plan<T>(s, ls);
+    const int last = s.nlev - 1, half = CL_THREADS / 2;
+    // (one block of cells per thread on the single-block levels)
+    int need_s = ((s.lnx[last] + 1) / 2) * ((s.lny[last] + 1) / 2);
+    if (ls < last) need_s = std::max(need_s, (s.lnx[ls] / 2) * (s.lny[ls] / 2));
+    for (int l0 = 1; l0 < nb; ++l0) {
+        if (ls - l0 > CL_MAX) continue;
+        size_t off = 0;
+        int need = need_s;
+        P.nl = ls - l0;
+        P.nt = nb - l0;
+        for (int k = 0; k < P.nl; ++k) {
+            const int l = l0 + k;
+            P.nx[k] = s.lnx[l];
+            P.ny[k] = s.lny[l];
+            P.rp[k] = 2 * ((s.lny[l] / 2 + CL_BLOCKS - 1) / CL_BLOCKS);
+            P.goff[k] = s.loff[l];
+            P.off[k] = (int)off;
+            if ((long long)P.rp[k] * P.nx[k] > 16 * CL_THREADS) {
+                off = SMEM_MAX + 1;
+                break;
+            }
+            off += ClMem<T, NR>::bytes(P.nx[k], P.rp[k]);
+            need = std::max(need, (P.rp[k] / 2) * (P.nx[k] / 2));
+        }
+        P.soff = (int)off;
+        smem = off + SmallMem<T, NR>::bytes(P.S);
+        if (smem > SMEM_MAX || need_s > CL_THREADS || need > (sizeof(T) == 4 ? 2 : 1) * CL_THREADS) continue;
+        threads = need > half ? CL_THREADS : half;
+        return l0;
+    }
     return nb;
 }
 
@@ -2998,7 +3500,12 @@ static void vcycle(Solver& s, const T* r, T* z, SolveState* st, cudaStream_t stm
     int nb = nbig_of<T>(s);
     ensure_tile_maps(s);
     const int pr = PT<T>::prec;
-    int l0 = coarse_start<T, NR>(s);   // tiled levels [l0, nb) go into the cooperative launch
+    ClPlan cp;
+    int cthreads = 0;
+    size_t csmem = 0;
+    const int lc = cluster_plan<T, NR>(s, cp, cthreads, csmem);
+    // tiled levels [l0, nb) go into the cluster or the cooperative launch
+    const int l0 = lc < nb ? lc : coarse_start<T, NR>(s);
     for (int l = 0; l < l0; ++l) {
         Lev<T> L = lev<T>(s, l);
         dim3 grid((L.nx + TX - 1) / TX, (L.ny + TY - 1) / TY, s.nz);
@@ -3012,12 +3519,28 @@ static void vcycle(Solver& s, const T* r, T* z, SolveState* st, cudaStream_t stm
         k_pre<T, NR><<<grid, tile_block<HPRE>(), smem, stm>>>(L, b, X2 + 2 * s.loff[l], bc, st,
                                                               s.timing && l == 0 ? s.timer : nullptr,
                                                               s.tmaps[ix], tma,
-                                                              l == 0 && l0 < nb ? s.tickets + 8 : nullptr);
+                                                              l == 0 && l0 < nb && lc == nb ? s.tickets + 8 : nullptr);
         if (!s.use_graph) ++s.launches;
         b = bc;
     }
     SmallPlan P = small_plan<T>(s);
-    if (l0 < nb) {
+    if (lc < nb) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(CL_BLOCKS);
+        cfg.blockDim = dim3(cthreads);
+        cfg.dynamicSmemBytes = csmem;
+        cfg.stream = stm;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = CL_BLOCKS;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, k_coarse_cluster<T, NR>, cp, (const T*)PT<T>::diag(s), (const T*)id_of<T>(s),
+                           (const T*)PT<T>::wl(s), (const T*)PT<T>::wb(s), (const T*)PT<T>::inv(s), b,
+                           X + 2 * s.loff[l0], (const SolveState*)st);
+        if (!s.use_graph) ++s.launches;
+    } else if (l0 < nb) {
         CoarsePlan<T> C;
         C.l0 = l0;
         C.nb = nb;
