@@ -93,6 +93,7 @@ struct ebit_ctx {
     cudaStream_t stream = nullptr;
     cudaStream_t aux[3] = {nullptr, nullptr, nullptr};   // capture streams of the solvers' loop bodies
     cudaStream_t side = nullptr;   // capture branch of the second viscous solve
+    cudaEvent_t ev[2] = {nullptr, nullptr};              // fork and join of the solvers' captured branches
     // batched steps: instance b replays its step graph on workers[b % workers.size()], between a
     // fork event recorded on the context stream and the workers' join events
     std::vector<cudaStream_t> workers;
@@ -634,11 +635,13 @@ ebit_status ebit_init(const ebit_config* cfgs, int batch, void* stream, const eb
     }
     for (int k = 0; k < 3; ++k) cudaStreamCreateWithFlags(&ctx->aux[k], cudaStreamNonBlocking);
     cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking);
+    for (auto& e : ctx->ev) cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
     for (int b = 0; b < batch; ++b) {
         Instance& I = ctx->inst[b];
         I.solver.st_host = ctx->host_states + b * Solver::NSLOT;
         I.solver2.st_host = ctx->host_states + (batch + b) * Solver::NSLOT;
         for (int k = 0; k < 3; ++k) I.solver.aux[k] = I.solver2.aux[k] = ctx->aux[k];
+        for (int k = 0; k < 2; ++k) I.solver.ev[k] = I.solver2.ev[k] = ctx->ev[k];
         I.side = ctx->side;
     }
     ctx->launch0 = g_launches.load();
@@ -1285,6 +1288,8 @@ void ebit_destroy(ebit_ctx* ctx) {
     for (auto& s : ctx->aux)
         if (s) cudaStreamDestroy(s);
     if (ctx->side) cudaStreamDestroy(ctx->side);
+    for (auto& e : ctx->ev)
+        if (e) cudaEventDestroy(e);
     for (auto& I : ctx->inst) {
         if (I.e_fork) cudaEventDestroy(I.e_fork);
         if (I.e_join) cudaEventDestroy(I.e_join);

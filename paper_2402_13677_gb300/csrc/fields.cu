@@ -8,6 +8,7 @@
 //   S13  diagnostics (mass-in-domain and mass-with-outflow equations, vapour volume)
 // Cell-band compaction uses one warp ballot + popcount prefix per warp and one atomic per
 // warp; the resulting list order is irrelevant to every consumer (Jacobi updates).
+#include <atomic>
 #include "common.cuh"
 #include "kernels.h"
 
@@ -879,21 +880,41 @@ __global__ void k_project_cells(Grid g, Phys p, const double* __restrict__ axf, 
 // ---------------------------------------------------------------------------------
 // S13: diagnostics (block partial sums, last block finalises in a fixed order)
 // ---------------------------------------------------------------------------------
-__device__ inline double block_sum(double v, double* sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (w == 0) {
-        r = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+constexpr int NDIAG_SUMS = 8;
+
+// the block sums of NDIAG_SUMS per-thread values (in thread 0's v), the shuffle trees of all of
+// them side by side between two barriers.  A warp whose values of one sum are all zero adds
+// nothing (most cells are neither cut nor on a boundary: six of the eight sums): a tree level costs
+// about 100 cycles of FP64 latency.  The eight trees one after the other, twice, were 10 us.
+__device__ inline void diag_block_sums(double* v, double (*sh)[32]) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int pass = 0; pass < 2; ++pass) {
+        bool any[NDIAG_SUMS];
+#pragma unroll
+        for (int q = 0; q < NDIAG_SUMS; ++q)
+            any[q] = __any_sync(0xffffffffu, (__double_as_longlong(v[q]) << 1) != 0);
+#pragma unroll
+        for (int q = 0; q < NDIAG_SUMS; ++q)
+            if (any[q])
+                for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+        if (pass == 1) break;
+        if (lane == 0)
+#pragma unroll
+            for (int q = 0; q < NDIAG_SUMS; ++q) sh[q][w] = v[q];
+        __syncthreads();
+        if (w != 0) break;
+#pragma unroll
+        for (int q = 0; q < NDIAG_SUMS; ++q) v[q] = lane < nw ? sh[q][lane] : 0.0;
     }
     __syncthreads();
-    return r;   // valid in thread 0
 }
-
-constexpr int NDIAG_SUMS = 8;
+// arrival of a block whose slots thread 0 wrote: they are published, and the last block sees the
+// others'
+__device__ inline unsigned diag_arrive(unsigned* p) {
+    unsigned v;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 
 // S13 and the film-boiling quantities of Sec. 3.7, one reduction over the cells:
 //   s0 vapour area, s1 sum mdot S_Gamma, s2 sum rho_c, s3 outlet mass flux (mass-with-outflow
@@ -932,7 +953,7 @@ __global__ void k_diagnostics(Grid g, Phys p, const double* __restrict__ vf, con
     ticket = zsh(ticket, zo);
     clock = zsh(clock, zo);
     out = zsh(out, zo);
-    __shared__ double sh[32];
+    __shared__ double sh[NDIAG_SUMS][32];
     __shared__ bool lastblk;
     // virtual blocks: the reduction is that of a vb-block launch whatever the launch's size
     // (blocks take the virtual blocks b, b + gridDim.x, ...), as in the solver's reductions
@@ -988,22 +1009,19 @@ __global__ void k_diagnostics(Grid g, Phys p, const double* __restrict__ vf, con
                 }
             }
         }
-        for (int q = 0; q < NDIAG_SUMS; ++q) {
-            double r = block_sum(s[q], sh);
-            if (threadIdx.x == 0) partial[q * vb + vblk] = r;
-        }
+        diag_block_sums(s, sh);
+        if (threadIdx.x == 0)
+            for (int q = 0; q < NDIAG_SUMS; ++q) partial[q * vb + vblk] = s[q];
     }
-    __threadfence();
-    if (threadIdx.x == 0) lastblk = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) lastblk = diag_arrive(ticket) == gridDim.x - 1;   // thread 0 wrote the slots
     __syncthreads();
     if (!lastblk) return;
-    __threadfence();
     for (int q = 0; q < NDIAG_SUMS; ++q) {
         double v = 0.0;
-        for (int b = threadIdx.x; b < vb; b += blockDim.x) v += partial[q * vb + b];
-        double r = block_sum(v, sh);
-        if (threadIdx.x == 0) tot[q] = r;
+        for (int b = threadIdx.x; b < vb; b += blockDim.x) v += __ldcg(partial + q * vb + b);
+        tot[q] = v;
     }
+    diag_block_sums(tot, sh);
     if (threadIdx.x == 0) {
         double h2 = g.h * g.h;
         const double ring = AXI ? 6.283185307179586 * g.h : 1.0;   // 2 pi r = 2 pi h times the radius in cells
@@ -1091,11 +1109,122 @@ k_extend_block(Grid g, int mode, int iters, const int* __restrict__ list, const 
     }
 }
 
+// One instance alone: the sweeps in one cluster of blocks.  In one block they were bound by that
+// SM's FP64 pipe (17 FP64 instructions a sweep and band cell, the division 12 of them, at 19
+// cycles per warp) and by four dependent reads per sweep (list, flags, index, value): 30 us for
+// the 512^2 bubble's 1500 band cells.  Here the cells are spread over 16 SMs, a thread finds its
+// first cell's two neighbours, their fixed values and their places in the band once, and a sweep
+// reads two values, divides and stores; a cluster barrier ends it.  The arithmetic is
+// extend_entry's.  30 -> 10.8 us at 512^2, 12 -> 8.8 at 64^2.  Batched instances keep one block each
+// (they fill the device).
+constexpr int EXT_CLUSTER = 16, EXT_CLUSTER_THREADS = 256;
+__device__ __forceinline__ void ext_cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__global__ void __launch_bounds__(EXT_CLUSTER_THREADS)
+k_extend_cluster(Grid g, int mode, int iters, const int* __restrict__ list, const int* __restrict__ count,
+                 const uint8_t* __restrict__ flags, const int* __restrict__ idxmap, const double2* __restrict__ nb,
+                 double* f0, double* va0, double* vb0, double* f1, double* va1, double* vb1) {
+    const int n = *count, T = EXT_CLUSTER * EXT_CLUSTER_THREADS;   // the grid is one cluster
+    // warps of 32 entries dealt to the blocks in turn: a short band still spreads over every SM
+    const int k0 = ((threadIdx.x >> 5) * EXT_CLUSTER + blockIdx.x) * 32 + (threadIdx.x & 31);
+    // the thread's first band cell: what its sweeps read, gathered once
+    bool own = false;
+    int c = 0;
+    double* f = nullptr;
+    double *va = nullptr, *vb = nullptr, wx = 0.0, wy = 0.0, w = 0.0, fx = 0.0, fy = 0.0, self = 0.0;
+    int ix = -1, iy = -1;   // places in the band of the neighbours that are extended themselves
+    if (k0 < n) {
+        c = list[k0];
+        const uint8_t fl = flags[c];
+        const int m = mode == 3 ? ((fl & F_CCOL) ? 1 : 0) : mode;
+        own = ext_update(fl, m);
+        if (own) {
+            const bool second = m == 1 && mode == 3;
+            f = second ? f1 : f0;
+            va = second ? va1 : va0;
+            vb = second ? vb1 : vb0;
+            const int i = c % g.nx, j = c / g.nx;
+            const double sgn = m == 0 ? 1.0 : (m == 1 ? -1.0 : ((fl & F_CCOL) ? -1.0 : 1.0));
+            const double2 nn = nb[c];
+            const double ax = nn.x * sgn, ay = nn.y * sgn;
+            int cx = -1, cy = -1;
+            if (ax > 0.0 && i - 1 >= 0) { cx = c - 1; wx = ax; }
+            else if (ax < 0.0 && i + 1 < g.nx) { cx = c + 1; wx = -ax; }
+            if (ay > 0.0 && j - 1 >= 0) { cy = c - g.nx; wy = ay; }
+            else if (ay < 0.0 && j + 1 < g.ny) { cy = c + g.nx; wy = -ay; }
+            if (cx >= 0) {
+                if (ext_update(flags[cx], m)) ix = idxmap[cx];
+                fx = f[cx];
+                w += wx;
+            }
+            if (cy >= 0) {
+                if (ext_update(flags[cy], m)) iy = idxmap[cy];
+                fy = f[cy];
+                w += wy;
+            }
+            self = f[c];
+            if (cx < 0) wx = 0.0;
+            if (cy < 0) wy = 0.0;
+        }
+    }
+    for (int it = 0; it < iters; ++it) {
+        const bool odd = it & 1, last = it == iters - 1;
+        if (own) {
+            const double* cur = odd ? vb : va;
+            const double x = it > 0 && ix >= 0 ? __ldcg(cur + ix) : fx, y = it > 0 && iy >= 0 ? __ldcg(cur + iy) : fy;
+            double acc = 0.0;
+            if (wx > 0.0) acc += wx * x;
+            if (wy > 0.0) acc += wy * y;
+            if (w > 0.0) self = acc / w;   // else the value stays
+            if (last) f[c] = self;
+            else (odd ? va : vb)[k0] = self;
+        }
+        for (int k = k0 + T; k < n; k += T)   // bands of more cells than threads
+            extend_entry(g, mode, it, last, k, list, flags, idxmap, nb, f0, odd ? vb0 : va0, odd ? va0 : vb0, f1,
+                         odd ? vb1 : va1, odd ? va1 : vb1);
+        if (!last) ext_cluster_barrier();
+    }
+}
+
+// one launch of every sweep: a cluster for an instance alone where the device takes it, else one
+// block per instance
+static void launch_extend_once(const Grid& g, int mode, int iters, const int* list, const int* count,
+                               const uint8_t* flags, const int* idxmap, const double2* nb, double* f0, double* va0,
+                               double* vb0, double* f1, double* va1, double* vb1, cudaStream_t st) {
+    static std::atomic<int> usable[64];   // per device: 0 not asked, 1 yes, 2 no
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(EXT_CLUSTER);
+    cfg.blockDim = dim3(EXT_CLUSTER_THREADS);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = EXT_CLUSTER;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    bool cluster = g.nz == 1 && dev >= 0 && dev < 64;
+    if (cluster && usable[dev].load() == 0) {
+        int n = 0;
+        cudaError_t e = cudaFuncSetAttribute(k_extend_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_extend_cluster, &cfg);
+        usable[dev].store(e == cudaSuccess && n > 0 ? 1 : 2);
+        if (e != cudaSuccess) cudaGetLastError();
+    }
+    if (cluster && usable[dev].load() == 1)
+        cudaLaunchKernelEx(&cfg, k_extend_cluster, g, mode, iters, list, count, flags, idxmap, nb, f0, va0, vb0, f1,
+                           va1, vb1);
+    else
+        k_extend_block<<<dim3(1, 1, g.nz), EXT_BLOCK_THREADS, 0, st>>>(g, mode, iters, list, count, flags, idxmap, nb,
+                                                                      f0, va0, vb0, f1, va1, vb1);
+}
+
 void launch_extend(const Grid& g, int mode, int iters, const int* list, const int* count, const uint8_t* flags,
                    const int* idxmap, const double2* nb, double* f, double* va, double* vb, cudaStream_t st) {
     if (g.ext_block) {
-        k_extend_block<<<dim3(1, 1, g.nz), EXT_BLOCK_THREADS, 0, st>>>(g, mode, iters, list, count, flags, idxmap, nb,
-                                                                      f, va, vb, nullptr, nullptr, nullptr);
+        launch_extend_once(g, mode, iters, list, count, flags, idxmap, nb, f, va, vb, nullptr, nullptr, nullptr, st);
         return;
     }
     int nb_ = extend_grid_blocks(g);
@@ -1111,8 +1240,7 @@ void launch_extend_T(const Grid& g, int iters, const int* list, const int* count
                      const int* idxmap, const double2* nb, double* T_l, double* T_v, double* const ext[4],
                      cudaStream_t st) {
     if (g.ext_block) {
-        k_extend_block<<<dim3(1, 1, g.nz), EXT_BLOCK_THREADS, 0, st>>>(g, 3, iters, list, count, flags, idxmap, nb,
-                                                                      T_l, ext[0], ext[1], T_v, ext[2], ext[3]);
+        launch_extend_once(g, 3, iters, list, count, flags, idxmap, nb, T_l, ext[0], ext[1], T_v, ext[2], ext[3], st);
         return;
     }
     int nb_ = extend_grid_blocks(g);

@@ -80,7 +80,8 @@ struct Solver {
     SolveState* st_host;   // pinned mirror of all slots (set by the owner)
     SolveState* st = nullptr;   // slot of the current solve
     int slot = 0;
-    cudaStream_t aux[3] = {nullptr, nullptr, nullptr};   // capture streams of loop bodies
+    cudaStream_t aux[3] = {nullptr, nullptr, nullptr};   // capture streams: two of loop bodies, one of a branch
+    cudaEvent_t ev[2] = {nullptr, nullptr};              // fork and join of that branch (the owner's)
     KTimer* timer;     // device, [2]: tiled level-0 pre / post kernels
     int timing = 0;
     long long launches = 0;
