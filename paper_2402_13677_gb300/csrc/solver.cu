@@ -40,6 +40,7 @@
 #include <atomic>
 #include <vector>
 #include <cfloat>
+#include <type_traits>
 #include <cstdio>
 #include "common.cuh"
 #include "kernels.h"
@@ -971,33 +972,27 @@ struct SmallPlan {
 // before: FP32 11.8 -> 8.2 us (one right-hand side), 14.8 -> 10.1 (two), FP64 29 -> 25 and 45 -> 40;
 // with a coarsest level solved by 48 half-sweeps (336^2 grid, 21^2 cells) a step 1.78 -> 1.35 ms.
 
-// shared-memory layout: x (colour-split) and b, NR per cell, then diag, wl, wb, id per cell and
-// the transposed inverse of the coarsest operator
+// shared-memory layout: x (colour-split) and b, NR per cell, then diag, wl, (FP64) the reciprocals of
+// the full diagonals, wb per cell and the transposed inverse of the coarsest operator
 template <typename T, int NR>
 struct SmallMem {
     Vec<T, NR>*x, *b;
-    T *d, *wl, *wb, *id, *inv;   // id: reciprocal of the full diagonal D + the four face weights
+    T *d, *wl, *wb, *id, *inv;
     __device__ SmallMem(unsigned char* base, const SmallPlan& P) {
         x = (Vec<T, NR>*)base;
         b = x + P.xtotal;
         d = (T*)(b + P.total);
         wl = d + P.total;
-        wb = wl + P.total;
-        id = wb + P.total;
-        inv = id + P.total;
+        id = wl + P.total;
+        wb = id + (sizeof(T) == 8 ? P.total : 0);
+        inv = wb + P.total;
     }
     static size_t bytes(int total, int xtotal) {
-        return ((size_t)total * (NR + 4) + (size_t)xtotal * NR + SMALL_INV) * sizeof(T);
+        return ((size_t)total * (NR + 3 + (sizeof(T) == 8 ? 1 : 0)) + (size_t)xtotal * NR + SMALL_INV) * sizeof(T);
     }
     static size_t bytes(const SmallPlan& P) { return bytes(P.total, P.xtotal); }
 };
 
-// the team of a level: the first `threads` threads of the block (a multiple of 32)
-__device__ inline int small_team(int nx, int ny) {
-    int n = ((nx + 1) >> 1) * ((ny + 1) >> 1);
-    const int cap = blockDim.x;
-    return n >= cap ? cap : (n + 31) & ~31;
-}
 __device__ inline void team_sync(int l, int threads) {
     if (threads <= 32) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(l + 1), "r"(threads) : "memory");
@@ -1012,225 +1007,405 @@ __device__ __forceinline__ int xidx(int hx, int I, int j) { return 1 + (j + 1) *
 // t / n for 0 <= t < 2^13 (the quotient of t + 1/2 is at least 1 / (2 n) from an integer)
 __device__ __forceinline__ int small_div(int t, int n) { return (int)__fdividef((float)t + 0.5f, (float)n); }
 
-// a thread's 2 x 2 block: [r][e] = row 2J + r, column 2I + e (colour e ^ r); wl[r][0..2] the
-// weights of the row's three vertical faces, wb[0..2][e] of the column's three horizontal ones
-// (zero where there is no neighbour).  Cells beyond an odd side (coarsest level only) have
-// b = x = 0 and zero weights.
-template <typename T, int NR>
-struct SmallBlk {
-    Vec<T, NR> b[2][2], x[2][2];
-    T id[2][2], wl[2][3], wb[3][2];
-    int q;        // x entry of the block's first row: row r of either colour at q + r hx
-    bool own;     // the thread owns a block
-};
-// the block's place: I, J of thread t on a level of hx x hy blocks
-template <typename T, int NR>
-__device__ __forceinline__ void small_place(SmallBlk<T, NR>& B, int hx, int hy, int t, int& I, int& J) {
-    J = small_div(t, hx);
-    I = t - J * hx;
-    B.own = J < hy;
-    B.q = xidx(hx, I, 2 * J);
-}
-
-// the block's weights, reciprocal diagonals and right-hand side from shared memory; DOWN: also D,
-// and in FP32 the reciprocal diagonals are computed here and kept in shared memory for the up leg
-// (read back by the same thread).  ODD: the level may have odd sides.
-template <typename T, int NR, bool DOWN, bool ODD>
-__device__ inline void small_load(SmallBlk<T, NR>& B, T (&d)[2][2], const SmallPlan& P, int l, SmallMem<T, NR>& M,
-                                  int I, int J) {
-    const int nx = P.nx[l], ny = P.ny[l], c0 = P.soff[l] + 2 * J * nx + 2 * I;   // cell (0, 0) of the block
-    const bool right = 2 * I + 2 < nx, up = 2 * J + 2 < ny;
-    using P2 = Vec<T, 2>;
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int c = c0 + r * nx;
-        if constexpr (ODD) {
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const bool in = 2 * I + e < nx && 2 * J + r < ny;
-                const int ce = in ? c + e : P.soff[l];
-                B.wl[r][e] = in ? M.wl[ce] : T(0);
-                B.wb[r][e] = in ? M.wb[ce] : T(0);
-                if (DOWN) d[r][e] = in ? M.d[ce] : T(1);
-                if (!DOWN || sizeof(T) == 8) B.id[r][e] = in ? M.id[ce] : T(1);
-                const Vec<T, NR> bv = M.b[ce];
-#pragma unroll
-                for (int k = 0; k < NR; ++k) B.b[r][e].v[k] = in ? bv.v[k] : T(0);
-            }
-            B.wl[r][2] = right && 2 * J + r < ny ? M.wl[c + 2] : T(0);
-        } else {
-            const P2 w = *reinterpret_cast<const P2*>(M.wl + c), v = *reinterpret_cast<const P2*>(M.wb + c);
-            const Vec<T, 2 * NR> bv = *reinterpret_cast<const Vec<T, 2 * NR>*>(M.b + c);
-            const T wr = M.wl[c + 2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                B.wl[r][e] = w.v[e];
-                B.wb[r][e] = v.v[e];
-#pragma unroll
-                for (int k = 0; k < NR; ++k) B.b[r][e].v[k] = bv.v[e * NR + k];
-            }
-            B.wl[r][2] = right ? wr : T(0);
-            if (DOWN) {
-                const P2 dv = *reinterpret_cast<const P2*>(M.d + c);
-                d[r][0] = dv.v[0];
-                d[r][1] = dv.v[1];
-            }
-            if (!DOWN || sizeof(T) == 8) {
-                const P2 iv = *reinterpret_cast<const P2*>(M.id + c);
-                B.id[r][0] = iv.v[0];
-                B.id[r][1] = iv.v[1];
-            }
-        }
-    }
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        if constexpr (ODD) {
-            B.wb[2][e] = up && 2 * I + e < nx ? M.wb[c0 + 2 * nx + e] : T(0);
-        } else {
-            const T wt = M.wb[c0 + 2 * nx + e];
-            B.wb[2][e] = up ? wt : T(0);
-        }
-    }
-    if (DOWN && sizeof(T) == 4) {
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                B.id[r][e] = rcp_diag(d[r][e] + B.wl[r][e] + B.wl[r][e + 1] + B.wb[r][e] + B.wb[r + 1][e]);
-                if (ODD && 2 * I + e < nx && 2 * J + r < ny) M.id[c0 + r * nx + e] = B.id[r][e];
-            }
-            if constexpr (!ODD) {
-                P2 iv;
-                iv.v[0] = B.id[r][0];
-                iv.v[1] = B.id[r][1];
-                *reinterpret_cast<P2*>(M.id + c0 + r * nx) = iv;
-            }
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) B.wl[r][0] = I > 0 ? B.wl[r][0] : T(0);
-#pragma unroll
-    for (int e = 0; e < 2; ++e) B.wb[0][e] = J > 0 ? B.wb[0][e] : T(0);
-}
-
-// (b + sum of w x_n) / diagonal of cell (r, e), its outer neighbours' values h (horizontal) and v
-// (vertical) given, the other two the thread's own cells
-template <typename T, int NR>
-__device__ __forceinline__ Vec<T, NR> small_update(const SmallBlk<T, NR>& B, int r, int e, const Vec<T, NR>& h,
-                                                   const Vec<T, NR>& v) {
-    Vec<T, NR> a;
-#pragma unroll
-    for (int k = 0; k < NR; ++k) {
-        const T xl = e == 1 ? B.x[r][0].v[k] : h.v[k], xr = e == 0 ? B.x[r][1].v[k] : h.v[k];
-        const T xd = r == 1 ? B.x[0][e].v[k] : v.v[k], xu = r == 0 ? B.x[1][e].v[k] : v.v[k];
-        a.v[k] = (B.b[r][e].v[k] + B.wl[r][e] * xl + B.wl[r][e + 1] * xr + B.wb[r][e] * xd + B.wb[r + 1][e] * xu) *
-                 B.id[r][e];
-    }
-    return a;
-}
-// the outer neighbours of the block's two cells of colour COLOR, (0, COLOR) and (1, 1 - COLOR)
-template <typename T, int NR, int COLOR>
-__device__ __forceinline__ void small_outer(const SmallBlk<T, NR>& B, const Vec<T, NR>* xo, int hx, Vec<T, NR>& h0,
-                                            Vec<T, NR>& v0, Vec<T, NR>& h1, Vec<T, NR>& v1) {
-    h0 = xo[B.q + (COLOR ? 1 : -1)];
-    v0 = xo[B.q - hx];
-    h1 = xo[B.q + hx + (COLOR ? -1 : 1)];
-    v1 = xo[B.q + 2 * hx];
-}
-
-// one red-black half-sweep of colour COLOR over the K blocks of a thread (x: nxc entries per colour)
-template <typename T, int NR, int K, int COLOR>
-__device__ inline void small_sweep(SmallBlk<T, NR> (&B)[K], Vec<T, NR>* x, int nxc, int hx, int l, int team) {
-    const Vec<T, NR>* xo = x + (1 - COLOR) * nxc;
-    Vec<T, NR>* xs = x + COLOR * nxc;
-#pragma unroll
-    for (int u = 0; u < K; ++u)
-        if (B[u].own) {
-            Vec<T, NR> h0, v0, h1, v1;
-            small_outer<T, NR, COLOR>(B[u], xo, hx, h0, v0, h1, v1);
-            const Vec<T, NR> a0 = small_update(B[u], 0, COLOR, h0, v0), a1 = small_update(B[u], 1, 1 - COLOR, h1, v1);
-            B[u].x[0][COLOR] = a0;
-            B[u].x[1][1 - COLOR] = a1;
-            xs[B[u].q] = a0;
-            xs[B[u].q + hx] = a1;
-        }
-    team_sync(l, team);
-}
-
 // residual of a cell of column parity e on the single-block levels: the flux form with the
-// rounding of its first sum fixed (one right-hand side fuses D x in the cells whose left
-// neighbour is in their block, two fuse the first flux)
+// rounding of its first sum fixed (one right-hand side fuses D x in the cells of odd columns, two
+// fuse the first flux).  The operands are selected, not the results: one FP64 instruction.
 template <typename T, int NR>
 __device__ __forceinline__ T small_residual(int e, T b, T d, T w0, T w1, T w2, T w3, T x, T xl, T xr, T xd, T xu) {
-    T ax;
-    if (NR == 1 && e == 1) ax = fma_rn(d, x, w0 * (x - xl));
-    else ax = fma_rn(w0, x - xl, d * x);
+    const bool dx = NR == 1 && e == 1;
+    const T f = x - xl;
+    T ax = fma_rn(dx ? d : w0, dx ? x : f, (dx ? w0 : d) * (dx ? f : x));
     ax = fma_rn(w1, x - xr, ax);
     ax = fma_rn(w2, x - xd, ax);
     ax = fma_rn(w3, x - xu, ax);
     return b - ax;
 }
-// sum of the residuals of the block's four cells; TILE: in the form of the tile kernels
-template <typename T, int NR, bool TILE>
-__device__ __forceinline__ Vec<T, NR> small_restrict(const SmallBlk<T, NR>& B, const T (&d)[2][2], const Vec<T, NR>* x,
-                                                     int nxc, int hx) {
-    Vec<T, NR> h[2][2], v[2][2], acc;   // outer neighbours of cell (r, e)
-    small_outer<T, NR, 0>(B, x + nxc, hx, h[0][0], v[0][0], h[1][1], v[1][1]);
-    small_outer<T, NR, 1>(B, x, hx, h[0][1], v[0][1], h[1][0], v[1][0]);
+
+// What a block reads of a level: nx columns, rows [0, ny) of it in these arrays (row pitch nx, and
+// one row more of wb), cell weights as in Lev
+template <typename T, int NR>
+struct BlkSrc {
+    int nx, ny;
+    const T *d, *wl, *wb, *id;
+    const Vec<T, NR>* b;
+};
+// which neighbours exist (weights of the others are 0)
+struct BlkSides {
+    bool left, right, down, up;
+};
+
+// A thread's cells in FP32: the 2 x 2 block of columns 2I, 2I + 1 and rows j, j + 1 (j even), the four
+// children of one coarser cell.  [r][e]: row j + r, column 2I + e, colour e ^ r; wl[r][0..2] the weights of
+// the row's three vertical faces, wb[0..2][e] of the column's three horizontal ones.  Cells beyond
+// an odd side (ODD levels) have b = x = 0 and zero weights.
+template <typename T, int NR>
+struct QuadBlk {
+    using V = Vec<T, NR>;
+    static constexpr int RB = 2;                       // rows of a block
+    V b[2][2], x[2][2];
+    T id[2][2], d[2][2], wl[2][3], wb[3][2];
+    int q;        // x entry of the first row: row r of either colour at q + r hx
+    bool own;     // the thread owns a block
+    __host__ __device__ static int units(int nx, int ny) { return ((nx + 1) >> 1) * ((ny + 1) >> 1); }
+    __device__ void place(int hx, int rows, int t, int& I, int& j) {
+        j = small_div(t, hx);
+        I = t - j * hx;
+        j *= 2;
+        own = j < rows;
+        q = xidx(hx, I, j);
+    }
+    template <bool ODD>
+    __device__ void load(const BlkSrc<T, NR>& S, int I, int j, const BlkSides& n) {
+        const int c0 = j * S.nx + 2 * I;
+        using P2 = Vec<T, 2>;
 #pragma unroll
-    for (int k = 0; k < NR; ++k) {
-        T res[2][2];
+        for (int r = 0; r < 2; ++r) {
+            const int c = c0 + r * S.nx;
+            if constexpr (ODD) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const bool in = 2 * I + e < S.nx && j + r < S.ny;
+                    const int ce = in ? c + e : 0;
+                    wl[r][e] = in ? S.wl[ce] : T(0);
+                    wb[r][e] = in ? S.wb[ce] : T(0);
+                    d[r][e] = in ? S.d[ce] : T(1);
+                    const V bv = S.b[ce];
+#pragma unroll
+                    for (int k = 0; k < NR; ++k) b[r][e].v[k] = in ? bv.v[k] : T(0);
+                }
+                wl[r][2] = n.right && j + r < S.ny ? S.wl[c + 2] : T(0);
+            } else {
+                const P2 w = *reinterpret_cast<const P2*>(S.wl + c), v = *reinterpret_cast<const P2*>(S.wb + c);
+                const P2 dv = *reinterpret_cast<const P2*>(S.d + c);
+                const Vec<T, 2 * NR> bv = *reinterpret_cast<const Vec<T, 2 * NR>*>(S.b + c);
+                const T wr = S.wl[c + 2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    wl[r][e] = w.v[e];
+                    wb[r][e] = v.v[e];
+                    d[r][e] = dv.v[e];
+#pragma unroll
+                    for (int k = 0; k < NR; ++k) b[r][e].v[k] = bv.v[e * NR + k];
+                }
+                wl[r][2] = n.right ? wr : T(0);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            if constexpr (ODD) {
+                wb[2][e] = n.up && 2 * I + e < S.nx ? S.wb[c0 + 2 * S.nx + e] : T(0);
+            } else {
+                const T wt = S.wb[c0 + 2 * S.nx + e];
+                wb[2][e] = n.up ? wt : T(0);
+            }
+        }
 #pragma unroll
         for (int r = 0; r < 2; ++r)
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const T xl = e == 1 ? B.x[r][0].v[k] : h[r][e].v[k], xr = e == 0 ? B.x[r][1].v[k] : h[r][e].v[k];
-                const T xd = r == 1 ? B.x[0][e].v[k] : v[r][e].v[k], xu = r == 0 ? B.x[1][e].v[k] : v[r][e].v[k];
-                if constexpr (TILE)
-                    res[r][e] = cell_residual(B.b[r][e].v[k], d[r][e], B.wl[r][e], B.wl[r][e + 1], B.wb[r][e],
-                                              B.wb[r + 1][e], B.x[r][e].v[k], xl, xr, xd, xu);
-                else
-                    res[r][e] = small_residual<T, NR>(e, B.b[r][e].v[k], d[r][e], B.wl[r][e], B.wl[r][e + 1],
-                                                      B.wb[r][e], B.wb[r + 1][e], B.x[r][e].v[k], xl, xr, xd, xu);
-            }
-        acc.v[k] = res[0][0] + res[0][1] + res[1][0] + res[1][1];
+            for (int e = 0; e < 2; ++e)
+                id[r][e] = rcp_diag(d[r][e] + wl[r][e] + wl[r][e + 1] + wb[r][e] + wb[r + 1][e]);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) wl[r][0] = n.left ? wl[r][0] : T(0);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) wb[0][e] = n.down ? wb[0][e] : T(0);
     }
-    return acc;
+    // the first colour-0 half-sweep from x = 0 reduces to x = b / (full diagonal)
+    __device__ void first() {
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int k = 0; k < NR; ++k) {
+                x[r][r].v[k] = b[r][r].v[k] * id[r][r];
+                x[r][1 - r].v[k] = T(0);
+            }
+    }
+    __device__ void zero() {
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int k = 0; k < NR; ++k) x[r][e].v[k] = T(0);
+    }
+    template <int COLOR>
+    __device__ void put(V* xs, int hx) const {   // xs: the colour's array
+        xs[q] = x[0][COLOR];
+        xs[q + hx] = x[1][1 - COLOR];
+    }
+    template <int COLOR>
+    __device__ void fetch(const V* xs, int hx) {
+        x[0][COLOR] = xs[q];
+        x[1][1 - COLOR] = xs[q + hx];
+    }
+    __device__ void add(const V& c) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int k = 0; k < NR; ++k) x[r][e].v[k] += c.v[k];
+    }
+    template <int COLOR>
+    __device__ const V& low() const { return x[0][COLOR]; }        // the colour's cell of the first row
+    template <int COLOR>
+    __device__ const V& high() const { return x[1][1 - COLOR]; }   // of the last row
+    // the outer neighbours of the block's two cells of colour COLOR, (0, COLOR) and (1, 1 - COLOR)
+    template <int COLOR>
+    __device__ void outer(const V* xo, int hx, V& h0, V& v0, V& h1, V& v1) const {
+        h0 = xo[q + (COLOR ? 1 : -1)];
+        v0 = xo[q - hx];
+        h1 = xo[q + hx + (COLOR ? -1 : 1)];
+        v1 = xo[q + 2 * hx];
+    }
+    // (b + sum of w x_n) / diagonal of cell (r, e) with the outer neighbours h and v
+    __device__ V update(int r, int e, const V& h, const V& v) const {
+        V a;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            const T xl = e == 1 ? x[r][0].v[k] : h.v[k], xr = e == 0 ? x[r][1].v[k] : h.v[k];
+            const T xd = r == 1 ? x[0][e].v[k] : v.v[k], xu = r == 0 ? x[1][e].v[k] : v.v[k];
+            a.v[k] = (b[r][e].v[k] + wl[r][e] * xl + wl[r][e + 1] * xr + wb[r][e] * xd + wb[r + 1][e] * xu) * id[r][e];
+        }
+        return a;
+    }
+    template <int COLOR>
+    __device__ void sweep(const V* xo, int hx) {   // xo: the other colour's array
+        V h0, v0, h1, v1;
+        outer<COLOR>(xo, hx, h0, v0, h1, v1);
+        const V a0 = update(0, COLOR, h0, v0), a1 = update(1, 1 - COLOR, h1, v1);
+        x[0][COLOR] = a0;
+        x[1][1 - COLOR] = a1;
+    }
+    // the four cells' residuals summed; TILE: in the form of the tile kernels
+    template <bool TILE>
+    __device__ V residual(const V* xs, int nxc, int hx) const {
+        V h[2][2], v[2][2], acc;   // outer neighbours of cell (r, e)
+        outer<0>(xs + nxc, hx, h[0][0], v[0][0], h[1][1], v[1][1]);
+        outer<1>(xs, hx, h[0][1], v[0][1], h[1][0], v[1][0]);
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            T res[2][2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const T xl = e == 1 ? x[r][0].v[k] : h[r][e].v[k], xr = e == 0 ? x[r][1].v[k] : h[r][e].v[k];
+                    const T xd = r == 1 ? x[0][e].v[k] : v[r][e].v[k], xu = r == 0 ? x[1][e].v[k] : v[r][e].v[k];
+                    if constexpr (TILE)
+                        res[r][e] = cell_residual(b[r][e].v[k], d[r][e], wl[r][e], wl[r][e + 1], wb[r][e], wb[r + 1][e],
+                                                  x[r][e].v[k], xl, xr, xd, xu);
+                    else
+                        res[r][e] = small_residual<T, NR>(e, b[r][e].v[k], d[r][e], wl[r][e], wl[r][e + 1], wb[r][e],
+                                                          wb[r + 1][e], x[r][e].v[k], xl, xr, xd, xu);
+                }
+            acc.v[k] = res[0][0] + res[0][1] + res[1][0] + res[1][1];
+        }
+        return acc;
+    }
+};
+
+// A thread's cells in FP64: two neighbours of a row, columns 2I, 2I + 1 of row j, one of each colour
+// (arrays by colour).  A dependent FP64 operation takes 64 cycles whatever the lanes do, and a
+// scheduler's FP64 unit one warp instruction in that time: with one cell of a colour per thread a
+// half-sweep is one chain of six operations instead of two behind each other, and the level
+// spreads over twice the warps.  The restriction meets through shared memory.
+template <typename T, int NR>
+struct PairBlk {
+    using V = Vec<T, NR>;
+    static constexpr int RB = 1;
+    V b[2], x[2];
+    T id[2], d[2], wl[2], wr[2], wb[2], wt[2];
+    int q;
+    int par;      // j & 1: the cell of colour c is column 2I + (c ^ par)
+    bool own;
+    __host__ __device__ static int units(int nx, int ny) { return ((nx + 1) >> 1) * ny; }
+    __device__ void place(int hx, int rows, int t, int& I, int& j) {
+        j = small_div(t, hx);
+        I = t - j * hx;
+        own = j < rows;
+        q = xidx(hx, I, j);
+        par = j & 1;
+    }
+    template <bool ODD>
+    __device__ void load(const BlkSrc<T, NR>& S, int I, int j, const BlkSides& n) {
+        const int c = j * S.nx + 2 * I;
+        const bool two = !ODD || 2 * I + 1 < S.nx;   // the second cell exists
+        const T w0 = S.wl[c], w1 = two ? S.wl[c + 1] : T(0), w2 = n.right ? S.wl[c + 2] : T(0);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {                // colour k
+            const int e = k ^ par;
+            const bool in = e == 0 || two;
+            const int ce = in ? c + e : c;
+            wl[k] = e ? w1 : (n.left ? w0 : T(0));
+            wr[k] = e ? w2 : w1;
+            wb[k] = in && n.down ? S.wb[ce] : T(0);
+            wt[k] = in && n.up ? S.wb[ce + S.nx] : T(0);
+            d[k] = in ? S.d[ce] : T(1);
+            id[k] = in ? S.id[ce] : T(1);
+            const V bv = S.b[ce];
+#pragma unroll
+            for (int r = 0; r < NR; ++r) b[k].v[r] = in ? bv.v[r] : T(0);
+        }
+    }
+    __device__ void first() {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            x[0].v[k] = b[0].v[k] * id[0];
+            x[1].v[k] = T(0);
+        }
+    }
+    __device__ void zero() {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) x[0].v[k] = x[1].v[k] = T(0);
+    }
+    template <int COLOR>
+    __device__ void put(V* xs, int hx) const { xs[q] = x[COLOR]; }
+    template <int COLOR>
+    __device__ void fetch(const V* xs, int hx) { x[COLOR] = xs[q]; }
+    __device__ void add(const V& c) {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            x[0].v[k] += c.v[k];
+            x[1].v[k] += c.v[k];
+        }
+    }
+    template <int COLOR>
+    __device__ const V& low() const { return x[COLOR]; }
+    template <int COLOR>
+    __device__ const V& high() const { return x[COLOR]; }
+    template <int COLOR>
+    __device__ void sweep(const V* xo, int hx) {
+        const bool e = (COLOR ^ par) != 0;
+        const V h = xo[q + (e ? 1 : -1)], vd = xo[q - hx], vu = xo[q + hx];
+        V a;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            const T o = x[1 - COLOR].v[k], xl = e ? o : h.v[k], xr = e ? h.v[k] : o;
+            a.v[k] = (b[COLOR].v[k] + wl[COLOR] * xl + wr[COLOR] * xr + wb[COLOR] * vd.v[k] + wt[COLOR] * vu.v[k]) *
+                     id[COLOR];
+        }
+        x[COLOR] = a;
+    }
+    // the residuals of the cells in columns 2I and 2I + 1
+    template <bool TILE>
+    __device__ void residual(const V* xs, int nxc, int hx, V& r0, V& r1) const {
+        V r[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const V* xo = xs + (1 - c) * nxc;
+            const bool e = (c ^ par) != 0;
+            const V h = xo[q + (e ? 1 : -1)], vd = xo[q - hx], vu = xo[q + hx];
+#pragma unroll
+            for (int k = 0; k < NR; ++k) {
+                const T o = x[1 - c].v[k], xl = e ? o : h.v[k], xr = e ? h.v[k] : o;
+                if constexpr (TILE)
+                    r[c].v[k] = cell_residual(b[c].v[k], d[c], wl[c], wr[c], wb[c], wt[c], x[c].v[k], xl, xr, vd.v[k],
+                                              vu.v[k]);
+                else
+                    r[c].v[k] = small_residual<T, NR>(e, b[c].v[k], d[c], wl[c], wr[c], wb[c], wt[c], x[c].v[k], xl, xr,
+                                                      vd.v[k], vu.v[k]);
+            }
+        }
+        r0 = par ? r[1] : r[0];
+        r1 = par ? r[0] : r[1];
+    }
+};
+template <typename T, int NR>
+using Blk = std::conditional_t<sizeof(T) == 8, PairBlk<T, NR>, QuadBlk<T, NR>>;
+
+// the restricted residual of K blocks per thread: put(u, value) for each complete coarse cell; s: an
+// entry per coarse cell of the team's rows (one of s's barriers between the two rows of a cell
+// in FP64), slot(u) the block's
+template <typename T, int NR, int K, bool TILE, class Put, class Sync>
+__device__ inline void blk_restrict(const Blk<T, NR> (&B)[K], const int (&slot)[K], Vec<T, NR>* s, const Vec<T, NR>* x,
+                                    int nxc, int hx, Put&& put, Sync&& sync) {
+    if constexpr (Blk<T, NR>::RB == 2) {
+#pragma unroll
+        for (int u = 0; u < K; ++u)
+            if (B[u].own) put(u, B[u].template residual<TILE>(x, nxc, hx));
+    } else {
+        Vec<T, NR> r0[K], r1[K];
+#pragma unroll
+        for (int u = 0; u < K; ++u)
+            if (B[u].own) {
+                B[u].template residual<TILE>(x, nxc, hx, r0[u], r1[u]);
+                if (!B[u].par) {
+                    Vec<T, NR> a;
+#pragma unroll
+                    for (int k = 0; k < NR; ++k) a.v[k] = r0[u].v[k] + r1[u].v[k];
+                    s[slot[u]] = a;
+                }
+            }
+        sync();
+#pragma unroll
+        for (int u = 0; u < K; ++u)
+            if (B[u].own && B[u].par) {
+                Vec<T, NR> a = s[slot[u]];
+#pragma unroll
+                for (int k = 0; k < NR; ++k) a.v[k] = a.v[k] + r0[u].v[k] + r1[u].v[k];
+                put(u, a);
+            }
+    }
 }
 
-// down leg of level l from x = 0 (its first colour-0 half-sweep reads only zeros and reduces to
-// x = b / (full diagonal)), then the residual restricted to level l + 1
+// the team of a level: the first `threads` threads of the block (a multiple of 32)
+template <typename T>
+__device__ inline int small_team(int nx, int ny) {
+    const int n = Blk<T, 1>::units(nx, ny), cap = blockDim.x;
+    return n >= cap ? cap : (n + 31) & ~31;
+}
+
+// the blocks of a thread on single-block level l
+template <typename T, int NR, int K, bool ODD>
+__device__ inline void small_blocks(Blk<T, NR> (&B)[K], int (&I)[K], int (&j)[K], const SmallPlan& P, int l,
+                                    const SmallMem<T, NR>& M, int team) {
+    const int o = P.soff[l], nx = P.nx[l], ny = P.ny[l], hx = (nx + 1) >> 1;
+    const BlkSrc<T, NR> S = {nx, ny, M.d + o, M.wl + o, M.wb + o, M.id + o, M.b + o};
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        B[u].place(hx, ny, threadIdx.x + u * team, I[u], j[u]);
+        if (B[u].own)
+            B[u].template load<ODD>(S, I[u], j[u],
+                                    {I[u] > 0, 2 * I[u] + 2 < nx, j[u] > 0, j[u] + Blk<T, NR>::RB < ny});
+    }
+}
+// one red-black half-sweep of colour COLOR over the K blocks of a thread (x: nxc entries per colour)
+template <typename T, int NR, int K, int COLOR>
+__device__ inline void small_sweep(Blk<T, NR> (&B)[K], Vec<T, NR>* x, int nxc, int hx, int l, int team) {
+#pragma unroll
+    for (int u = 0; u < K; ++u)
+        if (B[u].own) {
+            B[u].template sweep<COLOR>(x + (1 - COLOR) * nxc, hx);
+            B[u].template put<COLOR>(x + COLOR * nxc, hx);
+        }
+    team_sync(l, team);
+}
+
+// down leg of level l from x = 0, then the residual restricted to level l + 1
 template <typename T, int NR, int K>
 __device__ inline void small_down(const SmallPlan& P, int l, SmallMem<T, NR>& M, int team) {
     static_assert(NU_SMALL == 2, "the sweep sequences below are written out for two pairs");
-    const int hx = P.nx[l] >> 1, hy = P.ny[l] >> 1, nxc = x_entries(hx, 2 * hy);
+    const int hx = P.nx[l] >> 1, nxc = x_entries(hx, P.ny[l]);
     Vec<T, NR>* x = M.x + P.xoff[l];
-    SmallBlk<T, NR> B[K];
-    T d[K][2][2];
+    Blk<T, NR> B[K];
+    int I[K], j[K];
+    small_blocks<T, NR, K, false>(B, I, j, P, l, M, team);
 #pragma unroll
-    for (int u = 0; u < K; ++u) {
-        int I, J;
-        small_place(B[u], hx, hy, threadIdx.x + u * team, I, J);
-        if (!B[u].own) continue;
-        small_load<T, NR, true, false>(B[u], d[u], P, l, M, I, J);
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-#pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                B[u].x[r][r].v[k] = B[u].b[r][r].v[k] * B[u].id[r][r];
-                B[u].x[r][1 - r].v[k] = T(0);
-            }
-            x[B[u].q + r * hx] = B[u].x[r][r];
+    for (int u = 0; u < K; ++u)
+        if (B[u].own) {
+            B[u].first();
+            B[u].template put<0>(x, hx);
         }
-    }
     team_sync(l, team);
     small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
     small_sweep<T, NR, K, 0>(B, x, nxc, hx, l, team);
     small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
+    Vec<T, NR>* bc = M.b + P.soff[l + 1];
+    int slot[K];
 #pragma unroll
-    for (int u = 0; u < K; ++u)   // block t is the four children of cell t of level l + 1
-        if (B[u].own)
-            M.b[P.soff[l + 1] + threadIdx.x + u * team] = small_restrict<T, NR, false>(B[u], d[u], x, nxc, hx);
+    for (int u = 0; u < K; ++u) slot[u] = (j[u] >> 1) * hx + I[u];
+    blk_restrict<T, NR, K, false>(
+        B, slot, bc, x, nxc, hx, [&](int u, const Vec<T, NR>& v) { bc[slot[u]] = v; }, [&]() { team_sync(l, team); });
     team_sync(l, team);
 }
 
@@ -1239,9 +1414,9 @@ __device__ inline void small_down(const SmallPlan& P, int l, SmallMem<T, NR>& M,
 template <typename T, int NR>
 __device__ inline void small_coarsest(const SmallPlan& P, SmallMem<T, NR>& M, bool exact) {
     const int l = P.n - 1, o = P.soff[l], nx = P.nx[l], ny = P.ny[l], n = nx * ny;
-    const int hx = (nx + 1) >> 1, hy = (ny + 1) >> 1, nxc = x_entries(hx, 2 * hy);
+    const int hx = (nx + 1) >> 1, nxc = x_entries(hx, (ny + 1) & ~1);
     Vec<T, NR>* x = M.x + P.xoff[l];
-    const int team = exact ? 32 : small_team(nx, ny);
+    const int team = exact ? 32 : small_team<T>(nx, ny);
     if (threadIdx.x >= team) return;
     if (exact) {
         const int r = threadIdx.x;
@@ -1261,29 +1436,26 @@ __device__ inline void small_coarsest(const SmallPlan& P, SmallMem<T, NR>& M, bo
         }
         return;
     }
-    SmallBlk<T, NR> B[1];
-    T d[2][2];
-    int I, J;
-    small_place(B[0], hx, hy, threadIdx.x, I, J);
-    if (B[0].own) {
-        small_load<T, NR, true, true>(B[0], d, P, l, M, I, J);
+    // (x is zero from the start in a single cycle, not in the later ones of a kernel that runs several)
+    constexpr int K = sizeof(T) == 8 ? 2 : 1;   // up to 1024 cells, in pairs one or two per thread
+    Blk<T, NR> B[K];
+    int I[K], j[K];
+    small_blocks<T, NR, K, true>(B, I, j, P, l, M, team);
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-#pragma unroll
-                for (int k = 0; k < NR; ++k) B[0].x[r][e].v[k] = T(0);
-                x[(e ^ r) * nxc + B[0].q + r * hx] = B[0].x[r][e];
-            }
-    }
+    for (int u = 0; u < K; ++u)
+        if (B[u].own) {
+            B[u].zero();
+            B[u].template put<0>(x, hx);
+            B[u].template put<1>(x + nxc, hx);
+        }
     team_sync(l, team);
     for (int k = 0; k < COARSE_PAIRS; ++k) {
-        small_sweep<T, NR, 1, 0>(B, x, nxc, hx, l, team);
-        small_sweep<T, NR, 1, 1>(B, x, nxc, hx, l, team);
+        small_sweep<T, NR, K, 0>(B, x, nxc, hx, l, team);
+        small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
     }
     for (int k = 0; k < COARSE_PAIRS; ++k) {
-        small_sweep<T, NR, 1, 1>(B, x, nxc, hx, l, team);
-        small_sweep<T, NR, 1, 0>(B, x, nxc, hx, l, team);
+        small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
+        small_sweep<T, NR, K, 0>(B, x, nxc, hx, l, team);
     }
 }
 
@@ -1291,39 +1463,27 @@ __device__ inline void small_coarsest(const SmallPlan& P, SmallMem<T, NR>& M, bo
 // joins the level's team with the warps that worked on the coarser levels.
 template <typename T, int NR, int K>
 __device__ inline void small_up(const SmallPlan& P, int l, SmallMem<T, NR>& M, int team) {
-    const int hx = P.nx[l] >> 1, hy = P.ny[l] >> 1, nxc = x_entries(hx, 2 * hy);
+    const int hx = P.nx[l] >> 1, nxc = x_entries(hx, P.ny[l]);
     const int chx = (P.nx[l + 1] + 1) >> 1, cnxc = x_entries(chx, (P.ny[l + 1] + 1) & ~1);
     Vec<T, NR>* x = M.x + P.xoff[l];
     const Vec<T, NR>* xc = M.x + P.xoff[l + 1];
-    SmallBlk<T, NR> B[K];
-    int qc[K];
+    Blk<T, NR> B[K];
+    int I[K], j[K];
+    small_blocks<T, NR, K, false>(B, I, j, P, l, M, team);
 #pragma unroll
-    for (int u = 0; u < K; ++u) {
-        int I, J;
-        small_place(B[u], hx, hy, threadIdx.x + u * team, I, J);
-        qc[u] = ((I + J) & 1) * cnxc + xidx(chx, I >> 1, J);
-        T d[2][2];
+    for (int u = 0; u < K; ++u)
         if (B[u].own) {
-            small_load<T, NR, false, false>(B[u], d, P, l, M, I, J);
-#pragma unroll
-            for (int r = 0; r < 2; ++r)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) B[u].x[r][e] = x[(e ^ r) * nxc + B[u].q + r * hx];
+            B[u].template fetch<0>(x, hx);
+            B[u].template fetch<1>(x + nxc, hx);
         }
-    }
     team_sync(l, team);
 #pragma unroll
     for (int u = 0; u < K; ++u) {
         if (!B[u].own) continue;
-        const Vec<T, NR> cv = xc[qc[u]];
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-#pragma unroll
-                for (int k = 0; k < NR; ++k) B[u].x[r][e].v[k] += cv.v[k];
-                x[(e ^ r) * nxc + B[u].q + r * hx] = B[u].x[r][e];
-            }
+        const int J = j[u] >> 1;
+        B[u].add(xc[((I[u] + J) & 1) * cnxc + xidx(chx, I[u] >> 1, J)]);
+        B[u].template put<0>(x, hx);
+        B[u].template put<1>(x + nxc, hx);
     }
     team_sync(l, team);
     small_sweep<T, NR, K, 1>(B, x, nxc, hx, l, team);
@@ -1340,10 +1500,10 @@ template <typename T, int NR, bool BIG>
 __device__ inline void small_core(const SmallPlan& P, SmallMem<T, NR>& M, bool exact) {
     const int tid = threadIdx.x;
     int lmax = 0;   // levels [0, lmax) with this thread in the team
-    while (lmax < P.n - 1 && tid < small_team(P.nx[lmax], P.ny[lmax])) ++lmax;
-    const bool two = BIG && ((P.nx[0] + 1) >> 1) * ((P.ny[0] + 1) >> 1) > (int)blockDim.x;   // level 0: two blocks per thread
+    while (lmax < P.n - 1 && tid < small_team<T>(P.nx[lmax], P.ny[lmax])) ++lmax;
+    const bool two = BIG && Blk<T, NR>::units(P.nx[0], P.ny[0]) > (int)blockDim.x;   // level 0: two blocks per thread
     for (int l = 0; l < lmax; ++l) {
-        const int team = small_team(P.nx[l], P.ny[l]);
+        const int team = small_team<T>(P.nx[l], P.ny[l]);
         bool done = false;
         if constexpr (BIG)
             if (l == 0 && two) {
@@ -1357,7 +1517,7 @@ __device__ inline void small_core(const SmallPlan& P, SmallMem<T, NR>& M, bool e
         if (tid < 32) __syncwarp();
     }
     for (int l = lmax - 1; l >= 0; --l) {
-        const int team = small_team(P.nx[l], P.ny[l]);
+        const int team = small_team<T>(P.nx[l], P.ny[l]);
         bool done = false;
         if constexpr (BIG)
             if (l == 0 && two) {
@@ -1605,22 +1765,26 @@ __device__ __forceinline__ P* cluster_map(P* p, unsigned rank) {
     return reinterpret_cast<P*>((uintptr_t)r);
 }
 // a level's arrays in a block's shared memory: x (rows -1 .. rp, as on the single-block levels),
-// b, then D, wl, wb (one row more) and, in FP64, the reciprocal diagonals
+// b, (FP64) the restriction's partial sums, then D, wl, (FP64) the reciprocal diagonals, wb (one row
+// more)
 template <typename T, int NR>
 struct ClMem {
-    Vec<T, NR>*x, *b;
+    static constexpr bool F64 = sizeof(T) == 8;
+    Vec<T, NR>*x, *b, *s;
     T *d, *wl, *wb, *id;
     __host__ __device__ static int xn(int nx, int rp) { return (2 * x_entries(nx >> 1, rp) + 3) & ~3; }
+    __host__ __device__ static int sn(int nx, int rp) { return F64 ? (rp * nx / 4 + 3) & ~3 : 0; }
     __device__ ClMem(unsigned char* base, int nx, int rp) {
         x = (Vec<T, NR>*)base;
         b = x + xn(nx, rp);
-        d = (T*)(b + rp * nx);
+        s = b + rp * nx;
+        d = (T*)(s + sn(nx, rp));
         wl = d + rp * nx;
         id = wl + rp * nx;
-        wb = id + (sizeof(T) == 8 ? rp * nx : 0);
+        wb = id + (F64 ? rp * nx : 0);
     }
     static int bytes(int nx, int rp) {
-        size_t v = (size_t)(xn(nx, rp) + rp * nx) * NR, c = (size_t)(3 * rp + 1) * nx + (sizeof(T) == 8 ? rp * nx : 0);
+        size_t v = (size_t)(xn(nx, rp) + rp * nx + sn(nx, rp)) * NR, c = (size_t)(3 * rp + 1) * nx + (F64 ? rp * nx : 0);
         return (int)(((v + c + 2) * sizeof(T) + 127) & ~size_t(127));
     }
 };
@@ -1639,75 +1803,39 @@ struct ClSlab {
 // edge of a slab that a block of cells lies on (its new values are pushed there)
 constexpr unsigned CL_DOWN = 1, CL_UP = 2;
 
-// the block's place, weights, reciprocal diagonals, D and right-hand side
-template <typename T, int NR>
-__device__ inline unsigned cl_load(SmallBlk<T, NR>& B, T (&d)[2][2], const ClSlab& S, int ny, const ClMem<T, NR>& M,
-                                   int t, int& I, int& J) {
-    small_place(B, S.hx, (S.j1 - S.j0) >> 1, t, I, J);
-    if (!B.own) return 0;
-    const int c0 = 2 * J * S.nx + 2 * I;
-    using P2 = Vec<T, 2>;
+// the blocks of a thread on level l of the cluster
+template <typename T, int NR, int K>
+__device__ inline void cl_blocks(Blk<T, NR> (&B)[K], unsigned (&edge)[K], int (&I)[K], int (&j)[K], const ClSlab& S,
+                                 int ny, const ClMem<T, NR>& M) {
+    const BlkSrc<T, NR> src = {S.nx, S.j1 - S.j0, M.d, M.wl, M.wb, M.id, M.b};
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int c = c0 + r * S.nx;
-        const P2 w = *reinterpret_cast<const P2*>(M.wl + c), v = *reinterpret_cast<const P2*>(M.wb + c);
-        const P2 dv = *reinterpret_cast<const P2*>(M.d + c);
-        const Vec<T, 2 * NR> bv = *reinterpret_cast<const Vec<T, 2 * NR>*>(M.b + c);
-        const T wr = M.wl[c + 2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            B.wl[r][e] = w.v[e];
-            B.wb[r][e] = v.v[e];
-            d[r][e] = dv.v[e];
-#pragma unroll
-            for (int k = 0; k < NR; ++k) B.b[r][e].v[k] = bv.v[e * NR + k];
-        }
-        B.wl[r][2] = I + 1 < S.hx ? wr : T(0);
-        if (sizeof(T) == 8) {
-            const P2 iv = *reinterpret_cast<const P2*>(M.id + c);
-            B.id[r][0] = iv.v[0];
-            B.id[r][1] = iv.v[1];
-        }
+    for (int u = 0; u < K; ++u) {
+        B[u].place(S.hx, S.j1 - S.j0, threadIdx.x + u * blockDim.x, I[u], j[u]);
+        edge[u] = 0;
+        if (!B[u].own) continue;
+        // the rows below and above are halo rows (zero beyond the grid)
+        B[u].template load<false>(src, I[u], j[u], {I[u] > 0, I[u] + 1 < S.hx, true, true});
+        edge[u] = (j[u] == 0 && S.j0 > 0 ? CL_DOWN : 0u) |
+                  (S.j0 + j[u] + Blk<T, NR>::RB == S.j1 && S.j1 < ny ? CL_UP : 0u);
     }
-    const P2 wt = *reinterpret_cast<const P2*>(M.wb + c0 + 2 * S.nx);
-    B.wb[2][0] = wt.v[0];
-    B.wb[2][1] = wt.v[1];
-    if (sizeof(T) == 4) {
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-                B.id[r][e] = rcp_diag(d[r][e] + B.wl[r][e] + B.wl[r][e + 1] + B.wb[r][e] + B.wb[r + 1][e]);
-    }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) B.wl[r][0] = I > 0 ? B.wl[r][0] : T(0);
-    return (J == 0 && S.j0 > 0 ? CL_DOWN : 0u) | (S.j0 + 2 * J + 2 == S.j1 && S.j1 < ny ? CL_UP : 0u);
 }
 // the new values of colour COLOR in the block's edge rows, into the neighbour slabs' halo rows
-template <typename T, int NR>
-__device__ __forceinline__ void cl_push(const SmallBlk<T, NR>& B, unsigned edge, const ClSlab& S, Vec<T, NR>* xdn,
-                                        Vec<T, NR>* xup, int color) {
-    // entries of the block's column in row rp of the slab below and in row -1 of the slab above
-    if (edge & CL_DOWN) xdn[color * S.nxc + B.q + S.rp * S.hx] = color ? B.x[0][1] : B.x[0][0];
-    if (edge & CL_UP) xup[color * S.nxc + B.q - (S.j1 - S.j0 - 1) * S.hx] = color ? B.x[1][0] : B.x[1][1];
+template <typename T, int NR, int COLOR>
+__device__ __forceinline__ void cl_push(const Blk<T, NR>& B, unsigned edge, int I, const ClSlab& S, Vec<T, NR>* xdn,
+                                        Vec<T, NR>* xup) {
+    if (edge & CL_DOWN) xdn[COLOR * S.nxc + xidx(S.hx, I, S.rp)] = B.template low<COLOR>();
+    if (edge & CL_UP) xup[COLOR * S.nxc + xidx(S.hx, I, -1)] = B.template high<COLOR>();
 }
 template <typename T, int NR, int K, int COLOR, bool LAST = false>
-__device__ inline void cl_sweep(SmallBlk<T, NR> (&B)[K], const unsigned (&edge)[K], const ClSlab& S, Vec<T, NR>* x,
-                                Vec<T, NR>* xdn, Vec<T, NR>* xup) {
-    const Vec<T, NR>* xo = x + (1 - COLOR) * S.nxc;
-    Vec<T, NR>* xs = x + COLOR * S.nxc;
+__device__ inline void cl_sweep(Blk<T, NR> (&B)[K], const unsigned (&edge)[K], const int (&I)[K], const ClSlab& S,
+                                Vec<T, NR>* x, Vec<T, NR>* xdn, Vec<T, NR>* xup) {
 #pragma unroll
     for (int u = 0; u < K; ++u) {
         if (!B[u].own) continue;
-        Vec<T, NR> h0, v0, h1, v1;
-        small_outer<T, NR, COLOR>(B[u], xo, S.hx, h0, v0, h1, v1);
-        const Vec<T, NR> a0 = small_update(B[u], 0, COLOR, h0, v0), a1 = small_update(B[u], 1, 1 - COLOR, h1, v1);
-        B[u].x[0][COLOR] = a0;
-        B[u].x[1][1 - COLOR] = a1;
+        B[u].template sweep<COLOR>(x + (1 - COLOR) * S.nxc, S.hx);
         if (!LAST) {
-            xs[B[u].q] = a0;
-            xs[B[u].q + S.hx] = a1;
-            if (edge[u]) cl_push(B[u], edge[u], S, xdn, xup, COLOR);
+            B[u].template put<COLOR>(x + COLOR * S.nxc, S.hx);
+            if (edge[u]) cl_push<T, NR, COLOR>(B[u], edge[u], I[u], S, xdn, xup);
         }
     }
     if (!LAST) cluster_barrier();
@@ -1720,46 +1848,40 @@ __device__ inline void cl_down(const ClPlan& P, int l, int rank, unsigned char* 
     const ClMem<T, NR> M(smem + P.off[l], S.nx, S.rp);
     Vec<T, NR>* xdn = cluster_map(M.x, rank > 0 ? rank - 1 : 0);
     Vec<T, NR>* xup = cluster_map(M.x, rank + 1 < CL_BLOCKS ? rank + 1 : rank);
-    SmallBlk<T, NR> B[K];
-    T d[K][2][2];
+    Blk<T, NR> B[K];
     unsigned edge[K];
-    int I[K], J[K];
+    int I[K], j[K];
+    cl_blocks<T, NR, K>(B, edge, I, j, S, P.ny[l], M);
 #pragma unroll
     for (int u = 0; u < K; ++u) {
-        edge[u] = cl_load(B[u], d[u], S, P.ny[l], M, threadIdx.x + u * blockDim.x, I[u], J[u]);
         if (!B[u].own) continue;
-        // the first colour-0 half-sweep from x = 0 reduces to x = b / (full diagonal)
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-#pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                B[u].x[r][r].v[k] = B[u].b[r][r].v[k] * B[u].id[r][r];
-                B[u].x[r][1 - r].v[k] = T(0);
-            }
-            M.x[B[u].q + r * S.hx] = B[u].x[r][r];
-        }
-        if (edge[u]) cl_push(B[u], edge[u], S, xdn, xup, 0);
+        B[u].first();
+        B[u].template put<0>(M.x, S.hx);
+        if (edge[u]) cl_push<T, NR, 0>(B[u], edge[u], I[u], S, xdn, xup);
     }
     cluster_barrier();
-    cl_sweep<T, NR, K, 1>(B, edge, S, M.x, xdn, xup);
-    cl_sweep<T, NR, K, 0>(B, edge, S, M.x, xdn, xup);
-    cl_sweep<T, NR, K, 1>(B, edge, S, M.x, xdn, xup);
-    // the block's residual summed into the right-hand side of the next level, in the shared memory
-    // of the block that owns that cell
+    cl_sweep<T, NR, K, 1>(B, edge, I, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 0>(B, edge, I, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 1>(B, edge, I, S, M.x, xdn, xup);
+    // the restricted residual into the right-hand side of the next level, in the shared memory of
+    // the block that owns that cell
+    int slot[K];
 #pragma unroll
-    for (int u = 0; u < K; ++u) {
-        if (!B[u].own) continue;
-        const Vec<T, NR> acc = small_restrict<T, NR, TILE>(B[u], d[u], M.x, S.nxc, S.hx);
-        const int Jg = (S.j0 >> 1) + J[u];
-        if (l + 1 < P.nl) {
-            const int own = small_div(Jg, P.rp[l + 1]);
-            const ClMem<T, NR> N(smem + P.off[l + 1], P.nx[l + 1], P.rp[l + 1]);
-            cluster_map(N.b, own)[(Jg - own * P.rp[l + 1]) * P.nx[l + 1] + I[u]] = acc;
-        } else {
-            const SmallMem<T, NR> N(smem + P.soff, P.S);
-            cluster_map(N.b, 0)[Jg * P.S.nx[0] + I[u]] = acc;
-        }
-    }
+    for (int u = 0; u < K; ++u) slot[u] = (j[u] >> 1) * S.hx + I[u];
+    blk_restrict<T, NR, K, TILE>(
+        B, slot, M.s, M.x, S.nxc, S.hx,
+        [&](int u, const Vec<T, NR>& v) {
+            const int J = (S.j0 + j[u]) >> 1;
+            if (l + 1 < P.nl) {
+                const int own = small_div(J, P.rp[l + 1]);
+                const ClMem<T, NR> N(smem + P.off[l + 1], P.nx[l + 1], P.rp[l + 1]);
+                cluster_map(N.b, own)[(J - own * P.rp[l + 1]) * P.nx[l + 1] + I[u]] = v;
+            } else {
+                const SmallMem<T, NR> N(smem + P.soff, P.S);
+                cluster_map(N.b, 0)[J * P.S.nx[0] + I[u]] = v;
+            }
+        },
+        [&]() { __syncthreads(); });
     cluster_barrier();
 }
 
@@ -1770,55 +1892,54 @@ __device__ inline void cl_up(const ClPlan& P, int l, int rank, unsigned char* sm
     const ClMem<T, NR> M(smem + P.off[l], S.nx, S.rp);
     Vec<T, NR>* xdn = cluster_map(M.x, rank > 0 ? rank - 1 : 0);
     Vec<T, NR>* xup = cluster_map(M.x, rank + 1 < CL_BLOCKS ? rank + 1 : rank);
-    SmallBlk<T, NR> B[K];
+    Blk<T, NR> B[K];
     unsigned edge[K];
-    int I[K], J[K];
+    int I[K], j[K];
+    cl_blocks<T, NR, K>(B, edge, I, j, S, P.ny[l], M);
 #pragma unroll
     for (int u = 0; u < K; ++u) {
-        T d[2][2];
-        edge[u] = cl_load(B[u], d, S, P.ny[l], M, threadIdx.x + u * blockDim.x, I[u], J[u]);
         if (!B[u].own) continue;
-        const int Jg = (S.j0 >> 1) + J[u];
+        const int J = (S.j0 + j[u]) >> 1;
         Vec<T, NR> cv;
         if (l + 1 < P.nl) {
-            const int own = small_div(Jg, P.rp[l + 1]), chx = P.nx[l + 1] >> 1, cnxc = x_entries(chx, P.rp[l + 1]);
+            const int own = small_div(J, P.rp[l + 1]), chx = P.nx[l + 1] >> 1, cnxc = x_entries(chx, P.rp[l + 1]);
             const ClMem<T, NR> N(smem + P.off[l + 1], P.nx[l + 1], P.rp[l + 1]);
-            cv = cluster_map(N.x, own)[((I[u] + Jg) & 1) * cnxc + xidx(chx, I[u] >> 1, Jg - own * P.rp[l + 1])];
+            cv = cluster_map(N.x, own)[((I[u] + J) & 1) * cnxc + xidx(chx, I[u] >> 1, J - own * P.rp[l + 1])];
         } else {
             const int chx = (P.S.nx[0] + 1) >> 1, cnxc = x_entries(chx, (P.S.ny[0] + 1) & ~1);
             const SmallMem<T, NR> N(smem + P.soff, P.S);
-            cv = cluster_map(N.x, 0)[P.S.xoff[0] + ((I[u] + Jg) & 1) * cnxc + xidx(chx, I[u] >> 1, Jg)];
+            cv = cluster_map(N.x, 0)[P.S.xoff[0] + ((I[u] + J) & 1) * cnxc + xidx(chx, I[u] >> 1, J)];
         }
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                Vec<T, NR>* p = M.x + (e ^ r) * S.nxc + B[u].q + r * S.hx;
-                B[u].x[r][e] = *p;
-#pragma unroll
-                for (int k = 0; k < NR; ++k) B[u].x[r][e].v[k] += cv.v[k];
-                *p = B[u].x[r][e];
-            }
-        if (edge[u]) cl_push(B[u], edge[u], S, xdn, xup, 0);
+        B[u].template fetch<0>(M.x, S.hx);
+        B[u].template fetch<1>(M.x + S.nxc, S.hx);
+        B[u].add(cv);
+        B[u].template put<0>(M.x, S.hx);
+        B[u].template put<1>(M.x + S.nxc, S.hx);
+        if (edge[u]) cl_push<T, NR, 0>(B[u], edge[u], I[u], S, xdn, xup);
     }
     cluster_barrier();
-    cl_sweep<T, NR, K, 1>(B, edge, S, M.x, xdn, xup);
-    cl_sweep<T, NR, K, 0>(B, edge, S, M.x, xdn, xup);
-    cl_sweep<T, NR, K, 1>(B, edge, S, M.x, xdn, xup);
-    cl_sweep<T, NR, K, 0, TOP>(B, edge, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 1>(B, edge, I, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 0>(B, edge, I, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 1>(B, edge, I, S, M.x, xdn, xup);
+    cl_sweep<T, NR, K, 0, TOP>(B, edge, I, S, M.x, xdn, xup);
     if (TOP) {
 #pragma unroll
         for (int u = 0; u < K; ++u) {
             if (!B[u].own) continue;
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                Vec<T, 2 * NR> o;
+            for (int r = 0; r < Blk<T, NR>::RB; ++r) {
+                Vec<T, 2 * NR> o;   // columns 2I, 2I + 1 of row j + r
 #pragma unroll
                 for (int k = 0; k < NR; ++k) {
-                    o.v[k] = B[u].x[r][0].v[k];
-                    o.v[NR + k] = B[u].x[r][1].v[k];
+                    if constexpr (Blk<T, NR>::RB == 2) {
+                        o.v[k] = B[u].x[r][0].v[k];
+                        o.v[NR + k] = B[u].x[r][1].v[k];
+                    } else {
+                        o.v[k] = B[u].par ? B[u].x[1].v[k] : B[u].x[0].v[k];
+                        o.v[NR + k] = B[u].par ? B[u].x[0].v[k] : B[u].x[1].v[k];
+                    }
                 }
-                reinterpret_cast<Vec<T, 2 * NR>*>(x_out)[(size_t)(S.j0 + 2 * J[u] + r) * S.hx + I[u]] = o;
+                reinterpret_cast<Vec<T, 2 * NR>*>(x_out)[(size_t)(S.j0 + j[u] + r) * S.hx + I[u]] = o;
             }
         }
     }
@@ -1861,13 +1982,14 @@ k_coarse_cluster(const __grid_constant__ ClPlan P, const T* __restrict__ diag, c
     cp_async_wait_all();
     if (off) return;
     cluster_barrier();
+    auto two = [&](int l) { return Blk<T, NR>::units(P.nx[l], P.rp[l]) > (int)blockDim.x; };   // blocks per thread
     for (int l = 0; l < P.nl; ++l) {
-        if (P.rp[l] * (P.nx[l] >> 1) > 2 * (int)blockDim.x) {
-            if constexpr (sizeof(T) == 4) cl_down<T, NR, 2, true>(P, l, rank, smem);
-        } else if (sizeof(T) == 4 || l < P.nt) {
-            cl_down<T, NR, 1, true>(P, l, rank, smem);
-        } else {
+        if (sizeof(T) == 8 && l >= P.nt) {
             if constexpr (sizeof(T) == 8) cl_down<T, NR, 1, false>(P, l, rank, smem);
+        } else if (two(l)) {
+            cl_down<T, NR, 2, true>(P, l, rank, smem);
+        } else {
+            cl_down<T, NR, 1, true>(P, l, rank, smem);
         }
     }
     if (rank == 0) {
@@ -1876,16 +1998,12 @@ k_coarse_cluster(const __grid_constant__ ClPlan P, const T* __restrict__ diag, c
     }
     cluster_barrier();
     for (int l = P.nl - 1; l >= 0; --l) {
-        const bool two = P.rp[l] * (P.nx[l] >> 1) > 2 * (int)blockDim.x;
-        if (two) {
-            if constexpr (sizeof(T) == 4) {
-                if (l == 0) cl_up<T, NR, 2, true>(P, l, rank, smem, x_out);
-                else cl_up<T, NR, 2, false>(P, l, rank, smem, nullptr);
-            }
-        } else if (l == 0) {
-            cl_up<T, NR, 1, true>(P, l, rank, smem, x_out);
+        if (l == 0) {
+            if (two(l)) cl_up<T, NR, 2, true>(P, l, rank, smem, x_out);
+            else cl_up<T, NR, 1, true>(P, l, rank, smem, x_out);
         } else {
-            cl_up<T, NR, 1, false>(P, l, rank, smem, nullptr);
+            if (two(l)) cl_up<T, NR, 2, false>(P, l, rank, smem, nullptr);
+            else cl_up<T, NR, 1, false>(P, l, rank, smem, nullptr);
         }
     }
 }
@@ -3496,10 +3614,12 @@ static int cluster_plan(Solver& s, ClPlan& P, int& threads, size_t& smem) {
     if (sizeof(T) == 8)
         while (ls < s.nlev - 1 && s.lnx[ls] * s.lny[ls] > 256) ++ls;
     P.S = small_plan<T>(s, ls);
-    const int last = s.nlev - 1, half = CL_THREADS / 2;
-    // (one block of cells per thread on the single-block levels)
-    int need_s = ((s.lnx[last] + 1) / 2) * ((s.lny[last] + 1) / 2);
-    if (ls < last) need_s = std::max(need_s, (s.lnx[ls] / 2) * (s.lny[ls] / 2));
+    const int half = CL_THREADS / 2;
+    // threads the single-block levels want (one block of cells per thread; the coarsest may have two)
+    int need_s = 32;
+    if (ls < s.nlev - 1) need_s = Blk<T, NR>::units(s.lnx[ls], s.lny[ls]);
+    const int uc = Blk<T, NR>::units(s.lnx[s.nlev - 1], s.lny[s.nlev - 1]);
+    need_s = std::max(need_s, sizeof(T) == 8 ? (uc + 1) / 2 : uc);
     for (int l0 = 1; l0 < nb; ++l0) {
         if (ls - l0 > CL_MAX) continue;
         size_t off = 0;
@@ -3518,11 +3638,14 @@ static int cluster_plan(Solver& s, ClPlan& P, int& threads, size_t& smem) {
                 break;
             }
             off += ClMem<T, NR>::bytes(P.nx[k], P.rp[k]);
-            need = std::max(need, (P.rp[k] / 2) * (P.nx[k] / 2));
+            // two blocks of cells per thread at most (one on the FP64 levels below the tiled ones)
+            const int u = Blk<T, NR>::units(P.nx[k], P.rp[k]);
+            if (u > (k < P.nt ? 2 : 1) * CL_THREADS) off = SMEM_MAX + 1;
+            need = std::max(need, std::min(u, CL_THREADS));
         }
         P.soff = (int)off;
         smem = off + SmallMem<T, NR>::bytes(P.S);
-        if (smem > SMEM_MAX || need_s > CL_THREADS || need > (sizeof(T) == 4 ? 2 : 1) * CL_THREADS) continue;
+        if (smem > SMEM_MAX || need_s > CL_THREADS) continue;
         threads = need > half ? CL_THREADS : half;
         return l0;
     }
