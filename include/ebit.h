@@ -307,7 +307,9 @@ ebit_status ebit_get_schedule(ebit_ctx* ctx, int inst, int* small_max, double* i
  *   levels in one launch: a thread-block cluster that keeps them in its shared memory (levels up
  *   to about 256 x 256 cells in FP32, 128 x 128 in FP64), or, where the device takes no such
  *   cluster or a barrier bound is set, a cooperative launch with grid barriers between the phases
- *   (levels whose tiles fit one per co-resident block); 0 launches each level separately.  All
+ *   (levels whose tiles fit one per co-resident block); on grids of at most 16384 cells that fit a
+ *   cluster whole, a complete FP64 solve (mixed precision: each inner FP32 solve) is one launch,
+ *   except while smoothers are timed; 0 launches each level separately.  All
  *   give the same values.  2 (mixed precision) runs each whole inner FP32 solve of the refinement, every
  *   V-cycle and CG update until the inner tolerance, in one cooperative launch with bounded
  *   grid barriers between its phases (grids whose finest tiles fit the reduction slots; others

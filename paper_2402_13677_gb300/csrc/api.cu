@@ -346,18 +346,24 @@ static void collect_stats(Instance& I, bool graph_step) {
     if (!m) return;
     SolveResult r[4];
     bool ok = true;
-    long long body = I.solver.body_size(I.cfg.precision), n = 0;
+    long long n = 0;
     for (int k = 0; k < 4; ++k) {
         if (!(m & (1u << k))) continue;
         r[k] = (k == SLOT_VISC_Y ? I.solver2 : I.solver).result_from_host(k, I.cfg.precision);
         ok = ok && r[k].converged;
         if (r[k].fault) I.fault = true;
         if (r[k].nonfinite) I.nonfinite = true;
-        // kernels executed inside the conditional loop bodies of a graph step
-        n += r[k].iters * body;
-        if (I.cfg.precision == EBIT_MIXED) n += 2 * r[k].outer - 1;
+        // kernels executed inside the conditional loop bodies of a graph step (a batched launch
+        // counts once)
+        if (graph_step && I.bz == 0) {
+            bool whole = false;
+            Solver& sv = k == SLOT_VISC_Y ? I.solver2 : I.solver;
+            const bool two = k == SLOT_VISC_X || k == SLOT_VISC_Y;
+            n += (long long)r[k].iters * sv.body_size(I.cfg.precision, two ? 2 : 1, I.batch < 0, &whole);
+            if (I.cfg.precision == EBIT_MIXED) n += (whole ? 3 : 2) * r[k].outer - (whole ? 2 : 1);
+        }
     }
-    if (graph_step && I.bz == 0) g_launches += (uint64_t)n;   // a batched launch counts once
+    g_launches += (uint64_t)n;
     if (m & (1u << SLOT_ENERGY)) {
         I.stats[0] = r[SLOT_ENERGY].iters;
         I.stats[3] = r[SLOT_ENERGY].rel_res;
@@ -1223,8 +1229,21 @@ ebit_status ebit_get_diagnostics(ebit_ctx* ctx, int inst, double* dst, int n) {
 
 uint64_t ebit_launch_count(const ebit_ctx* ctx) { return ctx ? g_launches.load() - ctx->launch0 : 0; }
 
+// the timed kernels are launches of their own: while they are timed no solve runs as one launch
+// (same values), and captured graphs of the other form are dropped
+static void select_whole_solves(ebit_ctx* ctx, int on) {
+    if (ctx->stream) cudaStreamSynchronize(ctx->stream);
+    for (auto& I : ctx->inst) {
+        if (I.solver.use_cgc == on) continue;
+        I.solver.use_cgc = I.solver2.use_cgc = on;
+        for (auto& gx : I.graph)
+            if (gx) { cudaGraphExecDestroy(gx); gx = nullptr; }
+    }
+}
+
 ebit_status ebit_timing_begin(ebit_ctx* ctx, int kernel_class) {
     if (!ctx || kernel_class != EBIT_KT_SMOOTH_L0) return EBIT_EINVAL;
+    select_whole_solves(ctx, 0);
     for (auto& I : ctx->inst) {
         KTimer z[2];
         for (auto& t : z) {
@@ -1240,6 +1259,7 @@ ebit_status ebit_timing_begin(ebit_ctx* ctx, int kernel_class) {
 
 ebit_status ebit_timing_end(ebit_ctx* ctx, double* total_ms, uint64_t* launches, double* bytes_per_launch) {
     if (!ctx || !total_ms || !launches || !bytes_per_launch) return EBIT_EINVAL;
+    select_whole_solves(ctx, 1);
     double tot = 0.0, bytes = 0.0;
     uint64_t n = 0;
     std::vector<KTimer> t(4 * ctx->inst.size());

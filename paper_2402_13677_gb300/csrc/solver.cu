@@ -1145,6 +1145,16 @@ struct QuadBlk {
 #pragma unroll
                 for (int k = 0; k < NR; ++k) x[r][e].v[k] += c.v[k];
     }
+    // the block's cells in the order of the finest post-smoothing's r.z: (row, column parity, left,
+    // right, lower, upper weight, D, b, x)
+    static constexpr int CELLS = 4;
+    template <class F>
+    __device__ __forceinline__ void cells(F&& f) {
+        f(0, 0, 0, wl[0][0], wl[0][1], wb[0][0], wb[1][0], d[0][0], b[0][0], x[0][0]);
+        f(1, 0, 1, wl[0][1], wl[0][2], wb[0][1], wb[1][1], d[0][1], b[0][1], x[0][1]);
+        f(2, 1, 1, wl[1][1], wl[1][2], wb[1][1], wb[2][1], d[1][1], b[1][1], x[1][1]);
+        f(3, 1, 0, wl[1][0], wl[1][1], wb[1][0], wb[2][0], d[1][0], b[1][0], x[1][0]);
+    }
     template <int COLOR>
     __device__ const V& low() const { return x[0][COLOR]; }        // the colour's cell of the first row
     template <int COLOR>
@@ -1268,6 +1278,12 @@ struct PairBlk {
             x[0].v[k] += c.v[k];
             x[1].v[k] += c.v[k];
         }
+    }
+    static constexpr int CELLS = 2;
+    template <class F>
+    __device__ __forceinline__ void cells(F&& f) {
+        f(0, 0, par, wl[0], wr[0], wb[0], wt[0], d[0], b[0], x[0]);
+        f(1, 0, 1 - par, wl[1], wr[1], wb[1], wt[1], d[1], b[1], x[1]);
     }
     template <int COLOR>
     __device__ const V& low() const { return x[COLOR]; }
@@ -1411,7 +1427,7 @@ __device__ inline void small_down(const SmallPlan& P, int l, SmallMem<T, NR>& M,
 
 // coarsest level: exact solve with the precomputed inverse (up to 32 cells), else a symmetric
 // red-black sweep sequence from zero
-template <typename T, int NR>
+template <typename T, int NR, int K>
 __device__ inline void small_coarsest(const SmallPlan& P, SmallMem<T, NR>& M, bool exact) {
     const int l = P.n - 1, o = P.soff[l], nx = P.nx[l], ny = P.ny[l], n = nx * ny;
     const int hx = (nx + 1) >> 1, nxc = x_entries(hx, (ny + 1) & ~1);
@@ -1437,7 +1453,6 @@ __device__ inline void small_coarsest(const SmallPlan& P, SmallMem<T, NR>& M, bo
         return;
     }
     // (x is zero from the start in a single cycle, not in the later ones of a kernel that runs several)
-    constexpr int K = sizeof(T) == 8 ? 2 : 1;   // up to 1024 cells, in pairs one or two per thread
     Blk<T, NR> B[K];
     int I[K], j[K];
     small_blocks<T, NR, K, true>(B, I, j, P, l, M, team);
@@ -1496,7 +1511,20 @@ __device__ inline void small_up(const SmallPlan& P, int l, SmallMem<T, NR>& M, i
 // level's down leg on its team, the coarsest solve, the up legs.  A warp leaves at the first level
 // it owns no cells of and waits for the others at the up leg of the level before.  BIG: the first
 // level may have more blocks than the team has threads (two per thread).
-template <typename T, int NR, bool BIG>
+// CALL: the legs as calls of their own (inlined into a kernel of many phases they spill).
+template <typename T, int NR>
+__device__ __noinline__ void small_down_call(const SmallPlan& P, int l, SmallMem<T, NR>& M, int team) {
+    small_down<T, NR, 1>(P, l, M, team);
+}
+template <typename T, int NR, int K>
+__device__ __noinline__ void small_coarsest_call(const SmallPlan& P, SmallMem<T, NR>& M, bool exact) {
+    small_coarsest<T, NR, K>(P, M, exact);
+}
+template <typename T, int NR>
+__device__ __noinline__ void small_up_call(const SmallPlan& P, int l, SmallMem<T, NR>& M, int team) {
+    small_up<T, NR, 1>(P, l, M, team);
+}
+template <typename T, int NR, bool BIG, bool CALL = false>
 __device__ inline void small_core(const SmallPlan& P, SmallMem<T, NR>& M, bool exact) {
     const int tid = threadIdx.x;
     int lmax = 0;   // levels [0, lmax) with this thread in the team
@@ -1510,10 +1538,19 @@ __device__ inline void small_core(const SmallPlan& P, SmallMem<T, NR>& M, bool e
                 small_down<T, NR, 2>(P, l, M, team);
                 done = true;
             }
-        if (!done) small_down<T, NR, 1>(P, l, M, team);
+        if constexpr (CALL) small_down_call<T, NR>(P, l, M, team);
+        else if (!done) small_down<T, NR, 1>(P, l, M, team);
     }
     if (lmax == P.n - 1) {
-        small_coarsest<T, NR>(P, M, exact);
+        // up to 1024 cells: blocks of four one per thread, pairs one or two
+        const bool pair2 = sizeof(T) == 8 && Blk<T, NR>::units(P.nx[P.n - 1], P.ny[P.n - 1]) > (int)blockDim.x;
+        if constexpr (CALL) {
+            if (!pair2) small_coarsest_call<T, NR, 1>(P, M, exact);
+            else if constexpr (sizeof(T) == 8) small_coarsest_call<T, NR, 2>(P, M, exact);
+        } else {
+            if (!pair2) small_coarsest<T, NR, 1>(P, M, exact);
+            else if constexpr (sizeof(T) == 8) small_coarsest<T, NR, 2>(P, M, exact);
+        }
         if (tid < 32) __syncwarp();
     }
     for (int l = lmax - 1; l >= 0; --l) {
@@ -1524,7 +1561,8 @@ __device__ inline void small_core(const SmallPlan& P, SmallMem<T, NR>& M, bool e
                 small_up<T, NR, 2>(P, l, M, team);
                 done = true;
             }
-        if (!done) small_up<T, NR, 1>(P, l, M, team);
+        if constexpr (CALL) small_up_call<T, NR>(P, l, M, team);
+        else if (!done) small_up<T, NR, 1>(P, l, M, team);
     }
     __syncthreads();
 }
@@ -1814,7 +1852,8 @@ __device__ inline void cl_blocks(Blk<T, NR> (&B)[K], unsigned (&edge)[K], int (&
         edge[u] = 0;
         if (!B[u].own) continue;
         // the rows below and above are halo rows (zero beyond the grid)
-        B[u].template load<false>(src, I[u], j[u], {I[u] > 0, I[u] + 1 < S.hx, true, true});
+        B[u].template load<false>(src, I[u], j[u],
+                                  {I[u] > 0, I[u] + 1 < S.hx, S.j0 + j[u] > 0, S.j0 + j[u] + Blk<T, NR>::RB < ny});
         edge[u] = (j[u] == 0 && S.j0 > 0 ? CL_DOWN : 0u) |
                   (S.j0 + j[u] + Blk<T, NR>::RB == S.j1 && S.j1 < ny ? CL_UP : 0u);
     }
@@ -1885,16 +1924,13 @@ __device__ inline void cl_down(const ClPlan& P, int l, int rank, unsigned char* 
     cluster_barrier();
 }
 
-// up leg; the result of the first kept level (TOP) goes to x_out, the others' stay in shared memory
+// up leg on the blocks B of the thread (their x is the result); the last half-sweep of the first
+// kept level (TOP) stays in the registers
 template <typename T, int NR, int K, bool TOP>
-__device__ inline void cl_up(const ClPlan& P, int l, int rank, unsigned char* smem, T* __restrict__ x_out) {
-    const ClSlab S(P, l, rank);
-    const ClMem<T, NR> M(smem + P.off[l], S.nx, S.rp);
+__device__ inline void cl_up_blocks(Blk<T, NR> (&B)[K], unsigned (&edge)[K], int (&I)[K], int (&j)[K], const ClSlab& S,
+                                    const ClMem<T, NR>& M, const ClPlan& P, int l, int rank, unsigned char* smem) {
     Vec<T, NR>* xdn = cluster_map(M.x, rank > 0 ? rank - 1 : 0);
     Vec<T, NR>* xup = cluster_map(M.x, rank + 1 < CL_BLOCKS ? rank + 1 : rank);
-    Blk<T, NR> B[K];
-    unsigned edge[K];
-    int I[K], j[K];
     cl_blocks<T, NR, K>(B, edge, I, j, S, P.ny[l], M);
 #pragma unroll
     for (int u = 0; u < K; ++u) {
@@ -1922,6 +1958,16 @@ __device__ inline void cl_up(const ClPlan& P, int l, int rank, unsigned char* sm
     cl_sweep<T, NR, K, 0>(B, edge, I, S, M.x, xdn, xup);
     cl_sweep<T, NR, K, 1>(B, edge, I, S, M.x, xdn, xup);
     cl_sweep<T, NR, K, 0, TOP>(B, edge, I, S, M.x, xdn, xup);
+}
+// up leg; the result of the first kept level (TOP) goes to x_out, the others' stay in shared memory
+template <typename T, int NR, int K, bool TOP>
+__device__ inline void cl_up(const ClPlan& P, int l, int rank, unsigned char* smem, T* __restrict__ x_out) {
+    const ClSlab S(P, l, rank);
+    const ClMem<T, NR> M(smem + P.off[l], S.nx, S.rp);
+    Blk<T, NR> B[K];
+    unsigned edge[K];
+    int I[K], j[K];
+    cl_up_blocks<T, NR, K, TOP>(B, edge, I, j, S, M, P, l, rank, smem);
     if (TOP) {
 #pragma unroll
         for (int u = 0; u < K; ++u) {
@@ -1945,14 +1991,12 @@ __device__ inline void cl_up(const ClPlan& P, int l, int rank, unsigned char* sm
     }
 }
 
+// the cluster's levels into shared memory: operators and the first level's right-hand side, all
+// copies in flight at once (the caller waits and meets at a cluster barrier), x zeroed; block 0
+// also the single-block levels (true if their coarsest one has its inverse)
 template <typename T, int NR>
-__global__ void __launch_bounds__(CL_THREADS, 1)
-k_coarse_cluster(const __grid_constant__ ClPlan P, const T* __restrict__ diag, const T* __restrict__ id,
-                 const T* __restrict__ wl, const T* __restrict__ wb, const T* __restrict__ inv,
-                 const T* __restrict__ b_in, T* __restrict__ x_out, const SolveState* st) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    const int rank = cluster_rank();
-    // operators and the first level's right-hand side, all copies in flight at once; x zeroed
+__device__ inline bool cl_operators(const ClPlan& P, int rank, unsigned char* smem, const T* diag, const T* id,
+                                    const T* wl, const T* wb, const T* inv, const T* b_in) {
     for (int l = 0; l < P.nl; ++l) {
         const ClSlab S(P, l, rank);
         const ClMem<T, NR> M(smem + P.off[l], S.nx, S.rp);
@@ -1978,13 +2022,28 @@ k_coarse_cluster(const __grid_constant__ ClPlan P, const T* __restrict__ diag, c
         SmallMem<T, NR> M(smem + P.soff, P.S);
         exact = small_operators<T, NR>(P.S, M, diag, id, wl, wb, inv);
     }
-    const bool off = skip(st);   // written by an earlier launch: the same for every block
-    cp_async_wait_all();
-    if (off) return;
-    cluster_barrier();
-    auto two = [&](int l) { return Blk<T, NR>::units(P.nx[l], P.rp[l]) > (int)blockDim.x; };   // blocks per thread
+    return exact;
+}
+// (as above) the legs as calls of their own
+template <typename T, int NR, bool TILE>
+__device__ __noinline__ void cl_down_call(const ClPlan& P, int l, int rank, unsigned char* smem) {
+    cl_down<T, NR, 1, TILE>(P, l, rank, smem);
+}
+template <typename T, int NR>
+__device__ __noinline__ void cl_up_call(const ClPlan& P, int l, int rank, unsigned char* smem) {
+    cl_up<T, NR, 1, false>(P, l, rank, smem, nullptr);
+}
+// the down legs, the single-block levels in block 0, and the up legs of the levels below the first;
+// CALL: as calls, one block of cells per thread (else two on the first level where it needs them)
+template <typename T, int NR, bool CALL>
+__device__ inline void cl_cycle(const ClPlan& P, int rank, unsigned char* smem, bool exact) {
+    auto two = [&](int l) { return Blk<T, NR>::units(P.nx[l], P.rp[l]) > (int)blockDim.x; };
     for (int l = 0; l < P.nl; ++l) {
-        if (sizeof(T) == 8 && l >= P.nt) {
+        const bool tile = sizeof(T) == 4 || l < P.nt;
+        if constexpr (CALL) {
+            if (tile) cl_down_call<T, NR, true>(P, l, rank, smem);
+            else if constexpr (sizeof(T) == 8) cl_down_call<T, NR, false>(P, l, rank, smem);
+        } else if (!tile) {
             if constexpr (sizeof(T) == 8) cl_down<T, NR, 1, false>(P, l, rank, smem);
         } else if (two(l)) {
             cl_down<T, NR, 2, true>(P, l, rank, smem);
@@ -1994,18 +2053,31 @@ k_coarse_cluster(const __grid_constant__ ClPlan P, const T* __restrict__ diag, c
     }
     if (rank == 0) {
         SmallMem<T, NR> M(smem + P.soff, P.S);
-        small_core<T, NR, false>(P.S, M, exact);
+        small_core<T, NR, false, CALL>(P.S, M, exact);
     }
     cluster_barrier();
-    for (int l = P.nl - 1; l >= 0; --l) {
-        if (l == 0) {
-            if (two(l)) cl_up<T, NR, 2, true>(P, l, rank, smem, x_out);
-            else cl_up<T, NR, 1, true>(P, l, rank, smem, x_out);
-        } else {
-            if (two(l)) cl_up<T, NR, 2, false>(P, l, rank, smem, nullptr);
-            else cl_up<T, NR, 1, false>(P, l, rank, smem, nullptr);
-        }
+    for (int l = P.nl - 1; l >= 1; --l) {
+        if constexpr (CALL) cl_up_call<T, NR>(P, l, rank, smem);
+        else if (two(l)) cl_up<T, NR, 2, false>(P, l, rank, smem, nullptr);
+        else cl_up<T, NR, 1, false>(P, l, rank, smem, nullptr);
     }
+}
+
+template <typename T, int NR>
+__global__ void __launch_bounds__(CL_THREADS, 1)
+k_coarse_cluster(const __grid_constant__ ClPlan P, const T* __restrict__ diag, const T* __restrict__ id,
+                 const T* __restrict__ wl, const T* __restrict__ wb, const T* __restrict__ inv,
+                 const T* __restrict__ b_in, T* __restrict__ x_out, const SolveState* st) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int rank = cluster_rank();
+    const bool exact = cl_operators<T, NR>(P, rank, smem, diag, id, wl, wb, inv, b_in);
+    const bool off = skip(st);   // written by an earlier launch: the same for every block
+    cp_async_wait_all();
+    if (off) return;
+    cluster_barrier();
+    cl_cycle<T, NR, false>(P, rank, smem, exact);
+    if (Blk<T, NR>::units(P.nx[0], P.rp[0]) > (int)blockDim.x) cl_up<T, NR, 2, true>(P, 0, rank, smem, x_out);
+    else cl_up<T, NR, 1, true>(P, 0, rank, smem, x_out);
 }
 
 // dense inverse of the coarsest operator (at most 32 cells), Gauss-Jordan in precision T by the
@@ -2946,6 +3018,364 @@ k_cg_persist(CoarsePlan<T> C, SmallPlan P, const T* __restrict__ diag, const T* 
     }
 }
 
+// ---- a whole CG solve in one thread-block cluster (grids of up to 16384 cells, instances alone) ---
+// On these grids a CG iteration is five launches of 5 to 50 us whose work is a microsecond or two:
+// launch, first reads of the state, the reduction's tail.  The cluster of the coarse levels also
+// keeps level 0: r and x (z) with its slab, the search direction p with halo rows, the solution;
+// an iteration is the V-cycle's phases, four reductions' worth of cluster barriers and no launch.
+// A reduction's partial sums are stored into every block's shared memory, so all blocks form the
+// same totals, alpha, beta and convergence decision.
+//   * r.z: the sums of the post-smoothing tiles (32 x 32, the shuffle trees of its 13 warps) are
+//     formed by the block tile t belongs to (t % 16), in the tile kernel's precision and order.
+//   * p.q and r.r: the sums of the element kernels.  A unit is what one of their threads sums (FP64
+//     a cell; FP32, by FP32-pair sums, four cells of a row, two with two right-hand sides, one where
+//     rows are not a multiple of four), units go in groups of 32 (a warp's tree), eight groups a
+//     block's slot, then the slots' tree.  Four lanes take a group: a lane-parallel tree is nine
+//     FP64 instructions per 8 groups where shuffle trees are 40.
+// So a solve is bit for bit that of the separate launches.  Bound: latency, a chain of some 60
+// cluster and block barriers and FP64 sweeps (64 cycles an operation) an iteration.  Measured, one
+// solve of the separate launches -> this kernel: 120x104 FP64 to 1e-10 1.27 -> 0.94 ms; ten steps on
+// 64x64 in FP64 8.7 -> 6.5 ms.
+struct CgPlan {
+    ClPlan C;
+    int p_off, x_off, prod_off, w_off, tb_off, tw_off, ts_off;   // byte offsets in shared memory
+    int tx, nt, tslots;          // 32 x 32 tiles: a row, all, per block
+    int unit;                    // cells of a unit of p.q and r.r
+    int pstride;                 // entries of prod per right-hand side
+    int ngrp, nslot;             // slots of 8 groups of 32 units, and their groups
+};
+constexpr int CG_GRP = 36;       // a group of 32 products takes 36 (fewer bank conflicts)
+
+// totals over the whole cluster; buf: which of the two sets of partial sums.  The FP64 work on a
+// total (a division is ten dependent operations) is one lane's, fin(k, total) by lane 0 of warp k:
+// every thread of the block doing it would keep the FP64 pipe busy for 2 us.
+template <typename T, int NR>
+struct CgSum {
+    const CgPlan& P;
+    unsigned char* smem;
+    int rank, buf;
+    // prod[k][unit] is in shared memory (every unit of the slab written): its `units` units, the first
+    // one of group g0
+    template <class Fin>
+    __device__ void total(int units, int g0, Fin&& fin) {
+        double* prod = (double*)(smem + P.prod_off);
+        double* W = (double*)(smem + P.w_off) + buf * NR * P.ngrp;
+        const int ps = P.pstride, ng = (units + 31) / 32, m = threadIdx.x & 3, lane = threadIdx.x & 31;
+        __syncthreads();
+        for (int q0 = 0; q0 < ng * NR; q0 += blockDim.x >> 2) {
+            const int q = q0 + (threadIdx.x >> 2), k = q >= ng && NR > 1 ? 1 : 0, g = q - k * ng;
+            const bool in = q < ng * NR;
+            double v[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) v[t] = in ? prod[k * ps + g * CG_GRP + m + 4 * t] : 0.0;
+            // lanes i and i + 16, i + 8, i + 4 of the warp tree: i = m + 4 t
+            double c = ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+            c += __shfl_down_sync(0xffffffffu, c, 2, 4);
+            c += __shfl_down_sync(0xffffffffu, c, 1, 4);
+            c = __shfl_sync(0xffffffffu, c, lane & ~3);
+            if (in)
+#pragma unroll
+                for (int r = 0; r < CL_BLOCKS / 4; ++r) cluster_map(W, m + 4 * r)[k * P.ngrp + g0 + g] = c;
+        }
+        cluster_barrier();
+        if (threadIdx.x < 32 * NR) {   // warp k
+            const int k = threadIdx.x >> 5;
+            double s[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int v = lane + 32 * h;
+                s[h] = 0.0;
+                if (v < P.nslot) {
+                    const double* w = W + k * P.ngrp + 8 * v;
+                    s[h] = ((w[0] + w[4]) + (w[2] + w[6])) + ((w[1] + w[5]) + (w[3] + w[7]));
+                }
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                s[0] += __shfl_down_sync(0xffffffffu, s[0], o);
+                if (P.nslot > 32) s[1] += __shfl_down_sync(0xffffffffu, s[1], o);
+            }
+            if (lane == 0) fin(k, P.nslot > 32 ? s[0] + s[1] : s[0]);
+        }
+        __syncthreads();
+    }
+};
+
+template <typename T, int NR>
+__global__ void __launch_bounds__(CL_THREADS, 1)
+k_cg_cluster(const __grid_constant__ CgPlan G, const T* __restrict__ diag, const T* __restrict__ id,
+             const T* __restrict__ wl, const T* __restrict__ wb, const T* __restrict__ inv, const T* __restrict__ r_in,
+             T* x_io, SolveState* st) {
+    using V = Vec<T, NR>;
+    extern __shared__ __align__(128) unsigned char smem[];
+    // the solve's scalars, the same in every block
+    __shared__ double rz[2], alpha[2], beta[2], pq[2], rr[2], tol2[2];
+    __shared__ int cont[2], nonfin[2];   // the residual is above the tolerance / not finite
+    const ClPlan& P = G.C;
+    const int rank = cluster_rank();
+    const bool exact = cl_operators<T, NR>(P, rank, smem, diag, id, wl, wb, inv, r_in);
+    const ClSlab S(P, 0, rank);
+    const ClMem<T, NR> M(smem + P.off[0], S.nx, S.rp);
+    V* pa = (V*)(smem + G.p_off);            // p, as a level's x array
+    V* xs = (V*)(smem + G.x_off);            // the solution, [cell of the block][thread]
+    V* xg = reinterpret_cast<V*>(x_io);
+    const int nthr = blockDim.x, rows = S.j1 - S.j0;
+    for (int i = threadIdx.x; i < 2 * S.nxc; i += nthr) {
+        V z;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) z.v[k] = T(0);
+        pa[i] = z;
+    }
+    {   // partial sums that no block writes count as 0; cells of the last group beyond the grid too
+        const int bytes = G.ts_off + (int)sizeof(double) * NR * 64 - G.prod_off;
+        for (int i = threadIdx.x; i < bytes / 4; i += nthr) reinterpret_cast<int*>(smem + G.prod_off)[i] = 0;
+    }
+    if (threadIdx.x < 2) {
+        rz[threadIdx.x] = st->rz[threadIdx.x];
+        tol2[threadIdx.x] = st->tol2[threadIdx.x];
+    }
+    int iters = ld_now(&st->iters);
+    const int maxit = ld_now(&st->max_iters);
+    const bool off = skip(st);   // written by an earlier launch: the same for every block
+    Blk<T, NR> B[1];
+    unsigned edge[1];
+    int I[1], j[1];
+    B[0].place(S.hx, rows, threadIdx.x, I[0], j[0]);
+    // global index of the block's cell (row r, column e), or of the local one
+    auto gcell = [&](int r, int e) { return (S.j0 + j[0] + r) * S.nx + 2 * I[0] + e; };
+    if (!off && B[0].own)
+        B[0].cells([&](int n, int r, int e, T, T, T, T, T, const V&, const V&) { xs[n * nthr + threadIdx.x] = xg[gcell(r, e)]; });
+    cp_async_wait_all();
+    if (off) return;
+    cluster_barrier();
+    V* pdn = cluster_map(pa, rank > 0 ? rank - 1 : 0);
+    V* pup = cluster_map(pa, rank + 1 < CL_BLOCKS ? rank + 1 : rank);
+    bool done = false, bad = false;
+    while (!done && iters < maxit) {
+        // ---- z = M r
+        cl_cycle<T, NR, true>(P, rank, smem, exact);
+        cl_up_blocks<T, NR, 1, true>(B, edge, I, j, S, M, P, 0, rank, smem);
+        // ---- r.z of the block's 2 x 2 cells to the owner of its tile
+        {
+            const int Jg = (S.j0 + j[0]) >> 1, t = (Jg >> 4) * G.tx + (I[0] >> 4);
+            T* TB = (T*)(smem + G.tb_off);
+            V dot;
+#pragma unroll
+            for (int k = 0; k < NR; ++k) dot.v[k] = T(0);
+            auto add = [&]() {
+                B[0].cells([&](int, int, int, T, T, T, T, T, const V& bv, const V& xv) {
+#pragma unroll
+                    for (int k = 0; k < NR; ++k) dot.v[k] = fma_rn(xv.v[k], bv.v[k], dot.v[k]);
+                });
+            };
+            bool send = B[0].own;
+            if constexpr (Blk<T, NR>::RB == 1) {   // the even row's two cells, then the odd row's
+                const int slot = (j[0] >> 1) * S.hx + I[0];
+                if (B[0].own && !(j[0] & 1)) {
+                    add();
+                    M.s[slot] = dot;
+                    send = false;
+                }
+                __syncthreads();
+                if (B[0].own && (j[0] & 1)) {
+                    dot = M.s[slot];
+                    add();
+                }
+            } else if (B[0].own) {
+                add();
+            }
+            if (send) {
+                T* dst = cluster_map(TB, t & (CL_BLOCKS - 1)) + (t / CL_BLOCKS) * NR * 256 + (Jg & 15) * 16 + (I[0] & 15);
+#pragma unroll
+                for (int k = 0; k < NR; ++k) dst[k * 256] = dot.v[k];
+            }
+            cluster_barrier();
+            // the trees of the tile kernel's 13 warps over its 20 x 20 threads (16 x 16 of them with cells)
+            T* TW = (T*)(smem + G.tw_off);
+            double* TS = (double*)(smem + G.ts_off);
+            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = nthr >> 5, jobs = G.tslots * NR;
+            for (int q = warp; q < jobs * 13; q += nw) {
+                const int sk = q / 13, ix = 32 * (q - sk * 13) + lane, kk = ix % 20 - 2, sg = ix / 20 - 2;
+                T v = kk >= 0 && kk < 16 && sg >= 0 && sg < 16 ? TB[sk * 256 + sg * 16 + kk] : T(0);
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+                if (lane == 0) TW[sk * 16 + q - sk * 13] = v;
+            }
+            __syncthreads();
+            for (int sk = warp; sk < jobs; sk += nw) {
+                T v = lane < 13 ? TW[sk * 16 + lane] : T(0);
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+                const double w = widen(__shfl_sync(0xffffffffu, v, 0));
+                const int tt = (sk / NR) * CL_BLOCKS + rank;
+                if (tt < G.nt && lane < CL_BLOCKS) cluster_map(TS, lane)[(sk % NR) * 64 + tt] = w;
+            }
+            cluster_barrier();
+            if (warp < NR) {
+                double a = TS[warp * 64 + lane], b = TS[warp * 64 + 32 + lane];   // 0 beyond the tiles
+                for (int o = 16; o > 0; o >>= 1) {
+                    a += __shfl_down_sync(0xffffffffu, a, o);
+                    if (G.nt > 32) b += __shfl_down_sync(0xffffffffu, b, o);
+                }
+                if (lane == 0) {
+                    const double tot = G.nt > 32 ? a + b : a, old = rz[warp];
+                    beta[warp] = old != 0.0 ? tot / old : 0.0;
+                    rz[warp] = tot;
+                }
+            }
+            __syncthreads();
+        }
+        // ---- p = z + beta p, its edge rows to the neighbours
+        T bt[NR];
+#pragma unroll
+        for (int k = 0; k < NR; ++k) bt[k] = (T)beta[k];
+        auto pidx = [&](int r, int e) { return ((e ^ r ^ (j[0] & 1)) ? S.nxc : 0) + xidx(S.hx, I[0], j[0] + r); };
+        if (B[0].own)
+            B[0].cells([&](int, int r, int e, T, T, T, T, T, const V&, V& xv) {
+                V* q = pa + pidx(r, e);
+                const V po = *q;
+#pragma unroll
+                for (int k = 0; k < NR; ++k)
+                    if (bt[k] != T(0)) xv.v[k] = fma_rn(bt[k], po.v[k], xv.v[k]);
+                *q = xv;   // the block's x is now p
+                if ((edge[0] & CL_DOWN) && r == 0) pdn[(q - pa) + S.rp * S.hx] = xv;
+                if ((edge[0] & CL_UP) && r == Blk<T, NR>::RB - 1) pup[(q - pa) - rows * S.hx] = xv;
+            });
+        cluster_barrier();
+        // ---- q = A p, p.q
+        V qv[Blk<T, NR>::CELLS];
+        // the cells' terms a.b summed by unit into shared memory, then over the cluster
+        auto dot = [&](const V (&a)[Blk<T, NR>::CELLS], const V (&b)[Blk<T, NR>::CELLS], int buf, auto&& fin) {
+            double* prod = (double*)(smem + G.prod_off);
+            auto put = [&](int k, int c, double v) {   // unit of local cell c (its last one)
+                const int u = c / G.unit;
+                prod[k * G.pstride + u + 4 * (u >> 5)] = v;
+            };
+            if constexpr (sizeof(T) == 8) {
+                if (B[0].own)
+#pragma unroll
+                    for (int n = 0; n < 2; ++n)
+#pragma unroll
+                        for (int k = 0; k < NR; ++k)
+                            put(k, j[0] * S.nx + 2 * I[0] + (n ^ B[0].par), a[n].v[k] * b[n].v[k]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int c = (j[0] + r) * S.nx + 2 * I[0], n0 = r ? 3 : 0, n1 = r ? 2 : 1;   // columns 2I, 2I + 1
+                    DotAcc<T, NR> acc;
+                    if (G.unit == 1) {
+                        if (B[0].own)
+#pragma unroll
+                            for (int k = 0; k < NR; ++k) {
+                                DotAcc<T, NR> one;
+                                one.add(k, a[n0].v[k], b[n0].v[k]);
+                                one.flush();
+                                put(k, c, one.tot[k]);
+                                acc.add(k, a[n1].v[k], b[n1].v[k]);
+                                acc.flush();
+                                put(k, c + 1, acc.tot[k]);
+                            }
+                        continue;
+                    }
+                    if (B[0].own)
+#pragma unroll
+                        for (int k = 0; k < NR; ++k) {
+                            acc.add(k, a[n0].v[k], b[n0].v[k]);
+                            acc.add(k, a[n1].v[k], b[n1].v[k]);
+                        }
+                    if (G.unit == 4) {   // the odd thread of two neighbours goes on from the even one's sum
+                        DotAcc<T, NR> go = acc;
+#pragma unroll
+                        for (int k = 0; k < NR; ++k) {
+                            go.sum[k].hi = __shfl_up_sync(0xffffffffu, acc.sum[k].hi, 1);
+                            go.sum[k].lo = __shfl_up_sync(0xffffffffu, acc.sum[k].lo, 1);
+                        }
+                        if (B[0].own && (I[0] & 1))
+#pragma unroll
+                            for (int k = 0; k < NR; ++k) {
+                                go.add(k, a[n0].v[k], b[n0].v[k]);
+                                go.add(k, a[n1].v[k], b[n1].v[k]);
+                                go.flush();
+                                put(k, c, go.tot[k]);
+                            }
+                    } else if (B[0].own) {
+#pragma unroll
+                        for (int k = 0; k < NR; ++k) {
+                            acc.flush();
+                            put(k, c, acc.tot[k]);
+                        }
+                    }
+                }
+            }
+            CgSum<T, NR>{G, smem, rank, buf}.total(rows * S.nx / G.unit, S.j0 * S.nx / (32 * G.unit), fin);
+        };
+        V pv_[Blk<T, NR>::CELLS];
+        if (B[0].own)
+            B[0].cells([&](int n, int r, int e, T w0, T w1, T w2, T w3, T dg, const V&, const V& pv) {
+                const int row = j[0] + r;
+                const V* q = pa + (((e ^ row) & 1) ? 0 : S.nxc);   // the other colour
+                const int x0 = xidx(S.hx, I[0], row);
+                const V pl = q[e ? x0 : x0 - 1], pr = q[e ? x0 + 1 : x0], pd = q[x0 - S.hx], pu = q[x0 + S.hx];
+#pragma unroll
+                for (int k = 0; k < NR; ++k) {
+                    const T pc = pv.v[k];
+                    T a = fma_rn(w0, pc - pl.v[k], dg * pc);
+                    a = fma_rn(w1, pc - pr.v[k], a);
+                    a = fma_rn(w2, pc - pd.v[k], a);
+                    a = fma_rn(w3, pc - pu.v[k], a);
+                    qv[n].v[k] = a;
+                }
+            });
+        if (B[0].own)
+            B[0].cells([&](int n, int, int, T, T, T, T, T, const V&, const V& p) { pv_[n] = p; });
+        dot(pv_, qv, 0, [&](int k, double t) {
+            pq[k] = t;
+            alpha[k] = t != 0.0 ? rz[k] / t : 0.0;
+        });
+        // ---- x += alpha p, r -= alpha q, r.r
+        T al[NR];
+#pragma unroll
+        for (int k = 0; k < NR; ++k) al[k] = (T)alpha[k];
+        if (B[0].own)
+            B[0].cells([&](int n, int r, int e, T, T, T, T, T, V& bv, const V& pv) {
+                V xv = xs[n * nthr + threadIdx.x];
+#pragma unroll
+                for (int k = 0; k < NR; ++k) {
+                    xv.v[k] = fma_rn(al[k], pv.v[k], xv.v[k]);
+                    bv.v[k] = fma_rn(-al[k], qv[n].v[k], bv.v[k]);
+                }
+                qv[n] = bv;
+                xs[n * nthr + threadIdx.x] = xv;
+                M.b[(j[0] + r) * S.nx + 2 * I[0] + e] = bv;
+            });
+        dot(qv, qv, 1, [&](int k, double t) {
+            rr[k] = t;
+            cont[k] = !(t <= tol2[k]);
+            nonfin[k] = !isfinite(t);
+        });
+        iters += 1;
+        done = true;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            if (cont[k]) done = false;
+            bad = bad || nonfin[k] != 0;
+        }
+        if (bad) done = true;   // a NaN or infinity: no further iteration can recover
+    }
+    if (B[0].own)
+        B[0].cells([&](int n, int r, int e, T, T, T, T, T, const V&, const V&) { xg[gcell(r, e)] = xs[n * nthr + threadIdx.x]; });
+    if (rank == 0 && threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            st->rz[k] = rz[k];
+            st->beta[k] = beta[k];
+            st->pq[k] = pq[k];
+            st->alpha[k] = alpha[k];
+            st->rr[k] = rr[k];
+        }
+        st->iters = iters;
+        if (bad) st->nonfinite = 1;
+        if (done) st->done = 1;
+    }
+}
+
 // FP64 CG start: r = b - A x, r.r, b.b, tolerance, state reset
 template <int NR>
 __global__ void __launch_bounds__(256)
@@ -3574,26 +4004,19 @@ static int coarse_start(Solver& s) {
     return nb;
 }
 
-// Plan of the cluster launch: the first tiled level l0 >= 1 from which every level fits the
-// cluster's shared memory and threads (l0 = nb: none; the finest level stays separate, its
-// post-smoothing carries the r.z of CG).  In FP64, where a half-sweep of 32 x 32 cells takes one
-// SM 0.8 us of FP64 issue against 0.45 us over the cluster, the levels above 256 cells stay in the
-// cluster; in FP32 those above the single-block size.  Single instances; a bound set for the grid
-// barriers (EBIT_OPT_BARRIER_SPIN) asks for the grid-barrier launch.
-template <typename T, int NR>
-static int cluster_plan(Solver& s, ClPlan& P, int& threads, size_t& smem) {
-    const int nb = nbig_of<T>(s);
-    if (s.use_coop != 1 || s.barrier_spin > 0 || s.nz != 1 || nb < 2) return nb;
-    static std::atomic<int> usable[64][2][2];   // per device, precision, NR: 0 not asked, 1 yes, 2 no
+constexpr size_t SMEM_MAX = 216 * 1024;   // dynamic shared memory of the cluster kernels, at most
+
+// whether the current device takes a cluster of CL_BLOCKS blocks of the kernel (asked once per
+// device and kernel slot)
+static bool cluster_usable(const void* kern, int slot) {
+    static std::atomic<int> usable[64][8];   // 0 not asked, 1 yes, 2 no
     int dev = 0;
     cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return nb;
-    constexpr size_t SMEM_MAX = 216 * 1024;
-    std::atomic<int>& u = usable[dev][PT<T>::prec][NR - 1];
+    if (dev < 0 || dev >= 64) return false;
+    std::atomic<int>& u = usable[dev][slot];
     if (u.load() == 0) {
-        cudaError_t first = cudaSuccess;
-        allow_smem(k_coarse_cluster<T, NR>, (int)SMEM_MAX, &first);
-        cudaError_t e = cudaFuncSetAttribute(k_coarse_cluster<T, NR>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(CL_BLOCKS);
         cfg.blockDim = dim3(CL_THREADS);
@@ -3605,21 +4028,44 @@ static int cluster_plan(Solver& s, ClPlan& P, int& threads, size_t& smem) {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int n = 0;
-        if (first == cudaSuccess && e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_coarse_cluster<T, NR>, &cfg);
-        u.store(first == cudaSuccess && e == cudaSuccess && n > 0 ? 1 : 2);
-        cudaGetLastError();
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+        u.store(e == cudaSuccess && n > 0 ? 1 : 2);
+        if (e != cudaSuccess) cudaGetLastError();
     }
-    if (u.load() != 1) return nb;
-    int ls = nb;   // first single-block level
+    return u.load() == 1;
+}
+
+// threads that the single-block levels from ls on want (one block of cells per thread; the
+// coarsest FP64 one may have two)
+template <typename T, int NR>
+static int small_threads(const Solver& s, int ls) {
+    int need = 32;
+    if (ls < s.nlev - 1) need = Blk<T, NR>::units(s.lnx[ls], s.lny[ls]);
+    const int uc = Blk<T, NR>::units(s.lnx[s.nlev - 1], s.lny[s.nlev - 1]);
+    return std::max(need, sizeof(T) == 8 ? (uc + 1) / 2 : uc);
+}
+// first level that block 0 of the cluster runs alone
+template <typename T>
+static int cluster_small(const Solver& s, int nb) {
+    int ls = nb;
     if (sizeof(T) == 8)
         while (ls < s.nlev - 1 && s.lnx[ls] * s.lny[ls] > 256) ++ls;
+    return ls;
+}
+
+// Plan of the cluster launch: the first tiled level l0 >= 1 from which every level fits the
+// cluster's shared memory and threads (l0 = nb: none; the finest level stays separate, its
+// post-smoothing carries the r.z of CG).  In FP64, where a half-sweep of 32 x 32 cells takes one
+// SM 0.8 us of FP64 issue against 0.45 us over the cluster, the levels above 256 cells stay in the
+// cluster; in FP32 those above the single-block size.  Single instances; a bound set for the grid
+// barriers (EBIT_OPT_BARRIER_SPIN) asks for the grid-barrier launch.
+template <typename T, int NR>
+static int cluster_plan(Solver& s, ClPlan& P, int& threads, size_t& smem) {
+    const int nb = nbig_of<T>(s);
+    if (s.use_coop != 1 || s.barrier_spin > 0 || s.nz != 1 || nb < 2) return nb;
+    if (!cluster_usable((const void*)k_coarse_cluster<T, NR>, PT<T>::prec * 2 + NR - 1)) return nb;
+    const int ls = cluster_small<T>(s, nb), half = CL_THREADS / 2, need_s = small_threads<T, NR>(s, ls);
     P.S = small_plan<T>(s, ls);
-    const int half = CL_THREADS / 2;
-    // threads the single-block levels want (one block of cells per thread; the coarsest may have two)
-    int need_s = 32;
-    if (ls < s.nlev - 1) need_s = Blk<T, NR>::units(s.lnx[ls], s.lny[ls]);
-    const int uc = Blk<T, NR>::units(s.lnx[s.nlev - 1], s.lny[s.nlev - 1]);
-    need_s = std::max(need_s, sizeof(T) == 8 ? (uc + 1) / 2 : uc);
     for (int l0 = 1; l0 < nb; ++l0) {
         if (ls - l0 > CL_MAX) continue;
         size_t off = 0;
@@ -3650,6 +4096,81 @@ static int cluster_plan(Solver& s, ClPlan& P, int& threads, size_t& smem) {
         return l0;
     }
     return nb;
+}
+
+// Plan of the whole-solve cluster kernel; false where the grid does not fit it (or the separate
+// launches are asked for: EBIT_OPT_COOP other than 1, a barrier bound, smoother timing, a batch)
+template <typename T, int NR>
+static bool cg_plan(Solver& s, CgPlan& G, int& threads, size_t& smem) {
+    const int nb = nbig_of<T>(s);
+    if (s.use_coop != 1 || s.barrier_spin > 0 || s.nz != 1 || !s.use_cgc || nb < 1) return false;
+    const int nx = s.nx, ny = s.ny;
+    // 16 blocks then have more work than launches cost: a 160x160 mixed step took 930 us separate, 940 whole
+    if ((long long)nx * ny > 16384) return false;
+    if (!cluster_usable((const void*)k_cg_cluster<T, NR>, 4 + PT<T>::prec * 2 + NR - 1)) return false;
+    ClPlan& P = G.C;
+    const int ls = cluster_small<T>(s, nb);
+    if (ls > CL_MAX) return false;
+    P.S = small_plan<T>(s, ls);
+    P.nl = ls;
+    P.nt = nb;
+    G.unit = sizeof(T) == 8 ? 1 : NR == 2 ? 2 : nx % 4 == 0 ? 4 : 1;   // as cg_body chooses its kernels
+    G.nslot = (nx * ny / G.unit + 255) / 256;
+    G.ngrp = 8 * G.nslot;
+    if (G.nslot > 64) return false;
+    int need = small_threads<T, NR>(s, ls);
+    size_t off = 0;
+    for (int l = 0; l < ls; ++l) {
+        P.nx[l] = s.lnx[l];
+        P.ny[l] = s.lny[l];
+        P.rp[l] = 2 * ((s.lny[l] / 2 + CL_BLOCKS - 1) / CL_BLOCKS);
+        // level 0: a slab starts at a group of 32 units of the reductions
+        while (l == 0 && (long long)P.rp[0] * nx % (32 * G.unit) != 0) P.rp[0] += 2;
+        P.goff[l] = s.loff[l];
+        P.off[l] = (int)off;
+        off += ClMem<T, NR>::bytes(P.nx[l], P.rp[l]);
+        need = std::max(need, Blk<T, NR>::units(P.nx[l], P.rp[l]));
+        if (need > CL_THREADS || off > SMEM_MAX) return false;
+    }
+    threads = need > CL_THREADS / 2 ? CL_THREADS : CL_THREADS / 2;
+    P.soff = (int)off;
+    off += (SmallMem<T, NR>::bytes(P.S) + 127) & ~size_t(127);
+    auto take = [&](size_t bytes) {
+        const int o = (int)off;
+        off += (bytes + 127) & ~size_t(127);
+        return o;
+    };
+    G.tx = (nx + TX - 1) / TX;
+    G.nt = G.tx * ((ny + TY - 1) / TY);
+    if (G.nt > 64) return false;
+    G.tslots = (G.nt + CL_BLOCKS - 1) / CL_BLOCKS;
+    G.p_off = take(sizeof(T) * NR * ClMem<T, NR>::xn(nx, P.rp[0]));
+    G.x_off = take(sizeof(T) * NR * Blk<T, NR>::CELLS * threads);
+    // (these are cleared by the kernel as one range)
+    G.pstride = (P.rp[0] * nx / G.unit / 32 + 1) * CG_GRP;
+    G.prod_off = take(sizeof(double) * NR * G.pstride);
+    G.w_off = take(sizeof(double) * 2 * NR * G.ngrp);
+    G.tb_off = take(sizeof(T) * G.tslots * NR * 256);
+    G.tw_off = take(sizeof(T) * G.tslots * NR * 16);
+    G.ts_off = take(sizeof(double) * NR * 64);
+    smem = off;
+    return smem <= SMEM_MAX;
+}
+template <typename T, int NR>
+static void launch_cg(Solver& s, const CgPlan& G, int threads, size_t smem, const T* r, T* x, cudaStream_t stm) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(CL_BLOCKS);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stm;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = CL_BLOCKS;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_cg_cluster<T, NR>, G, (const T*)PT<T>::diag(s), (const T*)id_of<T>(s),
+                       (const T*)PT<T>::wl(s), (const T*)PT<T>::wb(s), (const T*)PT<T>::inv(s), r, x, s.st);
 }
 
 // blocks of a persistent (TMA-staged) tile launch: one per tile, at most as many as are resident
@@ -3893,6 +4414,16 @@ static void solve_fp64(Solver& s, const double* b, double* x, double rtol, int m
     int N = s.nx * s.ny;
     Lev<double> L0 = lev<double>(s, 0);
     double* z = s.d_x;   // level-0 slot of the per-level x is z
+    CgPlan G;
+    int cthreads = 0;
+    size_t csmem = 0;
+    if (cg_plan<double, NR>(s, G, cthreads, csmem)) {   // the whole solve in one launch
+        k_init64<NR><<<dim3(lblocks(N, s.nz), 1, s.nz), RB, 0, stm>>>(L0, b, x, s.d_r, s.st, s.partial, s.tickets,
+                                                                      rtol * rtol, max_iter, 0, 0, nblocks(N));
+        launch_cg<double, NR>(s, G, cthreads, csmem, s.d_r, x, stm);
+        s.launches += 2;
+        return;
+    }
     if (s.use_graph) {
         cudaGraph_t g;
         cudaGraphConditionalHandle h = make_handle(stm, &g);
@@ -4013,16 +4544,21 @@ static void solve_mixed(Solver& s, const double* cd, const double* dd, const dou
     int PG = 0;
     size_t psmem = 0;
     bool persist = persist_plan<NR>(s, PC, PS, PG, psmem);
+    CgPlan G;
+    int cthreads = 0;
+    size_t csmem = 0;
+    const bool whole = !persist && cg_plan<float, NR>(s, G, cthreads, csmem);   // each inner solve in one launch
     unsigned* pbar = persist ? s.tickets + 8 : nullptr;
     if (s.use_graph) {
         cudaGraph_t g;
         cudaGraphConditionalHandle ho = make_handle(stm, &g);
         cudaStream_t obs = begin_while(stm, s.aux[0], ho);
         int mode = s.nz > 1 ? 2 : 1;
-        if (persist) {
+        if (persist || whole) {
             k_ir_residual<NR><<<dim3(lb, 1, s.nz), RB, 0, obs>>>(L64, b, x, s.f_r, s.f_e, s.st, s.partial,
                                                                  s.tickets + 5, ho, ho, mode, 0, pbar, vb);
-            launch_persist<NR>(s, PC, PS, PG, psmem, obs);
+            if (persist) launch_persist<NR>(s, PC, PS, PG, psmem, obs);
+            else launch_cg<float, NR>(s, G, cthreads, csmem, s.f_r, s.f_e, obs);
         } else {
             cudaGraph_t og;
             cudaGraphConditionalHandle hi = make_handle(obs, &og);
@@ -4045,6 +4581,9 @@ static void solve_mixed(Solver& s, const double* cd, const double* dd, const dou
         if (s.st_host[s.slot].odone) break;
         if (persist) {
             launch_persist<NR>(s, PC, PS, PG, psmem, stm);
+        } else if (whole) {
+            launch_cg<float, NR>(s, G, cthreads, csmem, s.f_r, s.f_e, stm);
+            ++s.launches;
         } else {
             for (int it = 0; it < max_iter && !s.st_host[s.slot].done; ++it) {
                 cg_body<float, NR>(s, s.f_e, s.f_r, z, s.f_p, s.f_q, s.st, 0, 0, stm);
@@ -4082,7 +4621,29 @@ bool Solver::set_schedule(int small_max, double inner) {
     return true;
 }
 
-int Solver::body_size(int precision) const { return 2 * (precision == 0 ? nbig_d : nbig_f) + 1 + 2; }
+template <typename T, int NR>
+static int loop_kernels(Solver& s, bool alone, bool* whole) {
+    const int nb = nbig_of<T>(s);
+    *whole = false;
+    if (alone) {
+        CgPlan G;
+        ClPlan P;
+        int t = 0;
+        size_t m = 0;
+        if (cg_plan<T, NR>(s, G, t, m)) {
+            *whole = true;
+            return 0;
+        }
+        int l0 = cluster_plan<T, NR>(s, P, t, m);
+        if (l0 == nb) l0 = coarse_start<T, NR>(s);
+        return 2 * l0 + 1 + 2;
+    }
+    return 2 * nb + 1 + 2;
+}
+int Solver::body_size(int precision, int nr, bool alone, bool* whole) {
+    if (precision == 0) return nr == 1 ? loop_kernels<double, 1>(*this, alone, whole) : loop_kernels<double, 2>(*this, alone, whole);
+    return nr == 1 ? loop_kernels<float, 1>(*this, alone, whole) : loop_kernels<float, 2>(*this, alone, whole);
+}
 
 bool Solver::supported(int nx, int ny) {
     Solver s;

@@ -93,6 +93,7 @@ struct Solver {
     bool tma_ready = false;
     int use_tma = 1;       // 0: the tile kernels load their regions with plain loads
     int use_coop = 1;      // 0: no cooperative launch for the coarse part of the V-cycle
+    int use_cgc = 1;       // 0: no whole solve in one cluster launch (its smoothers cannot be timed)
     int barrier_spin = 0;  // polls of the cooperative launch's grid barrier before it gives up (0: 2^22)
     // batched launches: this solver drives nz instances whose arenas lie zs bytes apart (the
     // solvers of instances 1..nz-1 are bound to their own arenas, read only for statistics)
@@ -123,7 +124,9 @@ struct Solver {
     void fetch_states(cudaStream_t st);
     SolveResult result_from_host(int slot, int precision) const;
     static bool supported(int nx, int ny);
-    int body_size(int precision) const;   // kernels of one CG iteration (V-cycle + apply + update)
+    // kernels of one CG iteration of an nr-right-hand-side solve (V-cycle + apply + update); alone: not
+    // in a batch; *whole: the solve (FP64) or each inner solve (mixed) is one launch instead (then 0)
+    int body_size(int precision, int nr, bool alone, bool* whole);
 };
 
 }  // namespace ebit
