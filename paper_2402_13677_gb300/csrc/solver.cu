@@ -308,10 +308,14 @@ __global__ void k_cond_reset(cudaGraphConditionalHandle h0, cudaGraphConditional
 // weights, D) in registers; only x lives in shared memory, split by colour.  The region starts
 // at an even global cell (tile origins are multiples of TX, TY and the halos are even), so
 // region cell (rx, ry) has colour c = (rx + ry) & 1, known at compile time for each of a
-// thread's cells, and sits in column k = rx >> 1 of row ry of colour c's array (HX = SX / 2
-// columns).  A colour-c cell with
-// e = rx & 1 finds its left / right neighbours (colour 1 - c) in columns k - 1 + e / k + e of
-// its row and its lower / upper neighbours in column k of rows ry -+ 1.
+// thread's cells.  Colour c's array holds the even rows' cells, then the odd rows', each in thread
+// order: cell (r, c) of thread t is entry r TH + t, so a warp's accesses are consecutive words (one
+// row of columns after another in the array gave 2.5-way bank conflicts where a warp spans two row
+// pairs; with this layout and the paired loads of tile_load_cells k_pre / k_post of 1024x2048 cells take
+// 17.1 / 23.4 us, 20.3 / 25.5 before; bound: issue slots and the barriers between half-sweeps).  A
+// colour-c cell with e = rx & 1 finds its left / right neighbours (colour 1 - c) at
+// threads t - 1 + e / t + e of its row r, its lower / upper ones at row 1 - r of threads t - HX / t
+// (r = 0) or t / t + HX (r = 1).
 template <typename T, int NR, int H>
 struct Region {
     static constexpr int SX = TX + 2 * H, SY = TY + 2 * H, HX = SX / 2, NC = SY * HX;
@@ -320,6 +324,7 @@ struct Region {
     T* x0;   // x of colour 0 (NR per cell), then colour 1
     __device__ Region(unsigned char* base) { x0 = (T*)base; }
     __device__ T* x(int c) const { return x0 + c * (NR * NC); }
+    __device__ static int at(int r, int t) { return r * THREADS + t; }
     static constexpr size_t BYTES = (size_t)2 * NC * NR * sizeof(T);
     __host__ __device__ static constexpr size_t bytes() { return BYTES; }
 };
@@ -490,54 +495,82 @@ struct Cells {
     T x[2][2][NR];
 };
 
+// n consecutive elements (8 or a multiple of 16 bytes, aligned to 8 or 16) from shared memory
+template <int N, typename T>
+__device__ inline void load_row(const T* s, T* o) {
+    constexpr int W = N * sizeof(T) > 16 ? 16 / (int)sizeof(T) : N;
+    static_assert(N % W == 0, "whole words");
+#pragma unroll
+    for (int q = 0; q < N; q += W) {
+        const Vec<T, W> v = *reinterpret_cast<const Vec<T, W>*>(s + q);
+#pragma unroll
+        for (int w = 0; w < W; ++w) o[q + w] = v.v[w];
+    }
+}
+
 // load the thread's cells (coefficients to registers, x to shared memory: for pre-smoothing
 // the result of the first colour-0 half-sweep from x = 0, for post-smoothing xin + the
 // prolongated coarse x); cells outside the domain get D = 1, zero weights, b = x = 0, so
-// sweeps leave them 0
-template <typename T, int NR, int H, bool POST, bool CHECK>
+// sweeps leave them 0.  Staged: the two cells of a row are adjacent in the boxes, one 8 or 16 byte
+// load per operand
+template <typename T, int NR, int H, bool POST, bool STAGED, bool CHECK>
 __device__ inline void tile_load_cells(Region<T, NR, H>& R, Cells<T, NR>& C, int k, int ry0, const Lev<T>& L,
                                        const T* __restrict__ b, const T* __restrict__ xin, const T* __restrict__ xc,
                                        int cnx, int gx0, int gy0, const unsigned char* stage) {
-    constexpr int HX = Region<T, NR, H>::HX;
+    using Rg = Region<T, NR, H>;
     using Sg = Stage<T, NR, H, POST>;
     static_assert(H % 2 == 0 && TX % 2 == 0 && TY % 2 == 0, "regions must start at an even cell");
+    static_assert(Sg::OXS % 2 == 0 && Sg::OXV % 2 == 0, "a cell pair is aligned in its box");
+    constexpr bool ID = sizeof(T) == 8;
+    T dp[2][2], idp[2][2], wlp[2][3], wbp[3][2], bp[2][2 * NR], xp[2][2 * NR];   // [row][column]
+    if constexpr (STAGED) {
+        // from the TMA boxes (zeros outside the grid)
+        const T* sd = reinterpret_cast<const T*>(stage + Sg::OFF_D);
+        const T* swl = reinterpret_cast<const T*>(stage + Sg::OFF_WL);
+        const T* swb = reinterpret_cast<const T*>(stage + Sg::OFF_WB);
+        const T* sb = reinterpret_cast<const T*>(stage + Sg::OFF_B);
+        const int q0 = ry0 * Sg::BWS + 2 * k + Sg::OXS;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int qs = q0 + r * Sg::BWS, qv = ((ry0 + r) * Sg::BWV + 2 * k + Sg::OXV) * NR;
+            load_row<2>(sd + qs, dp[r]);
+            if constexpr (Sg::ID_BOX) load_row<2>(reinterpret_cast<const T*>(stage + Sg::OFF_ID) + qs, idp[r]);
+            load_row<2>(swl + qs, wlp[r]);
+            wlp[r][2] = swl[qs + 2];
+            load_row<2>(swb + qs, wbp[r]);
+            load_row<2 * NR>(sb + qv, bp[r]);
+            if constexpr (POST) load_row<2 * NR>(reinterpret_cast<const T*>(stage + Sg::OFF_XIN) + qv, xp[r]);
+        }
+        load_row<2>(swb + q0 + 2 * Sg::BWS, wbp[2]);
+        if constexpr (POST) {   // the block's four cells have one coarse parent
+            T cv[NR];
+            load_row<NR>(reinterpret_cast<const T*>(stage + Sg::OFF_XC) + ((ry0 >> 1) * Sg::BWC + k + Sg::OXC) * NR, cv);
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int q = 0; q < 2 * NR; ++q) xp[r][q] += cv[q % NR];
+        }
+    }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        int ry = ry0 + r;
-        int gj = gy0 + ry;
+        const int gj = gy0 + ry0 + r;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            int rx = 2 * k + e;
-            int gi = gx0 + rx;
+            const int gi = gx0 + 2 * k + e;
             bool in = !CHECK || (gj >= 0 && gj < L.ny && gi >= 0 && gi < L.nx);
             Vec<T, NR> bv, xv;
             T dv, wlv, wbv, wrv, wtv, idv = T(1);   // FP64: idv loaded (and D only where a residual follows)
-            constexpr bool ID = sizeof(T) == 8;
-            if (stage) {
-                // from the TMA boxes (zeros outside the grid)
-                const T* sd = reinterpret_cast<const T*>(stage + Sg::OFF_D);
-                const T* swl = reinterpret_cast<const T*>(stage + Sg::OFF_WL);
-                const T* swb = reinterpret_cast<const T*>(stage + Sg::OFF_WB);
-                const T* sb = reinterpret_cast<const T*>(stage + Sg::OFF_B);
-                int qs = ry * Sg::BWS + rx + Sg::OXS, qv = (ry * Sg::BWV + rx + Sg::OXV) * NR;
-                dv = sd[qs];
-                if (ID) idv = POST ? dv : reinterpret_cast<const T*>(stage + Sg::OFF_ID)[qs];
-                wlv = swl[qs];
-                wbv = swb[qs];
-                wrv = swl[qs + 1];
-                wtv = swb[qs + Sg::BWS];
+            if constexpr (STAGED) {
+                dv = dp[r][e];
+                if (ID) idv = Sg::ID_BOX ? idp[r][e] : dv;
+                wlv = wlp[r][e];
+                wbv = wbp[r][e];
+                wrv = wlp[r][e + 1];
+                wtv = wbp[r + 1][e];
 #pragma unroll
-                for (int k2 = 0; k2 < NR; ++k2) bv.v[k2] = sb[qv + k2];
-                if (POST) {
-                    const T* sx = reinterpret_cast<const T*>(stage + Sg::OFF_XIN);
-                    const T* sc = reinterpret_cast<const T*>(stage + Sg::OFF_XC);
-                    int cx = (gi >> 1) - ((gx0 >> 1) - Sg::OXC), cy = (gj >> 1) - (gy0 >> 1);
-                    int qc = (cy * Sg::BWC + cx) * NR;
-#pragma unroll
-                    for (int k2 = 0; k2 < NR; ++k2) xv.v[k2] = sx[qv + k2] + sc[qc + k2];
-                } else {
-#pragma unroll
-                    for (int k2 = 0; k2 < NR; ++k2) xv.v[k2] = T(0);
+                for (int k2 = 0; k2 < NR; ++k2) {
+                    bv.v[k2] = bp[r][e * NR + k2];
+                    xv.v[k2] = POST ? xp[r][e * NR + k2] : T(0);
                 }
             } else {
                 // unconditional loads (clamped, then masked): all of them can be in flight at once
@@ -592,7 +625,7 @@ __device__ inline void tile_load_cells(Region<T, NR, H>& R, Cells<T, NR>& C, int
 #pragma unroll
                 for (int k2 = 0; k2 < NR; ++k2) xv.v[k2] = bv.v[k2] * idv;
             }
-            T* xd = R.x(cc) + (ry * HX + k) * NR;
+            T* xd = R.x(cc) + Rg::at(r, threadIdx.x) * NR;
 #pragma unroll
             for (int k2 = 0; k2 < NR; ++k2) {
                 xd[k2] = xv.v[k2];
@@ -604,15 +637,15 @@ __device__ inline void tile_load_cells(Region<T, NR, H>& R, Cells<T, NR>& C, int
 
 // A region wholly inside the grid, with the right and upper faces of its last cells too (all
 // but the tiles along the grid's edges), needs no range tests or masks
-template <typename T, int NR, int H, bool POST>
+template <typename T, int NR, int H, bool POST, bool STAGED>
 __device__ inline void tile_load(Region<T, NR, H>& R, Cells<T, NR>& C, int k, int ry0, const Lev<T>& L,
                                  const T* __restrict__ b, const T* __restrict__ xin, const T* __restrict__ xc,
                                  int cnx, int gx0, int gy0, const unsigned char* stage) {
     constexpr int SX = Region<T, NR, H>::SX, SY = Region<T, NR, H>::SY;
     if (gx0 >= 0 && gy0 >= 0 && gx0 + SX < L.nx && gy0 + SY < L.ny)
-        tile_load_cells<T, NR, H, POST, false>(R, C, k, ry0, L, b, xin, xc, cnx, gx0, gy0, stage);
+        tile_load_cells<T, NR, H, POST, STAGED, false>(R, C, k, ry0, L, b, xin, xc, cnx, gx0, gy0, stage);
     else
-        tile_load_cells<T, NR, H, POST, true>(R, C, k, ry0, L, b, xin, xc, cnx, gx0, gy0, stage);
+        tile_load_cells<T, NR, H, POST, STAGED, true>(R, C, k, ry0, L, b, xin, xc, cnx, gx0, gy0, stage);
 }
 
 // A thread's place in a tile region, the same for every tile of a launch (computed once per
@@ -658,7 +691,6 @@ __device__ inline void tile_sweep(Region<T, NR, H>& R, Cells<T, NR>& C, const Ti
     static_assert(COLOR == (S & 1), "half-sweep S has colour S & 1");
     using Rg = Region<T, NR, H>;
     constexpr int HX = Rg::HX;
-    const int k = threadIdx.x % HX, ry0 = 2 * (threadIdx.x / HX);
     if (tt.act()) {
         const T* xo = R.x(1 - COLOR);
         T acc[2][NR];
@@ -666,18 +698,18 @@ __device__ inline void tile_sweep(Region<T, NR, H>& R, Cells<T, NR>& C, const Ti
         int qs[2];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            int ry = ry0 + r;
             const int e = COLOR ^ r;
             ok[r] = tt.sweeps(S, r);
-            int q = ok[r] ? ry * HX + k : HX + 1;   // a harmless in-range slot otherwise
+            const int t = ok[r] ? threadIdx.x : HX + 1;   // a harmless in-range slot otherwise
+            const int q = Rg::at(r, t), qv = r == 1 ? Rg::at(0, t + HX) : Rg::at(1, t - HX);
             qs[r] = q;
 #pragma unroll
             for (int k2 = 0; k2 < NR; ++k2) {
                 const T own_h = C.x[r][1 - COLOR][k2], own_v = C.x[1 - r][1 - COLOR][k2];
                 T xl = e == 1 ? own_h : xo[(q - 1) * NR + k2];
                 T xrt = e == 0 ? own_h : xo[(q + 1) * NR + k2];
-                T xd = r == 1 ? own_v : xo[(q - HX) * NR + k2];
-                T xu = r == 0 ? own_v : xo[(q + HX) * NR + k2];
+                T xd = r == 1 ? own_v : xo[qv * NR + k2];
+                T xu = r == 0 ? own_v : xo[qv * NR + k2];
                 acc[r][k2] = (C.b[r][COLOR][k2] + C.wl[r][COLOR] * xl + C.wr[r][COLOR] * xrt +
                               C.wb[r][COLOR] * xd + C.wt[r][COLOR] * xu) *
                              C.id[r][COLOR];
@@ -696,7 +728,7 @@ __device__ inline void tile_sweep(Region<T, NR, H>& R, Cells<T, NR>& C, const Ti
     __syncthreads();
 }
 
-// the thread's core cells (inside the TX x TY tile and the domain): f(r, c, rx, ry, q, gi, gj)
+// the thread's core cells (inside the TX x TY tile and the domain): f(r, c, gi, gj)
 template <typename T, int NR, int H, class Fn>
 __device__ inline void tile_core_cells(const Cells<T, NR>& C, const TileThread& tt, int gx0, int gy0,
                                        const Lev<T>& L, Fn&& f) {
@@ -709,7 +741,7 @@ __device__ inline void tile_core_cells(const Cells<T, NR>& C, const TileThread& 
         for (int c = 0; c < 2; ++c) {
             int rx = 2 * k + (c ^ r);
             int gi = gx0 + rx, gj = gy0 + ry;
-            if (tt.core(r, c) && gi < L.nx && gj < L.ny) f(r, c, rx, ry, ry * HX + k, gi, gj);
+            if (tt.core(r, c) && gi < L.nx && gj < L.ny) f(r, c, gi, gj);
         }
     }
 }
@@ -719,9 +751,9 @@ struct NoOp {
 };
 
 // pre-smoothing of tile (bx, by): x = S^nu(0; b) on the tile (red-black order), coarse
-// b = R (b - A x); smem holds the region (stage: its TMA boxes, already landed, or null);
+// b = R (b - A x); smem holds the region (STAGED: `stage` its TMA boxes, already landed);
 // after_load() runs in every thread once the boxes have been read
-template <typename T, int NR, class AfterLoad = NoOp>
+template <typename T, int NR, bool STAGED = false, class AfterLoad = NoOp>
 __device__ inline void pre_tile(const Lev<T>& L, const T* __restrict__ b, T* __restrict__ x, T* __restrict__ bc,
                                 int bx, int by, unsigned char* smem, const unsigned char* stage,
                                 const TileThread& tt, AfterLoad after_load = AfterLoad()) {
@@ -734,7 +766,7 @@ __device__ inline void pre_tile(const Lev<T>& L, const T* __restrict__ b, T* __r
     const bool act = tt.act();
     const int k = threadIdx.x % HX, ry0 = 2 * (threadIdx.x / HX);
     Cells<T, NR> C;
-    if (act) tile_load<T, NR, H, false>(R, C, k, ry0, L, b, nullptr, nullptr, 0, gx0, gy0, stage);
+    if (act) tile_load<T, NR, H, false, STAGED>(R, C, k, ry0, L, b, nullptr, nullptr, 0, gx0, gy0, stage);
     __syncthreads();
     after_load();
     // the first colour-0 half-sweep (from x = 0) was done by tile_load
@@ -745,9 +777,10 @@ __device__ inline void pre_tile(const Lev<T>& L, const T* __restrict__ b, T* __r
     // column 2k + e)
     T res[2][2][NR];
     if (act)
-        tile_core_cells<T, NR, H>(C, tt, gx0, gy0, L, [&](int r, int c, int rx, int ry, int q, int gi, int gj) {
+        tile_core_cells<T, NR, H>(C, tt, gx0, gy0, L, [&](int r, int c, int gi, int gj) {
             const T* xo = R.x(1 - c);
-            const int e = c ^ r;   // rx = 2k + e
+            const int e = c ^ r;   // column 2k + e
+            const int q = Rg::at(r, threadIdx.x), qv = r == 1 ? Rg::at(0, threadIdx.x + HX) : Rg::at(1, threadIdx.x - HX);
             Vec<T, NR> xv;
 #pragma unroll
             for (int k2 = 0; k2 < NR; ++k2) {
@@ -756,8 +789,8 @@ __device__ inline void pre_tile(const Lev<T>& L, const T* __restrict__ b, T* __r
                 const T own_h = C.x[r][1 - c][k2], own_v = C.x[1 - r][1 - c][k2];
                 T xl = e == 1 ? own_h : xo[(q - 1) * NR + k2];
                 T xrt = e == 0 ? own_h : xo[(q + 1) * NR + k2];
-                T xd = r == 1 ? own_v : xo[(q - HX) * NR + k2];
-                T xu = r == 0 ? own_v : xo[(q + HX) * NR + k2];
+                T xd = r == 1 ? own_v : xo[qv * NR + k2];
+                T xu = r == 0 ? own_v : xo[qv * NR + k2];
                 res[r][e][k2] = cell_residual(C.b[r][c][k2], C.d[r][c], C.wl[r][c], C.wr[r][c], C.wb[r][c],
                                               C.wt[r][c], x0v, xl, xrt, xd, xu);
             }
@@ -816,7 +849,7 @@ k_pre(Lev<T> L, const T* __restrict__ b, T* __restrict__ x, T* __restrict__ bc, 
         int tx = (L.nx + TX - 1) / TX, nt = tx * ((L.ny + TY - 1) / TY);
         const TileThread tt = tile_thread<H>();
         staged_tiles<T, NR, H, false>(stage, maps, tx, nt, st, [&](int, int bx, int by, auto after_load) {
-            pre_tile<T, NR>(L, b, x, bc, bx, by, smem, stage, tt, after_load);
+            pre_tile<T, NR, true>(L, b, x, bc, bx, by, smem, stage, tt, after_load);
         });
     } else {
         pre_tile<T, NR>(L, b, x, bc, blockIdx.x, blockIdx.y, smem, nullptr, tile_thread<H>());
@@ -827,7 +860,7 @@ k_pre(Lev<T> L, const T* __restrict__ b, T* __restrict__ x, T* __restrict__ bc, 
 
 // post-smoothing of tile (bx, by): x = xin + P xc, then black-red sweeps; returns the tile's
 // part of r.z (each right-hand side) when DOT; after_load() as for pre_tile
-template <typename T, int NR, bool DOT, class AfterLoad = NoOp>
+template <typename T, int NR, bool DOT, bool STAGED = false, class AfterLoad = NoOp>
 __device__ inline Vec<T, 2> post_tile(const Lev<T>& L, const T* __restrict__ b, const T* __restrict__ xin,
                                     T* __restrict__ x, const T* __restrict__ xc, int bx, int by, unsigned char* smem,
                                     const unsigned char* stage, const TileThread& tt,
@@ -840,8 +873,8 @@ __device__ inline Vec<T, 2> post_tile(const Lev<T>& L, const T* __restrict__ b, 
     const bool act = tt.act();
     Cells<T, NR> C;
     if (act)
-        tile_load<T, NR, H, true>(R, C, threadIdx.x % HX, 2 * (threadIdx.x / HX), L, b, xin, xc, L.nx / 2, gx0, gy0,
-                                  stage);
+        tile_load<T, NR, H, true, STAGED>(R, C, threadIdx.x % HX, 2 * (threadIdx.x / HX), L, b, xin, xc, L.nx / 2, gx0, gy0,
+                                          stage);
     __syncthreads();
     after_load();
     tile_sweep<T, NR, H, 1, 1>(R, C, tt);
@@ -852,7 +885,7 @@ __device__ inline Vec<T, 2> post_tile(const Lev<T>& L, const T* __restrict__ b, 
     Vec<T, 2> dot;
     dot.v[0] = dot.v[1] = T(0);
     if (act)
-        tile_core_cells<T, NR, H>(C, tt, gx0, gy0, L, [&](int r, int c, int rx, int ry, int q, int gi, int gj) {
+        tile_core_cells<T, NR, H>(C, tt, gx0, gy0, L, [&](int r, int c, int gi, int gj) {
             Vec<T, NR> xv;
 #pragma unroll
             for (int k2 = 0; k2 < NR; ++k2) {
@@ -906,7 +939,7 @@ k_post(Lev<T> L, const T* __restrict__ b, const T* __restrict__ xin, T* __restri
         // r.z: one slot per tile, summed in tile order as with one block per tile
         const TileThread tt = tile_thread<H>();
         staged_tiles<T, NR, H, true>(stage, maps, tx, nt, st, [&](int t, int bx, int by, auto after_load) {
-            Vec<T, 2> d = post_tile<T, NR, DOT>(L, b, xin, x, xc, bx, by, smem, stage, tt, after_load);
+            Vec<T, 2> d = post_tile<T, NR, DOT, true>(L, b, xin, x, xc, bx, by, smem, stage, tt, after_load);
             if (DOT) block_partial_t<T, NR>(d.v, partial, nt, t);
         });
         nslot = nt;
