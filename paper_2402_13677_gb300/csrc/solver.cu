@@ -3539,13 +3539,36 @@ __global__ void __launch_bounds__(256) k_ir_init(int N, long long zs, const doub
 }
 
 // refinement sweep: r64 = b - A64 x, outer test, r32 = r64, e = 0, inner state reset
-template <int NR>
-__global__ void __launch_bounds__(256) k_ir_residual(Lev<double> L, const double* __restrict__ b,
+// Bound: the FP64 pipe (19 cycles a warp instruction and SM).  A thread walks R rows of W cells: a
+// difference of x across a face serves both its cells (the other one's is its exact negative), 8.6
+// FP64 instructions a cell where one cell at a time needs 10, and the vertical ones need no second
+// load of x.  W = 2: four cells a row save 0.4 more but leave 16 warps an SM, the pipe half idle
+// (1024x2048, two right-hand sides: 112 us); loading a row ahead likewise (110).  Measured on 4096^2
+// films, one -> two right-hand sides: 331 and 652 us before, a step 22.0 -> 21.0 ms; 512^2 16.7 and 25.6
+// -> 15.6 and 22.4 us.
+// n consecutive values of a row (one, or an even number at a 16-byte boundary)
+template <int n>
+__device__ __forceinline__ void row_ld(const double* __restrict__ p, double* o) {
+    if constexpr (n == 1) {
+        o[0] = p[0];
+    } else {
+#pragma unroll
+        for (int q = 0; q < n; q += 2) {
+            const double2 v = *reinterpret_cast<const double2*>(p + q);
+            o[q] = v.x;
+            o[q + 1] = v.y;
+        }
+    }
+}
+
+constexpr int IR_THREADS = 128;
+template <int NR, int W>
+__global__ void __launch_bounds__(IR_THREADS) k_ir_residual(Lev<double> L, const double* __restrict__ b,
                                                       const double* __restrict__ x, float* __restrict__ r32,
                                                       float* __restrict__ e32, SolveState* st, double* partial,
                                                       unsigned* ticket, cudaGraphConditionalHandle ho,
                                                       cudaGraphConditionalHandle hi, int use_h, int set_hi,
-                                                      unsigned* coop_bar, int vb) {
+                                                      unsigned* coop_bar, int R) {
     // the whole-solve cooperative launch that follows counts its barrier arrivals from 0 (its
     // previous launch has completed: stream order)
     if (coop_bar && blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.x == 0) *coop_bar = 0u;
@@ -3576,48 +3599,100 @@ __global__ void __launch_bounds__(256) k_ir_residual(Lev<double> L, const double
     for (int k = 0; k < NR; ++k) {
         ksc[k] = (int)((__double_as_longlong(sc[k]) >> 52) & 0x7ff) - 1023;
     }
-    const Vec<double, NR>* X = reinterpret_cast<const Vec<double, NR>*>(x);
-    const Vec<double, NR>* B = reinterpret_cast<const Vec<double, NR>*>(b);
-    for (int v = blockIdx.x; v < vb; v += gridDim.x) {
-        DotAcc<float, NR> acc;
-        auto cell = [&](int c, int i, int j) {
-            Vec<double, NR> xv = X[c], bv = B[c], s;   // s = (A x)_i in flux form
-            double dg = L.diag[c];
+    const int nq = L.nx / W, u = blockIdx.x * IR_THREADS + threadIdx.x;
+    const int m = u % nq, j0 = u / nq * R, j1 = min(j0 + R, L.ny);
+    DotAcc<float, NR> acc;
+    if (j0 < L.ny) {
+        constexpr int V = W * NR;
+        const int c0 = j0 * L.nx + m * W;
+        const bool lft = m > 0, rgt = m < nq - 1;
+        // xc: the row's x; dv: its differences to the row below, dv = x_below - x (the sign of the
+        // row below's own term); wb: the weights of the faces between
+        double xc[V], dv[V], wb[W];
+        row_ld<V>(x + (size_t)c0 * NR, xc);
 #pragma unroll
-            for (int k = 0; k < NR; ++k) s.v[k] = dg * xv.v[k];
-            if (i > 0) { double w = L.wl[c]; for (int k = 0; k < NR; ++k) s.v[k] += w * (xv.v[k] - X[c - 1].v[k]); }
-            if (i < L.nx - 1) {
-                double w = L.wl[c + 1];
-                for (int k = 0; k < NR; ++k)
-                    s.v[k] += w * (xv.v[k] - X[c + 1].v[k]);
+        for (int q = 0; q < W; ++q) wb[q] = 0.0;
+#pragma unroll
+        for (int q = 0; q < V; ++q) dv[q] = 0.0;
+        if (j0 > 0) {
+            double xd[V];
+            row_ld<V>(x + (size_t)(c0 - L.nx) * NR, xd);
+            row_ld<W>(L.wb + c0, wb);
+#pragma unroll
+            for (int q = 0; q < V; ++q) dv[q] = xd[q] - xc[q];
+        }
+#pragma unroll 2
+        for (int j = j0, c = c0; j < j1; ++j, c += L.nx) {
+            double xu[V], wt[W], wl[W + 1], dg[W], bv[V], xl[NR], xr[NR];
+            const bool up = j + 1 < L.ny;
+#pragma unroll
+            for (int q = 0; q < W; ++q) wt[q] = 0.0;
+#pragma unroll
+            for (int q = 0; q < V; ++q) xu[q] = xc[q];
+            if (up) {
+                row_ld<V>(x + (size_t)(c + L.nx) * NR, xu);
+                row_ld<W>(L.wb + c + L.nx, wt);
             }
-            if (j > 0) { double w = L.wb[c]; for (int k = 0; k < NR; ++k) s.v[k] += w * (xv.v[k] - X[c - L.nx].v[k]); }
-            if (j < L.ny - 1) {
-                double w = L.wb[c + L.nx];
-                for (int k = 0; k < NR; ++k)
-                    s.v[k] += w * (xv.v[k] - X[c + L.nx].v[k]);
-            }
-            Vec<float, NR> rf, ez;
+            row_ld<W>(L.diag + c, dg);
+            row_ld<W>(L.wl + c, wl);
+            row_ld<V>(b + (size_t)c * NR, bv);
+            // the faces on the grid's sides: weight 0, difference 0
+            if (!lft) wl[0] = 0.0;
+            wl[W] = rgt ? L.wl[c + W] : 0.0;
 #pragma unroll
             for (int k = 0; k < NR; ++k) {
-                float f = d2f_rn2(bv.v[k] - s.v[k], ksc[k]);
-                rf.v[k] = f;
-                acc.add(k, f, f);
-                ez.v[k] = 0.0f;
+                xl[k] = lft ? x[(size_t)(c - 1) * NR + k] : xc[k];
+                xr[k] = rgt ? x[(size_t)(c + W) * NR + k] : xc[V - NR + k];
             }
-            reinterpret_cast<Vec<float, NR>*>(r32)[c] = rf;
-            reinterpret_cast<Vec<float, NR>*>(e32)[c] = ez;
-        };
-        CellWalk cw(L.nx, v, vb);
-        while (cw.c + (DOT_CHUNK - 1) * cw.stride < N) {
+            double s[V];   // A x in flux form
 #pragma unroll
-            for (int u = 0; u < DOT_CHUNK; ++u, cw.next()) cell(cw.c, cw.i, cw.j);
-            acc.flush();
+            for (int q = 0; q < V; ++q) s[q] = dg[q / NR] * xc[q];
+            double h[V + NR];
+#pragma unroll
+            for (int q = 0; q < V; ++q) h[q] = xc[q] - (q < NR ? xl[q] : xc[q - NR]);
+#pragma unroll
+            for (int k = 0; k < NR; ++k) h[V + k] = xr[k] - xc[V - NR + k];
+            alignas(16) float rf[V], ez[V];
+#pragma unroll
+            for (int q = 0; q < V; ++q) {
+                s[q] = fma(wl[q / NR], h[q], s[q]);
+                s[q] = fma(wl[q / NR + 1], -h[q + NR], s[q]);
+                s[q] = fma(wb[q / NR], -dv[q], s[q]);
+                dv[q] = xc[q] - xu[q];
+                s[q] = fma(wt[q / NR], dv[q], s[q]);
+                rf[q] = d2f_rn2(bv[q] - s[q], ksc[q % NR]);
+                acc.add(q % NR, rf[q], rf[q]);
+                ez[q] = 0.0f;
+                xc[q] = xu[q];
+            }
+#pragma unroll
+            for (int q = 0; q < W; ++q) wb[q] = wt[q];
+            using F = Vec<float, V % 4 == 0 ? 4 : V>;
+#pragma unroll
+            for (int q = 0; q < V; q += sizeof(F) / 4) {
+                *reinterpret_cast<F*>(r32 + (size_t)c * NR + q) = *reinterpret_cast<const F*>(rf + q);
+                *reinterpret_cast<F*>(e32 + (size_t)c * NR + q) = *reinterpret_cast<const F*>(ez + q);
+            }
         }
-        for (; cw.c < N; cw.next()) cell(cw.c, cw.i, cw.j);
         acc.flush();
-        block_partial<NR>(acc.tot, partial, vb, v);
     }
+    // the block's sum: over its warps lane by lane, then one warp's tree (a tree per warp would be a
+    // tenth of the kernel's FP64 instructions)
+    __shared__ double sh[NR][IR_THREADS];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) sh[k][threadIdx.x] = acc.tot[k];
+    __syncthreads();
+    const int vb = gridDim.x;
+    if (threadIdx.x < 32 * NR) {
+        const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        double a = sh[k][lane];
+#pragma unroll
+        for (int w = 1; w < IR_THREADS / 32; ++w) a += sh[k][lane + 32 * w];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+        if (lane == 0) partial[k * vb + blockIdx.x] = a;
+    }
+    __syncthreads();
     double tot[NR];
     if (last_block_total<NR>(partial, vb, ticket, tot)) {
         bool done = true;
@@ -4545,6 +4620,24 @@ static void launch_persist(Solver& s, const CoarsePlan<float>& C, const SmallPla
     if (!s.use_graph) ++s.launches;
 }
 
+// two cells of a row per thread where rows and arrays allow 16-byte accesses, else one; rows per
+// thread: eight (512 threads per SM from 2^20 cells on), two below (512^2: four take 5 % longer,
+// most SMs then have one block)
+template <int NR>
+static void launch_ir_residual(Solver& s, const Lev<double>& L, const double* b, const double* x,
+                               cudaGraphConditionalHandle ho, cudaGraphConditionalHandle hi, int mode, int set_hi,
+                               unsigned* bar, cudaStream_t stm) {
+    auto a16 = [](const void* p) { return ((uintptr_t)p & 15u) == 0; };
+    const bool pair = s.nx % 2 == 0 && s.zs % 16 == 0 && a16(b) && a16(x) && a16(L.diag) && a16(L.wl) && a16(L.wb) &&
+                      a16(s.f_r) && a16(s.f_e);
+    // (16 keep the one-cell form's blocks within the reduction's slots)
+    const int R = !pair ? 16 : (long long)s.nx * s.ny < (1 << 20) ? 2 : 8;
+    const long long units = (long long)(pair ? s.nx / 2 : s.nx) * ((s.ny + R - 1) / R);
+    const dim3 grid((unsigned)((units + IR_THREADS - 1) / IR_THREADS), 1, s.nz);
+    auto k = pair ? k_ir_residual<NR, 2> : k_ir_residual<NR, 1>;
+    k<<<grid, IR_THREADS, 0, stm>>>(L, b, x, s.f_r, s.f_e, s.st, s.partial, s.tickets + 5, ho, hi, mode, set_hi, bar, R);
+}
+
 template <int NR>
 static void solve_mixed(Solver& s, const double* cd, const double* dd, const double* wl, const double* wb,
                         const double* b, double* x, double rtol, int max_iter, cudaStream_t stm) {
@@ -4588,16 +4681,14 @@ static void solve_mixed(Solver& s, const double* cd, const double* dd, const dou
         cudaStream_t obs = begin_while(stm, s.aux[0], ho);
         int mode = s.nz > 1 ? 2 : 1;
         if (persist || whole) {
-            k_ir_residual<NR><<<dim3(lb, 1, s.nz), RB, 0, obs>>>(L64, b, x, s.f_r, s.f_e, s.st, s.partial,
-                                                                 s.tickets + 5, ho, ho, mode, 0, pbar, vb);
+            launch_ir_residual<NR>(s, L64, b, x, ho, ho, mode, 0, pbar, obs);
             if (persist) launch_persist<NR>(s, PC, PS, PG, psmem, obs);
             else launch_cg<float, NR>(s, G, cthreads, csmem, s.f_r, s.f_e, obs);
         } else {
             cudaGraph_t og;
             cudaGraphConditionalHandle hi = make_handle(obs, &og);
             if (mode == 2) k_cond_reset<<<1, 32, 0, obs>>>(ho, hi, 1);
-            k_ir_residual<NR><<<dim3(lb, 1, s.nz), RB, 0, obs>>>(L64, b, x, s.f_r, s.f_e, s.st, s.partial,
-                                                                 s.tickets + 5, ho, hi, mode, 1, nullptr, vb);
+            launch_ir_residual<NR>(s, L64, b, x, ho, hi, mode, 1, nullptr, obs);
             cudaStream_t ibs = begin_while(obs, s.aux[1], hi);
             cg_body<float, NR>(s, s.f_e, s.f_r, z, s.f_p, s.f_q, s.st, hi, mode, ibs);
             end_while(ibs);
@@ -4607,8 +4698,7 @@ static void solve_mixed(Solver& s, const double* cd, const double* dd, const dou
         return;
     }
     for (int o = 0; o <= max_outer; ++o) {
-        k_ir_residual<NR><<<dim3(lb, 1, s.nz), RB, 0, stm>>>(L64, b, x, s.f_r, s.f_e, s.st, s.partial,
-                                                             s.tickets + 5, 0, 0, 0, 0, pbar, vb);
+        launch_ir_residual<NR>(s, L64, b, x, 0, 0, 0, 0, pbar, stm);
         ++s.launches;
         poll(s, stm);
         if (s.st_host[s.slot].odone) break;
