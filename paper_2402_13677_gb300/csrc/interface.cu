@@ -812,12 +812,12 @@ __device__ double link_theta(const Grid& g, const uint16_t* cseg, const double* 
 //   b = cd T*_k + sum_cut lambda_k T_sat / theta + sum 2 lambda_k T_w,  x0 = T*_k;
 // axisymmetric: cd times the cell's radius, every face term times the radius of its face.
 template <bool AXI>
-__global__ void k_energy_operator(Grid g, Phys p, const uint8_t* __restrict__ flags,
+__global__ void __launch_bounds__(128) k_energy_operator(Grid g, Phys p, const uint8_t* __restrict__ flags,
                                   const uint16_t* __restrict__ cseg, const double* __restrict__ hpos,
                                   const double* __restrict__ vpos, const double* __restrict__ Ts_l,
                                   const double* __restrict__ Ts_v, double* __restrict__ cd,
                                   double* __restrict__ dd, double* __restrict__ wl, double* __restrict__ wb,
-                                  double* __restrict__ b, double* __restrict__ x0) {
+                                  double* __restrict__ b, double* __restrict__ x0, int rows) {
     zphys(g, p);
     const long long zo = zoff(g.zs);
     flags = zsh(flags, zo);
@@ -832,45 +832,63 @@ __global__ void k_energy_operator(Grid g, Phys p, const uint8_t* __restrict__ fl
     wb = zsh(wb, zo);
     b = zsh(b, zo);
     x0 = zsh(x0, zo);
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j0 = blockIdx.y * rows, j1 = min(j0 + rows, g.ny);
     if (i >= g.nx) return;
-    int c = cidx(g, i, j);
-    int k = flags[c] & F_CCOL;
-    double lam = k ? p.lam_l : p.lam_v;
-    double rc = k ? p.rho_l * p.cp_l : p.rho_v * p.cp_v;
     const double mc = rad_c<AXI>(g, i);
-    double coef = g.h * g.h * rc * p.inv_dt * mc;
-    double ts = k ? Ts_l[c] : Ts_v[c];
-    double dsum = 0.0, rhs = coef * ts;
+    // the two phases' coefficients, once for the thread's rows: the FP64 pipe bounded this kernel, with
+    // the boundary and cut links' instructions issued by every warp (4096^2: 453 -> 264 us)
+    const double coef_l = g.h * g.h * (p.rho_l * p.cp_l) * p.inv_dt * mc;
+    const double coef_v = g.h * g.h * (p.rho_v * p.cp_v) * p.inv_dt * mc;
+    const double lx_l = p.lam_l * rad_fx<AXI>(g, i), lx_v = p.lam_v * rad_fx<AXI>(g, i);
+    const double ly_l = p.lam_l * mc, ly_v = p.lam_v * mc;
     const int di[4] = {1, -1, 0, 0}, dj[4] = {0, 0, 1, -1};
     const int bside[4] = {1, 0, 3, 2};
-    for (int s = 0; s < 4; ++s) {
-        int ii = i + di[s], jj = j + dj[s];
-        // conductance of the face this link crosses
-        double lf = AXI ? lam * (s == 0 ? rad_fx<AXI>(g, i + 1) : (s == 1 ? rad_fx<AXI>(g, i) : mc)) : lam;
-        if (ii < 0 || ii >= g.nx || jj < 0 || jj >= g.ny) {
-            int bs = bside[s];
-            if (g.Tfix[bs]) {
-                dsum += 2.0 * lf;
-                rhs += 2.0 * lf * g.Tw[bs];
+#pragma unroll 2
+    for (int j = j0; j < j1; ++j) {
+        const int c = cidx(g, i, j);
+        const int k = flags[c] & F_CCOL;
+        // the neighbours' phases (its own beyond the grid)
+        int kn[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const int ii = i + di[s], jj = j + dj[s];
+            const bool in = ii >= 0 && ii < g.nx && jj >= 0 && jj < g.ny;
+            kn[s] = flags[in ? cidx(g, ii, jj) : c] & F_CCOL;
+        }
+        const double coef = k ? coef_l : coef_v;
+        const double ts = (k ? Ts_l : Ts_v)[c];
+        double dsum = 0.0, rhs = coef * ts;
+        const bool edge = i == 0 || j == 0 || i == g.nx - 1 || j == g.ny - 1;
+        if (edge || kn[0] != k || kn[1] != k || kn[2] != k || kn[3] != k) {
+            double lam = k ? p.lam_l : p.lam_v;
+            asm volatile("" : "+d"(lam));   // (few warps come here: no FP64 instruction moved out of the branch)
+            for (int s = 0; s < 4; ++s) {
+                const int ii = i + di[s], jj = j + dj[s];
+                // conductance of the face this link crosses
+                const double lf = AXI ? lam * (s == 0 ? rad_fx<AXI>(g, i + 1) : (s == 1 ? rad_fx<AXI>(g, i) : mc)) : lam;
+                if (ii < 0 || ii >= g.nx || jj < 0 || jj >= g.ny) {
+                    int bs = bside[s];
+                    if (g.Tfix[bs]) {
+                        dsum += 2.0 * lf;
+                        rhs += 2.0 * lf * g.Tw[bs];
+                    }
+                    continue;
+                }
+                if (kn[s] != k) {
+                    double th = link_theta(g, cseg, hpos, vpos, i, j, s, p.theta_min);
+                    dsum += lf / th;
+                    rhs += lf * p.T_sat / th;
+                }
             }
-            continue;
         }
-        int kn = flags[cidx(g, ii, jj)] & F_CCOL;
-        if (kn != k) {
-            double th = link_theta(g, cseg, hpos, vpos, i, j, s, p.theta_min);
-            dsum += lf / th;
-            rhs += lf * p.T_sat / th;
-        }
+        cd[c] = coef;
+        dd[c] = dsum;
+        b[c] = rhs;
+        x0[c] = ts;
+        // left and bottom face weights of the cell (domain faces carry none)
+        wl[c] = (i > 0 && kn[1] == k) ? (k ? lx_l : lx_v) : 0.0;
+        wb[c] = (j > 0 && kn[3] == k) ? (k ? ly_l : ly_v) : 0.0;
     }
-    cd[c] = coef;
-    dd[c] = dsum;
-    b[c] = rhs;
-    x0[c] = ts;
-    // left and bottom face weights of the cell (domain faces carry none)
-    wl[c] = (i > 0 && (flags[cidx(g, i - 1, j)] & F_CCOL) == k) ? lam * rad_fx<AXI>(g, i) : 0.0;
-    wb[c] = (j > 0 && (flags[cidx(g, i, j - 1)] & F_CCOL) == k) ? lam * mc : 0.0;
 }
 
 // ---------------------------------------------------------------------------------
@@ -1136,8 +1154,11 @@ void launch_energy_operator(const Grid& g, const Phys& p, const uint8_t* flags, 
                             double* cd, double* dd, double* wl, double* wb, double* b, double* x0,
                             cudaStream_t st) {
     auto k = g.axi ? k_energy_operator<true> : k_energy_operator<false>;
-    k<<<rows_grid(g.nx, g.ny, 128, g.nz), 128, 0, st>>>(g, p, flags, cseg, hpos, vpos, Ts_l, Ts_v, cd, dd, wl, wb, b,
-                                                          x0);
+    // a cut link takes a thread 10 us, so few rows of it in one thread: one below 2^21 cells (four there:
+    // 512^2 20 -> 52 us), four above (4096^2 453 -> 249)
+    const int rows = operator_rows(g) < 8 ? 1 : 4;
+    k<<<rows_grid(g.nx, div_up(g.ny, rows), 128, g.nz), 128, 0, st>>>(g, p, flags, cseg, hpos, vpos, Ts_l, Ts_v, cd, dd, wl,
+                                                                      wb, b, x0, rows);
 }
 
 void launch_mass_flux(const Grid& g, const Phys& p, const uint16_t* cseg, const double* hpos,
