@@ -1,6 +1,7 @@
 // C ABI of the EBIT phase-change step: context, memory, stage orchestration.
 // The time iteration follows Sec. 2.5 of arXiv 2402.13677 (see include/ebit.h).
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -69,6 +70,7 @@ struct Instance {
     unsigned solved = 0;                     // solve slots written since the last statistics read
     int batch = -1;                          // batch this instance belongs to (-1: stepped alone)
     int bz = 0;                              // its index inside the batch
+    int hix = 0;                             // its place in the context's host arrays
 };
 
 // Instances that share grid, boundary conditions and solver settings are stepped together when
@@ -489,22 +491,58 @@ static ebit_status run_stage(ebit_ctx* ctx, Instance& I, int stage) {
     return cuda_check(ctx, "run_stage");
 }
 
+// Read-back of the instances' status words and solver slots, queued on the context stream.  The
+// members of a batch lie `stride` bytes apart on the device and consecutively in the host arrays:
+// one strided copy of each array per batch instead of three copies per instance (2 us each: 8 % of
+// a step of 384 instances in 20 batches); the slots so only if every member has solved.
+static void queue_status(ebit_ctx* ctx) {
+    constexpr size_t SB = Solver::NSLOT * sizeof(SolveState);
+    for (auto& B : ctx->batches) {
+        const Instance& L = ctx->inst[B.members[0]];
+        bool all = true, all2 = true;
+        for (int m : B.members) {
+            all = all && ctx->inst[m].solved;
+            all2 = all2 && (ctx->inst[m].solved & (1u << SLOT_VISC_Y));
+        }
+        const size_t n = B.members.size();
+        auto rows = [&](void* dst, const void* src, size_t bytes) {
+            cudaMemcpy2DAsync(dst, bytes, src, B.stride, bytes, n, cudaMemcpyDeviceToHost, ctx->stream);
+        };
+        if (B.stride > (size_t)INT_MAX) {   // beyond a copy's pitch
+            for (int m : B.members)
+                cudaMemcpyAsync(ctx->host_status + ctx->inst[m].hix, ctx->inst[m].status, sizeof(int),
+                                cudaMemcpyDeviceToHost, ctx->stream);
+            all = all2 = false;
+        } else {
+            rows(ctx->host_status + L.hix, L.status, sizeof(int));
+            if (all) rows(L.solver.st_host, L.solver.st_base, SB);
+            if (all2) rows(L.solver2.st_host, L.solver2.st_base, SB);
+        }
+        for (int m : B.members) {
+            Instance& I = ctx->inst[m];
+            if (I.solved && !all) I.solver.fetch_states(ctx->stream);
+            if ((I.solved & (1u << SLOT_VISC_Y)) && !all2) I.solver2.fetch_states(ctx->stream);
+        }
+    }
+    for (auto& I : ctx->inst) {
+        if (I.batch >= 0) continue;
+        if (I.solved) I.solver.fetch_states(ctx->stream);
+        if (I.solved & (1u << SLOT_VISC_Y)) I.solver2.fetch_states(ctx->stream);
+        cudaMemcpyAsync(ctx->host_status + I.hix, I.status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+    }
+}
+
 // status and solver statistics of every instance: all read-backs are queued on the context
 // stream, then one synchronisation
 static ebit_status check_status(ebit_ctx* ctx, bool graph_step = false) {
-    for (size_t b = 0; b < ctx->inst.size(); ++b) {
-        Instance& I = ctx->inst[b];
-        if (I.solved) I.solver.fetch_states(ctx->stream);
-        if (I.solved & (1u << SLOT_VISC_Y)) I.solver2.fetch_states(ctx->stream);
-        cudaMemcpyAsync(ctx->host_status + b, I.status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
-    }
+    queue_status(ctx);
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return fail(ctx, EBIT_ECUDA, cudaGetErrorString(e));
     ebit_status worst = EBIT_OK;
     for (size_t b = 0; b < ctx->inst.size(); ++b) {
         Instance& I = ctx->inst[b];
         collect_stats(I, graph_step);
-        int s = ctx->host_status[b];
+        int s = ctx->host_status[I.hix];
         std::string where = ctx->inst.size() > 1 ? " (instance " + std::to_string(b) + ")" : "";
         if (s & 1) return fail(ctx, EBIT_ECFL, "a marker moved one cell or more in one sweep (reduce dt)" + where);
         if (s & 2) return fail(ctx, EBIT_ETOPO, "too many marker candidates on one edge" + where);
@@ -642,10 +680,15 @@ ebit_status ebit_init(const ebit_config* cfgs, int batch, void* stream, const eb
     for (int k = 0; k < 3; ++k) cudaStreamCreateWithFlags(&ctx->aux[k], cudaStreamNonBlocking);
     cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking);
     for (auto& e : ctx->ev) cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
+    int hix = 0;   // host arrays: the batches' members one after another, then the instances alone
+    for (auto& B : ctx->batches)
+        for (int m : B.members) ctx->inst[m].hix = hix++;
+    for (auto& I : ctx->inst)
+        if (I.batch < 0) I.hix = hix++;
     for (int b = 0; b < batch; ++b) {
         Instance& I = ctx->inst[b];
-        I.solver.st_host = ctx->host_states + b * Solver::NSLOT;
-        I.solver2.st_host = ctx->host_states + (batch + b) * Solver::NSLOT;
+        I.solver.st_host = ctx->host_states + I.hix * Solver::NSLOT;
+        I.solver2.st_host = ctx->host_states + (batch + I.hix) * Solver::NSLOT;
         for (int k = 0; k < 3; ++k) I.solver.aux[k] = I.solver2.aux[k] = ctx->aux[k];
         for (int k = 0; k < 2; ++k) I.solver.ev[k] = I.solver2.ev[k] = ctx->ev[k];
         I.side = ctx->side;
