@@ -495,7 +495,7 @@ struct Cells {
     T x[2][2][NR];
 };
 
-// n consecutive elements (8 or a multiple of 16 bytes, aligned to 8 or 16) from shared memory
+// n consecutive elements (4, 8 or a multiple of 16 bytes, so aligned)
 template <int N, typename T>
 __device__ inline void load_row(const T* s, T* o) {
     constexpr int W = N * sizeof(T) > 16 ? 16 / (int)sizeof(T) : N;
@@ -511,8 +511,9 @@ __device__ inline void load_row(const T* s, T* o) {
 // load the thread's cells (coefficients to registers, x to shared memory: for pre-smoothing
 // the result of the first colour-0 half-sweep from x = 0, for post-smoothing xin + the
 // prolongated coarse x); cells outside the domain get D = 1, zero weights, b = x = 0, so
-// sweeps leave them 0.  Staged: the two cells of a row are adjacent in the boxes, one 8 or 16 byte
-// load per operand
+// sweeps leave them 0.  The two cells of a row are adjacent, in the boxes and in the level's arrays:
+// one 8 or 16 byte load per operand (all tiled levels have even sides, their arrays and offsets are
+// aligned to a pair)
 template <typename T, int NR, int H, bool POST, bool STAGED, bool CHECK>
 __device__ inline void tile_load_cells(Region<T, NR, H>& R, Cells<T, NR>& C, int k, int ry0, const Lev<T>& L,
                                        const T* __restrict__ b, const T* __restrict__ xin, const T* __restrict__ xc,
@@ -551,49 +552,48 @@ __device__ inline void tile_load_cells(Region<T, NR, H>& R, Cells<T, NR>& C, int
                 for (int q = 0; q < 2 * NR; ++q) xp[r][q] += cv[q % NR];
         }
     }
+    // the block is in the grid or out of it as a whole (sides and tile origins are even)
+    const int gi0 = gx0 + 2 * k, gj0 = gy0 + ry0;
+    const bool in = !CHECK || (gj0 >= 0 && gj0 < L.ny && gi0 >= 0 && gi0 < L.nx);
+    if constexpr (!STAGED) {
+        // unconditional loads (clamped, then masked): all of them can be in flight at once
+        const int gic = CHECK ? min(max(gi0, 0), L.nx - 2) : gi0, gjc = CHECK ? min(max(gj0, 0), L.ny - 2) : gj0;
+        const bool rgt = !CHECK || gic + 2 < L.nx, up = !CHECK || gjc + 2 < L.ny;
+        const T* D = ID && POST ? L.id : L.diag;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int g = (gjc + r) * L.nx + gic;
+            load_row<2>(D + g, dp[r]);
+            if constexpr (Sg::ID_BOX) load_row<2>(L.id + g, idp[r]);
+            load_row<2>(L.wl + g, wlp[r]);
+            wlp[r][2] = L.wl[rgt ? g + 2 : g];
+            if (CHECK && !rgt) wlp[r][2] = T(0);
+            load_row<2>(L.wb + g, wbp[r]);
+            load_row<2 * NR>(b + (size_t)g * NR, bp[r]);
+            if constexpr (POST) load_row<2 * NR>(xin + (size_t)g * NR, xp[r]);
+        }
+        load_row<2>(L.wb + (up ? gjc + 2 : gjc) * L.nx + gic, wbp[2]);
+        if (CHECK && !up) wbp[2][0] = wbp[2][1] = T(0);
+        if constexpr (POST) {
+            T cv[NR];
+            load_row<NR>(xc + (size_t)((gjc >> 1) * cnx + (gic >> 1)) * NR, cv);
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int q = 0; q < 2 * NR; ++q) xp[r][q] += cv[q % NR];
+        }
+    }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        const int gj = gy0 + ry0 + r;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const int gi = gx0 + 2 * k + e;
-            bool in = !CHECK || (gj >= 0 && gj < L.ny && gi >= 0 && gi < L.nx);
             Vec<T, NR> bv, xv;
-            T dv, wlv, wbv, wrv, wtv, idv = T(1);   // FP64: idv loaded (and D only where a residual follows)
-            if constexpr (STAGED) {
-                dv = dp[r][e];
-                if (ID) idv = Sg::ID_BOX ? idp[r][e] : dv;
-                wlv = wlp[r][e];
-                wbv = wbp[r][e];
-                wrv = wlp[r][e + 1];
-                wtv = wbp[r + 1][e];
+            T dv = dp[r][e], wlv = wlp[r][e], wbv = wbp[r][e], wrv = wlp[r][e + 1], wtv = wbp[r + 1][e];
+            T idv = !ID ? T(1) : Sg::ID_BOX ? idp[r][e] : dv;   // FP64: loaded (and D only where a residual follows)
 #pragma unroll
-                for (int k2 = 0; k2 < NR; ++k2) {
-                    bv.v[k2] = bp[r][e * NR + k2];
-                    xv.v[k2] = POST ? xp[r][e * NR + k2] : T(0);
-                }
-            } else {
-                // unconditional loads (clamped, then masked): all of them can be in flight at once
-                int gic = CHECK ? min(max(gi, 0), L.nx - 1) : gi, gjc = CHECK ? min(max(gj, 0), L.ny - 1) : gj;
-                int g = gjc * L.nx + gic;
-                bv = reinterpret_cast<const Vec<T, NR>*>(b)[g];
-                if (!(ID && POST)) dv = L.diag[g];
-                if (ID) idv = L.id[g];
-                wlv = L.wl[g];
-                wbv = L.wb[g];
-                wrv = L.wl[!CHECK || gic + 1 < L.nx ? g + 1 : g];
-                wtv = L.wb[!CHECK || gjc + 1 < L.ny ? g + L.nx : g];
-                if (CHECK && gi + 1 >= L.nx) wrv = T(0);
-                if (CHECK && gj + 1 >= L.ny) wtv = T(0);
-                if (POST) {
-                    xv = reinterpret_cast<const Vec<T, NR>*>(xin)[g];
-                    Vec<T, NR> cv = reinterpret_cast<const Vec<T, NR>*>(xc)[(gjc >> 1) * cnx + (gic >> 1)];
-#pragma unroll
-                    for (int k2 = 0; k2 < NR; ++k2) xv.v[k2] += cv.v[k2];
-                } else {
-#pragma unroll
-                    for (int k2 = 0; k2 < NR; ++k2) xv.v[k2] = T(0);
-                }
+            for (int k2 = 0; k2 < NR; ++k2) {
+                bv.v[k2] = bp[r][e * NR + k2];
+                xv.v[k2] = POST ? xp[r][e * NR + k2] : T(0);
             }
             if (CHECK && !in) {
 #pragma unroll
