@@ -170,7 +170,7 @@ __device__ inline double tile_advect(const double (*v)[WSX], int rx, int ry, dou
 // along x at tile columns -1 .. WX (rows 0 .. WY-1) and along y at tile rows -1 .. WY (columns
 // 0 .. WX-1), formed once per cell and field.  In the upwind-ordered stencil the two second
 // differences are a1 = D_{i-1}, a2 = D_i for u >= 0 and a1 = D_{i+1}, a2 = D_i for u < 0, and
-// v2 + v3 = +-(T_{i+1} - T_{i-1}), so a stencil costs four FP64 operations instead of nine
+// v2 + v3 = +-(T_{i+1} - T_{i-1}), so a stencil costs three FP64 operations instead of eight
 // (the mathematical value is that of weno3_up; the rounding differs by a few ulps of T).
 constexpr int D2X_N = (WX + 2) * WY, D2Y_N = WX * (WY + 2);
 template <int NF>
