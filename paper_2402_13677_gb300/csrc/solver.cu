@@ -2362,8 +2362,8 @@ __global__ void __launch_bounds__(256) k_diag_inverse(SetupPlan P, const double*
 // sum (48-bit, FP32 instructions only), written to the FP64 total by flush().  An earlier form
 // summed FP32 chunks of eight cells into FP64 with a counter tested in the per-cell body, which
 // the compiler issued as a predicated FP64 add for every cell (the FP64 pipe 40-60 % busy in
-// these memory-bound kernels).  The loops of k_update and k_ir_residual walk their cells in
-// chunks of DOT_CHUNK (more loads in flight per thread).  The inner FP32 solves of the
+// these memory-bound kernels).  The loop of k_update walks its cells in chunks of DOT_CHUNK (more
+// loads in flight per thread).  The inner FP32 solves of the
 // refinement work on a residual scaled to values of order one (k_ir_residual), so FP32 products
 // neither underflow nor overflow there.
 constexpr int DOT_CHUNK = 8;
@@ -3543,9 +3543,9 @@ __global__ void __launch_bounds__(256) k_ir_init(int N, long long zs, const doub
 // difference of x across a face serves both its cells (the other one's is its exact negative), 8.6
 // FP64 instructions a cell where one cell at a time needs 10, and the vertical ones need no second
 // load of x.  W = 2: four cells a row save 0.4 more but leave 16 warps an SM, the pipe half idle
-// (1024x2048, two right-hand sides: 112 us); loading a row ahead likewise (110).  Measured on 4096^2
-// films, one -> two right-hand sides: 331 and 652 us before, a step 22.0 -> 21.0 ms; 512^2 16.7 and 25.6
-// -> 15.6 and 22.4 us.
+// (1024x2048, two right-hand sides: 112 us); loading a row ahead likewise (110).  Measured, one and two
+// right-hand sides: 512^2 16.7 and 25.6 -> 15.6 and 22.4 us; a step on 4096^2 (11 launches of 331 and
+// 652 us before) 21.6 -> 21.0 ms.
 // n consecutive values of a row (one, or an even number at a 16-byte boundary)
 template <int n>
 __device__ __forceinline__ void row_ld(const double* __restrict__ p, double* o) {
@@ -3591,8 +3591,8 @@ __global__ void __launch_bounds__(IR_THREADS) k_ir_residual(Lev<double> L, const
     // the inner FP32 system is solved for s r, s = 2^k a power of two that brings the residual's
     // cell values to order one, set from the previous residual norm (of b on the first pass) by
     // the launch that computed it: the same in every block.  The FP32 copy is rounded from
-    // r 2^k on the integer pipes and the norm is summed from that copy (FP32 chunks added in
-    // FP64; relative accuracy about 1e-7, ample for the convergence test), so the FP64 pipe
+    // r 2^k on the integer pipes and the norm is summed from that copy (a thread's FP32-pair sum,
+    // then FP64; relative accuracy about 1e-7, ample for the convergence test), so the FP64 pipe
     // carries the residual alone.
     int ksc[NR];
 #pragma unroll
