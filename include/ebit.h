@@ -230,8 +230,9 @@ uint64_t ebit_launch_count(const ebit_ctx* ctx);
  * launch records the span from its first block's start to its last block's end from the GPU
  * global timer.  kernel_class EBIT_KT_SMOOTH_L0: the finest-grid multigrid smoother kernels
  * (tiled red-black Gauss-Seidel "pre" and "post" kernels), the dominant kernels of the step.
- * ebit_timing_end synchronises and returns, for the launches since ebit_timing_begin (0 before the
- * first one: no launch is timed then), the summed kernel time, the number of timed
+ * ebit_timing_end synchronises, ends the timing and returns, for the launches from ebit_timing_begin
+ * to the first ebit_timing_end after it (0 before any; a further ebit_timing_end returns the same
+ * figures again), the summed kernel time, the number of timed
  * launches and the algorithmic bytes of an average launch (pre: b, diag, wl, wb read, x and a
  * quarter-size coarse b written; post: x, a quarter-size coarse x, b, diag, wl, wb read, x
  * written; one word per value, 4 bytes in the mixed mode, 8 in FP64, per right-hand side).  A

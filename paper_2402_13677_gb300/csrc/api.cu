@@ -1311,6 +1311,9 @@ ebit_status ebit_timing_end(ebit_ctx* ctx, double* total_ms, uint64_t* launches,
                         ctx->stream);
         cudaMemcpyAsync(&t[4 * b + 2], ctx->inst[b].solver2.timer, 2 * sizeof(KTimer), cudaMemcpyDeviceToHost,
                         ctx->stream);
+        // off again: later launches are neither timed nor slowed by the timer's atomics
+        for (Solver* sv : {&ctx->inst[b].solver, &ctx->inst[b].solver2})
+            cudaMemset2DAsync(&sv->timer[0].on, sizeof(KTimer), 0, sizeof(int), 2, ctx->stream);
     }
     cudaStreamSynchronize(ctx->stream);
     for (auto& k : t) {
