@@ -1273,12 +1273,14 @@ ebit_status ebit_get_diagnostics(ebit_ctx* ctx, int inst, double* dst, int n) {
 uint64_t ebit_launch_count(const ebit_ctx* ctx) { return ctx ? g_launches.load() - ctx->launch0 : 0; }
 
 // the timed kernels are launches of their own: while they are timed no solve runs as one launch
-// (same values), and captured graphs of the other form are dropped
+// (same values).  Step graphs that hold such solves (grids of at most 16384 cells) are dropped; the
+// others are the same either way and stay.
 static void select_whole_solves(ebit_ctx* ctx, int on) {
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     for (auto& I : ctx->inst) {
         if (I.solver.use_cgc == on) continue;
         I.solver.use_cgc = I.solver2.use_cgc = on;
+        if (!(I.graph[0] || I.graph[1]) || !I.solver.whole_solves(I.cfg.precision)) continue;
         for (auto& gx : I.graph)
             if (gx) { cudaGraphExecDestroy(gx); gx = nullptr; }
     }

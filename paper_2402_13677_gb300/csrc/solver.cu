@@ -4768,6 +4768,21 @@ int Solver::body_size(int precision, int nr, bool alone, bool* whole) {
     return nr == 1 ? loop_kernels<float, 1>(*this, alone, whole) : loop_kernels<float, 2>(*this, alone, whole);
 }
 
+template <typename T>
+static bool any_whole(Solver& s) {
+    CgPlan G;
+    int t = 0;
+    size_t m = 0;
+    return cg_plan<T, 1>(s, G, t, m) || cg_plan<T, 2>(s, G, t, m);
+}
+bool Solver::whole_solves(int precision) {
+    const int keep = use_cgc;
+    use_cgc = 1;
+    const bool w = precision == 0 ? any_whole<double>(*this) : any_whole<float>(*this);
+    use_cgc = keep;
+    return w;
+}
+
 bool Solver::supported(int nx, int ny) {
     Solver s;
     s.plan(nx, ny);

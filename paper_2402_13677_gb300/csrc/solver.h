@@ -127,6 +127,8 @@ struct Solver {
     // kernels of one CG iteration of an nr-right-hand-side solve (V-cycle + apply + update); alone: not
     // in a batch; *whole: the solve (FP64) or each inner solve (mixed) is one launch instead (then 0)
     int body_size(int precision, int nr, bool alone, bool* whole);
+    // whether an instance stepped alone runs some solve of a step as one launch where use_cgc allows it
+    bool whole_solves(int precision);
 };
 
 }  // namespace ebit

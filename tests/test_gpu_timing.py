@@ -1,4 +1,6 @@
 """Timing sessions (ebit_timing_begin .. ebit_timing_end) and what they leave behind."""
+import time
+
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -29,5 +31,35 @@ def test_launches_after_the_session_are_not_timed(dev, sides, graph):  # noqa: F
         assert first[0] > 0 and first[1] > 0
         E.ebit_timing_begin(ctx)
         assert E.ebit_timing_end(ctx)[:2] == (0.0, 0)
+    finally:
+        E.ebit_destroy(ctx)
+
+
+def test_a_session_keeps_the_step_graphs_it_can_use(dev):  # noqa: F811
+    """Above 16384 cells a timed step launches what an untimed one does: its graph is not captured
+    again.  The first step of a session is compared with a later one of it and with a step that does
+    capture (an option was set, which drops the graphs): it is the nearer to the former."""
+    ctx = make_ctx(dev, [bubble(160)], E.EBIT_MIXED)
+
+    def step():
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        E.ebit_step(ctx, 1)
+        return time.perf_counter() - t
+    try:
+        capture, first, later = [], [], []
+        for _ in range(9):
+            E.ebit_set_option(ctx, E.EBIT_OPT_TMA, 1)
+            step(), step()              # both sweep orders
+            E.ebit_timing_begin(ctx)
+            E.ebit_set_option(ctx, E.EBIT_OPT_TMA, 1)
+            capture.append(step())
+            step()
+            later.append(step())
+            E.ebit_timing_end(ctx)
+            E.ebit_timing_begin(ctx)
+            first.append(step())
+            E.ebit_timing_end(ctx)
+        assert 2 * min(first) < min(later) + min(capture), (min(first), min(later), min(capture))
     finally:
         E.ebit_destroy(ctx)
