@@ -895,6 +895,7 @@ static ebit_status capture_step(ebit_ctx* ctx, Instance& I, cudaStream_t st, cud
     cudaStream_t s = st;
     if (I.p.energy) {
         launch_advect_T(I.g, I.p, I.flags, I.T_l, I.T_v, I.u_l, I.u_v, I.Ts_l, I.Ts_v, s);
+        count(1);
         extend_T(I, I.Ts_l, I.Ts_v, s);
     }
     advance_interface(I, s);
