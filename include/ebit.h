@@ -313,8 +313,8 @@ ebit_status ebit_get_schedule(ebit_ctx* ctx, int inst, int* small_max, double* i
  *   except while smoothers are timed; 0 launches each level separately.  All
  *   give the same values.  2 (mixed precision) runs each whole inner FP32 solve of the refinement, every
  *   V-cycle and CG update until the inner tolerance, in one cooperative launch with bounded
- *   grid barriers between its phases (grids whose finest tiles fit the reduction slots; others
- *   fall back to 1); its dot products are grouped per block, so the iterates agree with the
+ *   grid barriers between its phases (grids whose finest tiles fit the reduction slots; others,
+ *   and FP64, run as with 1); its dot products are grouped per block, so the iterates agree with the
  *   other forms to rounding, not bit for bit (measured 10-30 % slower than 0 or 1 on 512^2 and
  *   1024x2048 grids, where its one block per SM and the spills of its 128 registers outweigh
  *   the saved launches).  Instances stepped in batches always launch each level separately.

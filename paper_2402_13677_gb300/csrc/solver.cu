@@ -4170,7 +4170,7 @@ static int cluster_small(const Solver& s, int nb) {
 template <typename T, int NR>
 static int cluster_plan(Solver& s, ClPlan& P, int& threads, size_t& smem) {
     const int nb = nbig_of<T>(s);
-    if (s.use_coop != 1 || s.barrier_spin > 0 || s.nz != 1 || nb < 2) return nb;
+    if (!s.use_coop || s.barrier_spin > 0 || s.nz != 1 || nb < 2) return nb;
     if (!cluster_usable((const void*)k_coarse_cluster<T, NR>, PT<T>::prec * 2 + NR - 1)) return nb;
     const int ls = cluster_small<T>(s, nb), half = CL_THREADS / 2, need_s = small_threads<T, NR>(s, ls);
     P.S = small_plan<T>(s, ls);
@@ -4207,11 +4207,11 @@ static int cluster_plan(Solver& s, ClPlan& P, int& threads, size_t& smem) {
 }
 
 // Plan of the whole-solve cluster kernel; false where the grid does not fit it (or the separate
-// launches are asked for: EBIT_OPT_COOP other than 1, a barrier bound, smoother timing, a batch)
+// launches are asked for: EBIT_OPT_COOP 0, a barrier bound, smoother timing, a batch)
 template <typename T, int NR>
 static bool cg_plan(Solver& s, CgPlan& G, int& threads, size_t& smem) {
     const int nb = nbig_of<T>(s);
-    if (s.use_coop != 1 || s.barrier_spin > 0 || s.nz != 1 || !s.use_cgc || nb < 1) return false;
+    if (!s.use_coop || s.barrier_spin > 0 || s.nz != 1 || !s.use_cgc || nb < 1) return false;
     const int nx = s.nx, ny = s.ny;
     // 16 blocks then have more work than launches cost: a 160x160 mixed step took 930 us separate, 940 whole
     if ((long long)nx * ny > 16384) return false;
@@ -4768,17 +4768,18 @@ int Solver::body_size(int precision, int nr, bool alone, bool* whole) {
     return nr == 1 ? loop_kernels<float, 1>(*this, alone, whole) : loop_kernels<float, 2>(*this, alone, whole);
 }
 
-template <typename T>
-static bool any_whole(Solver& s) {
+template <typename T, int NR>
+static bool whole_if_allowed(Solver& s) {
     CgPlan G;
     int t = 0;
     size_t m = 0;
-    return cg_plan<T, 1>(s, G, t, m) || cg_plan<T, 2>(s, G, t, m);
+    return cg_plan<T, NR>(s, G, t, m);
 }
 bool Solver::whole_solves(int precision) {
     const int keep = use_cgc;
     use_cgc = 1;
-    const bool w = precision == 0 ? any_whole<double>(*this) : any_whole<float>(*this);
+    const bool w = precision == 0 ? whole_if_allowed<double, 1>(*this) || whole_if_allowed<double, 2>(*this)
+                                  : whole_if_allowed<float, 1>(*this) || whole_if_allowed<float, 2>(*this);
     use_cgc = keep;
     return w;
 }
