@@ -4744,6 +4744,19 @@ bool Solver::set_schedule(int small_max, double inner) {
     return true;
 }
 
+// whether the inner solves of a mixed solve are cooperative launches (EBIT_OPT_COOP 2)
+template <typename T, int NR>
+static bool persistent(Solver& s) {
+    if constexpr (sizeof(T) == 4) {
+        CoarsePlan<float> C;
+        SmallPlan P;
+        int g = 0;
+        size_t m = 0;
+        return persist_plan<NR>(s, C, P, g, m);
+    }
+    return false;
+}
+
 template <typename T, int NR>
 static int loop_kernels(Solver& s, bool alone, bool* whole) {
     const int nb = nbig_of<T>(s);
@@ -4753,7 +4766,7 @@ static int loop_kernels(Solver& s, bool alone, bool* whole) {
         ClPlan P;
         int t = 0;
         size_t m = 0;
-        if (cg_plan<T, NR>(s, G, t, m)) {
+        if (persistent<T, NR>(s) || cg_plan<T, NR>(s, G, t, m)) {
             *whole = true;
             return 0;
         }
@@ -4773,7 +4786,7 @@ static bool whole_if_allowed(Solver& s) {
     CgPlan G;
     int t = 0;
     size_t m = 0;
-    return cg_plan<T, NR>(s, G, t, m);
+    return !persistent<T, NR>(s) && cg_plan<T, NR>(s, G, t, m);
 }
 bool Solver::whole_solves(int precision) {
     const int keep = use_cgc;

@@ -1,7 +1,7 @@
-"""EBIT_OPT_COOP 2 where it has no form of its own.
+"""EBIT_OPT_COOP 2 where it has no form of its own, and its launch counts.
 
 2 replaces the inner FP32 solves of the mixed mode; FP64 solves run as with 1: the same launches and
-the same values."""
+the same values.  A graph step counts the kernels that the same step launched from the host counts."""
 import numpy as np
 import pytest
 
@@ -32,3 +32,9 @@ def test_fp64_runs_as_with_one_launch_per_coarse_cycle(dev, n):  # noqa: F811
     assert n2 == n1 < n0
     for k in NAMES:
         assert np.array_equal(f1[k], f2[k], equal_nan=True) and np.array_equal(f0[k], f2[k], equal_nan=True), k
+
+
+@pytest.mark.parametrize("n", [64, 160, 256])
+@pytest.mark.parametrize("precision", [E.EBIT_FP64, E.EBIT_MIXED])
+def test_graph_step_counts_the_kernels_of_a_host_driven_one(dev, n, precision):  # noqa: F811
+    assert one_step(dev, n, precision, 2, 1)[0] == one_step(dev, n, precision, 2, 0)[0]
