@@ -53,7 +53,11 @@ constexpr int NRED = 608;        // blocks of grid-stride kernels (4 x 152 SMs)
 constexpr int SMALL_MAX_F = 1024; // default: levels with at most this many cells run inside k_small (FP32)
 constexpr int SMALL_MAX_F_LIMIT = 4096;   // the shared memory of k_small holds at most this level
 constexpr int SMALL_MAX_D = 1024; // (FP64: half the shared memory per value)
+// the most that the single-block levels of any grid hold: cells (64 x 64 and its levels, rounded up) and
+// entries of the bordered x arrays (2048 x 2 and 1024 x 1: their two border rows double them)
+constexpr int SMALL_CELLS = 5464, SMALL_XENTRIES = 12296;
 constexpr int SMALL_THREADS = 512;   // of the single-block levels (k_small, and block 0 of a cooperative launch)
+constexpr size_t SMEM_MAX = 216 * 1024;   // dynamic shared memory of the cluster kernels and the single-block levels, at most
 constexpr int SMALL_INV = 32 * 32;   // entries of the coarsest operator's dense inverse, at most
 constexpr int TX = 32, TY = 32;  // tile of the large-level kernels
 constexpr int NU = 2;            // smoothing sweeps (red-black pairs) before and after
@@ -3852,9 +3856,9 @@ cudaError_t Solver::bind(void* base, int nx_, int ny_, bool make_streams, cudaSt
     timer = (KTimer*)take(4 * sizeof(KTimer));
     if (make_streams)
         for (int k = 0; k < 3; ++k) cudaStreamCreateWithFlags(&aux[k], cudaStreamNonBlocking);
-    // shared-memory limits of the tile kernels
-    // shared-memory opt-in of the tile and small-level kernels (dynamic + static may pass 48 KB)
-    const int SM = 200 * 1024;
+    // shared-memory opt-in of the tile kernels, and of those that run the single-block levels (2048 x 2
+    // cells with two right-hand sides take 204864 bytes; dynamic + static may pass 48 KB)
+    const int SM = 200 * 1024, SML = (int)SMEM_MAX;
     cudaError_t err = cudaSuccess;
     allow_smem(k_pre<float, 1>, SM, &err);
     allow_smem(k_pre<float, 2>, SM, &err);
@@ -3868,20 +3872,20 @@ cudaError_t Solver::bind(void* base, int nx_, int ny_, bool make_streams, cudaSt
     allow_smem(k_post<double, 1, false>, SM, &err);
     allow_smem(k_post<double, 2, true>, SM, &err);
     allow_smem(k_post<double, 2, false>, SM, &err);
-    allow_smem(k_coarse_cycle<float, 1>, SM, &err);
-    allow_smem(k_coarse_cycle<float, 2>, SM, &err);
-    allow_smem(k_coarse_cycle<double, 1>, SM, &err);
-    allow_smem(k_coarse_cycle<double, 2>, SM, &err);
-    allow_smem(k_cg_persist<float, 1>, SM, &err);
-    allow_smem(k_cg_persist<float, 2>, SM, &err);
-    allow_smem(k_small<float, 1, true>, SM, &err);
-    allow_smem(k_small<float, 1, false>, SM, &err);
-    allow_smem(k_small<float, 2, true>, SM, &err);
-    allow_smem(k_small<float, 2, false>, SM, &err);
-    allow_smem(k_small<double, 1, true>, SM, &err);
-    allow_smem(k_small<double, 1, false>, SM, &err);
-    allow_smem(k_small<double, 2, true>, SM, &err);
-    allow_smem(k_small<double, 2, false>, SM, &err);
+    allow_smem(k_coarse_cycle<float, 1>, SML, &err);
+    allow_smem(k_coarse_cycle<float, 2>, SML, &err);
+    allow_smem(k_coarse_cycle<double, 1>, SML, &err);
+    allow_smem(k_coarse_cycle<double, 2>, SML, &err);
+    allow_smem(k_cg_persist<float, 1>, SML, &err);
+    allow_smem(k_cg_persist<float, 2>, SML, &err);
+    allow_smem(k_small<float, 1, true>, SML, &err);
+    allow_smem(k_small<float, 1, false>, SML, &err);
+    allow_smem(k_small<float, 2, true>, SML, &err);
+    allow_smem(k_small<float, 2, false>, SML, &err);
+    allow_smem(k_small<double, 1, true>, SML, &err);
+    allow_smem(k_small<double, 1, false>, SML, &err);
+    allow_smem(k_small<double, 2, true>, SML, &err);
+    allow_smem(k_small<double, 2, false>, SML, &err);
     // device state that must start at zero (tickets, solve states, timers; timer starts at ~0)
     cudaError_t e[4];
     e[0] = cudaMemsetAsync(timer, 0, 4 * sizeof(KTimer), init_stream);
@@ -4102,7 +4106,8 @@ static int coarse_start(Solver& s) {
         size_t smem = Region<T, NR, HPRE>::bytes() > Region<T, NR, HPOST>::bytes()
                           ? Region<T, NR, HPRE>::bytes()
                           : Region<T, NR, HPOST>::bytes();
-        smem = smem > SmallMem<T, NR>::bytes(5464, 2 * 3072) ? smem : SmallMem<T, NR>::bytes(5464, 2 * 3072);
+        smem = smem > SmallMem<T, NR>::bytes(SMALL_CELLS, SMALL_XENTRIES) ? smem
+                                                                          : SmallMem<T, NR>::bytes(SMALL_CELLS, SMALL_XENTRIES);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_coarse_cycle<T, NR>, CC_THREADS, smem);
         res = per * sms;
         cudaGetLastError();
@@ -4111,8 +4116,6 @@ static int coarse_start(Solver& s) {
         if ((long long)((s.lnx[l] + TX - 1) / TX) * ((s.lny[l] + TY - 1) / TY) <= res) return l;
     return nb;
 }
-
-constexpr size_t SMEM_MAX = 216 * 1024;   // dynamic shared memory of the cluster kernels, at most
 
 // whether the current device takes a cluster of CL_BLOCKS blocks of the kernel (asked once per
 // device and kernel slot)
