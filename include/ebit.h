@@ -235,7 +235,9 @@ uint64_t ebit_launch_count(const ebit_ctx* ctx);
  * figures again), the summed kernel time, the number of timed
  * launches and the algorithmic bytes of an average launch (pre: b, diag, wl, wb read, x and a
  * quarter-size coarse b written; post: x, a quarter-size coarse x, b, diag, wl, wb read, x
- * written; one word per value, 4 bytes in the mixed mode, 8 in FP64, per right-hand side).  A
+ * written; one word per value, 4 bytes in the mixed mode, 8 in FP64, per right-hand side).  That is
+ * what the method needs, not all that the FP64 kernels read: their reciprocal diagonals are stored,
+ * read besides diag by pre and instead of it by post.  A
  * batched launch counts once, with the bytes of all its instances that had not converged. */
 enum { EBIT_KT_SMOOTH_L0 = 1 };
 ebit_status ebit_timing_begin(ebit_ctx* ctx, int kernel_class);
@@ -286,8 +288,9 @@ ebit_status ebit_solve_system_noalloc(int nx, int ny, const double* D, const dou
  *   - the relative tolerance of the refinement's inner FP32 solves: 1e-4 or 1e-5 (mixed
  *     precision only);
  *   - TMA staging of the tile regions on or off (instances stepped alone);
- *   - the coarse tiled levels and the single-block levels in one cooperative launch (grid
- *     barriers between the phases) or one launch per level (instances stepped alone).
+ *   - the coarse tiled levels and the single-block levels in one launch (EBIT_OPT_COOP 1: a
+ *     thread-block cluster or a cooperative launch) or one launch per level (instances stepped
+ *     alone).
  * The state of every instance (fields, markers, time, step counter) is restored afterwards
  * from a device snapshot of the largest unit's arena, which is allocated with cudaMalloc for
  * the duration of the call.  Needs graph mode.  EBIT_ENOMEM when the snapshot does not fit. */
@@ -307,7 +310,8 @@ ebit_status ebit_get_schedule(ebit_ctx* ctx, int inst, int* small_max, double* i
  *   EBIT_OPT_COOP (default 1) runs the coarse tiled levels of each V-cycle and the single-block
  *   levels in one launch: a thread-block cluster that keeps them in its shared memory (levels up
  *   to about 256 x 256 cells in FP32, 128 x 128 in FP64), or, where the device takes no such
- *   cluster or a barrier bound is set, a cooperative launch with grid barriers between the phases
+ *   cluster, a barrier bound is set or the first single-block level has more than 2048 cells (the
+ *   autotuner's candidate of 4096), a cooperative launch with grid barriers between the phases
  *   (levels whose tiles fit one per co-resident block); on grids of at most 16384 cells that fit a
  *   cluster whole, a complete FP64 solve (mixed precision: each inner FP32 solve) is one launch,
  *   except while smoothers are timed; 0 launches each level separately.  All
@@ -324,8 +328,9 @@ ebit_status ebit_get_schedule(ebit_ctx* ctx, int inst, int* small_max, double* i
  *   a few polls makes the barriers give up before the other blocks arrive.  Changing it drops
  *   the captured step graphs.
  *   EBIT_OPT_EXT_BLOCK (default 1 on grids of at most 2^19 cells, 0 above) runs every Jacobi
- *   sweep of a narrow-band extension (extrapolation equation, Sec. 2.4) in one thread block per
- *   instance; 0 launches one kernel per sweep over the whole device.  Both give the same values.
+ *   sweep of a narrow-band extension (extrapolation equation, Sec. 2.4) in one launch: a
+ *   thread-block cluster for an instance stepped alone, one thread block per instance in a batch
+ *   or where the device takes no such cluster; 0 launches one kernel per sweep over the whole device.  Both give the same values.
  *   Changing it drops the captured step graphs.
  * A tile kernel that waits for its copies in vain, or a grid barrier that waits in vain, gives
  * up after a bounded wait and records a fault; ebit_step, ebit_solve_system and

@@ -268,7 +268,7 @@ static void reconstruct_full(Instance& I, cudaStream_t st) {
     count(3);   // + memset
 }
 
-// kernels of one narrow-band extension: one in a single block per instance, else one per sweep
+// kernels of one narrow-band extension: one where all sweeps share a launch, else one per sweep
 static int extend_launches(const Instance& I) { return I.g.ext_block ? 1 : I.p.extend_iters; }
 
 static void extend_T(Instance& I, double* Tl, double* Tv, cudaStream_t st) {
@@ -564,8 +564,10 @@ static ebit_status check_status(ebit_ctx* ctx, bool graph_step = false) {
     return worst;
 }
 
-// grids up to this many cells run each narrow-band extension in one CTA per instance (their
-// bands are a few thousand cells); larger ones launch one kernel per Jacobi sweep
+// grids up to this many cells run each narrow-band extension in one launch (their bands are a few
+// thousand cells); larger ones launch one kernel per Jacobi sweep.  The limit was measured for one
+// thread block per instance, which batches and devices without the cluster still run; an instance
+// alone runs k_extend_cluster, about three times as fast, for which it has not been measured.
 constexpr long long EXT_BLOCK_MAX_CELLS = 1LL << 19;
 
 // two configurations can share batched launches: the same grid, boundaries and solver settings

@@ -290,7 +290,8 @@ inline dim3 grid1(long long n, int bs, int nz) { return dim3(div_up(n, bs), 1, n
 inline dim3 rows_grid(int n, int rows, int bs, int nz) { return dim3(div_up(n, bs), rows, nz); }
 // rows of a column that a thread of the operator kernels takes: one on small grids (a short chain, and
 // a block for every SM), four from 2^17 cells on (512^2: viscous 12.4 -> 7.6 us, Poisson 15.2 -> 12.5),
-// eight from 2^21 on; one on axisymmetric grids, whose rows share no coefficient
+// eight from 2^21 on; one on axisymmetric grids, whose kernels do not look for equal rows (a column's
+// radii are the same in every row, so they could: not built, not measured)
 inline int operator_rows(const Grid& g) {
     const long long n = (long long)g.nx * g.ny * (g.nz > 0 ? g.nz : 1);
     return g.axi || n < (1 << 17) ? 1 : n < (1 << 21) ? 4 : 8;

@@ -1155,7 +1155,7 @@ void launch_energy_operator(const Grid& g, const Phys& p, const uint8_t* flags, 
                             cudaStream_t st) {
     auto k = g.axi ? k_energy_operator<true> : k_energy_operator<false>;
     // a cut link takes a thread 10 us, so few rows of it in one thread: one below 2^21 cells (four there:
-    // 512^2 20 -> 52 us), four above (4096^2 453 -> 249)
+    // 512^2 20 -> 52 us), four above (4096^2 453 -> 264)
     const int rows = operator_rows(g) < 8 ? 1 : 4;
     k<<<rows_grid(g.nx, div_up(g.ny, rows), 128, g.nz), 128, 0, st>>>(g, p, flags, cseg, hpos, vpos, Ts_l, Ts_v, cd, dd, wl,
                                                                       wb, b, x0, rows);

@@ -84,8 +84,7 @@ struct Lev {
     const T* id;    // FP64: reciprocal of the full diagonal (k_diag_inverse); null in FP32
 };
 
-// correctly rounded reciprocal (the same value as 1 / v)
-// reciprocal of a smoother's diagonal.  FP32 (the preconditioner of the inner solves): the
+// Reciprocal of a smoother's diagonal.  FP32 (the preconditioner of the inner solves): the
 // hardware approximation (one MUFU instruction, within about an ulp; the diagonals are normal
 // numbers), the same in every kernel, so that the tile, cooperative and single-block paths stay
 // identical; a preconditioner need only be fixed and symmetric, not correctly rounded.  FP64:
@@ -1808,8 +1807,8 @@ __global__ void __launch_bounds__(CC_THREADS) k_coarse_cycle(CoarsePlan<T> C, Sm
 // right-hand sides and corrections through distributed shared memory, and block 0 runs the
 // single-block levels.  The arithmetic of every cell is that of the tile kernels.
 // Measured per launch against the grid-barrier launch or the separate ones (one right-hand side):
-// FP32 on a 128^2 grid 17.6 -> 12.8 us, on 512^2 31.2 -> 29 (its 256^2 level costs what two separate
-// launches do); FP64 from the 128^2 level down 80 -> 47 us.  A 64^2 level of four rows per block
+// FP32 on a 128^2 grid 17.6 -> 12.8 us, on 512^2 31.2 -> 26 (28 with cold caches; its 256^2 level costs
+// what two separate launches do); FP64 from the 128^2 level down 80 -> 46 us.  A 64^2 level of four rows per block
 // spends about 1000 cycles a phase, 750 of them push and barrier.
 constexpr int CL_MAX = 6;            // levels kept by the cluster, at most
 constexpr int CL_BLOCKS = 16;        // blocks of the cluster (16 needs the non-portable attribute)
@@ -3548,8 +3547,9 @@ __global__ void __launch_bounds__(256) k_ir_init(int N, long long zs, const doub
 // FP64 instructions a cell where one cell at a time needs 10, and the vertical ones need no second
 // load of x.  W = 2: four cells a row save 0.4 more but leave 16 warps an SM, the pipe half idle
 // (1024x2048, two right-hand sides: 112 us); loading a row ahead likewise (110).  Measured, one and two
-// right-hand sides: 512^2 16.7 and 25.6 -> 15.6 and 22.4 us; a step on 4096^2 (11 launches of 331 and
-// 652 us before) 21.6 -> 21.0 ms.
+// right-hand sides: 512^2 16.7 and 25.6 -> 15.6 and 22.4 us; 4096^2 331 and 652 -> 302 and 566 (a step 21.6
+// -> 21.0 ms); 1024x2048 gains nothing with one right-hand side (54.1 -> 54.3 cold: fewer FP64
+// instructions, but 80 registers leave a third of the warps; the pipe is 52-70 % busy, 79 % with two).
 // n consecutive values of a row (one, or an even number at a 16-byte boundary)
 template <int n>
 __device__ __forceinline__ void row_ld(const double* __restrict__ p, double* o) {
@@ -4168,8 +4168,10 @@ static int cluster_small(const Solver& s, int nb) {
 // cluster's shared memory and threads (l0 = nb: none; the finest level stays separate, its
 // post-smoothing carries the r.z of CG).  In FP64, where a half-sweep of 32 x 32 cells takes one
 // SM 0.8 us of FP64 issue against 0.45 us over the cluster, the levels above 256 cells stay in the
-// cluster; in FP32 those above the single-block size.  Single instances; a bound set for the grid
-// barriers (EBIT_OPT_BARRIER_SPIN) asks for the grid-barrier launch.
+// cluster; in FP32 those above the single-block size (block 0 has a thread for each block of that
+// level's cells or there is no plan: with a single-block size of 4096 cells a first level of more than
+// 2048 takes the grid-barrier launch).  Single instances; a bound set for the grid barriers
+// (EBIT_OPT_BARRIER_SPIN) asks for the grid-barrier launch.
 template <typename T, int NR>
 static int cluster_plan(Solver& s, ClPlan& P, int& threads, size_t& smem) {
     const int nb = nbig_of<T>(s);
